@@ -871,8 +871,9 @@ ib_status engine_build(Engine& E) {
 
   // ---- reductions, solver state, streams
   const int64_t maxblk = std::max<int64_t>(E.nbricks, Mt / 8 + 1);
-  TRY(dalloc(E, &E.rb.partials, maxblk * 16 + int64_t(n) * 16 + 64, true));
-  TRY(dalloc(E, &E.rb.counter, 1, true));
+  // CTA partials, instance totals, group sums; one arrival word per CTA and one more
+  TRY(dalloc(E, &E.rb.partials, 2 * maxblk * 16 + int64_t(n) * 16 + 64, true));
+  TRY(dalloc(E, &E.rb.counter, 1 + maxblk, true));
   TRY(dalloc(E, &E.ks, 3 * n, true));
   TRY(dalloc(E, &E.os, n, true));
   TRY(dalloc(E, &E.recs, 4 * n, true));

@@ -252,41 +252,116 @@ __device__ __forceinline__ const T* stencil_factors(const DevGrid& g, int b) {
   else return reinterpret_cast<const T*>(g.sf64) + idx;
 }
 
-// Block-wide sum of NV values of type T (blockDim.x a multiple of 32, <= 1024);
-// the total is valid in thread 0.
+// Sums of NV values (NV <= 16) over the lanes of a warp, all values in one butterfly:
+// every step halves the values a lane still carries (it keeps one half and
+// hands the other to its partner), so NV = 6 costs 9 additions a lane instead
+// of the 30 of one tree per value.  On FP64, where an SM issues two lanes a clock,
+// that is the reduction's cost.  Each value's additions pair the lanes as a
+// shuffle-down tree does, so the sums have the same bits.  Value k ends in
+// sh[32 k + w], w the warp.
 template <typename T, int NV>
-__device__ __forceinline__ void block_sum(T (&v)[NV], T* sh /* [32*NV] */) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+__device__ __forceinline__ void warp_sums(const T (&v)[NV], T* sh, int w) {
+  static_assert(NV <= 16, "one value per pair of lanes at most");
+  constexpr int P = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : NV <= 8 ? 8 : 16;
+  constexpr int PB = P == 1 ? 0 : P == 2 ? 1 : P == 4 ? 2 : P == 8 ? 3 : 4;
+  const int lane = threadIdx.x & 31;
+  T a[P];
 #pragma unroll
-  for (int k = 0; k < NV; ++k)
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  __syncthreads();
-  if (lane == 0)
-    for (int k = 0; k < NV; ++k) sh[k * 32 + w] = v[k];
-  __syncthreads();
-  if (w == 0) {
+  for (int k = 0; k < P; ++k) a[k] = k < NV ? v[k < NV ? k : 0] : T(0);
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      v[k] = lane < nw ? sh[k * 32 + lane] : T(0);
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  for (int q = 0; q < PB; ++q) {
+    const int off = 16 >> q, h = P >> (q + 1);
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const T send = up ? a[j] : a[j + h], keep = up ? a[j + h] : a[j];
+      a[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
     }
   }
+#pragma unroll
+  for (int off = 16 >> PB; off > 0; off >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+  const int k = lane >> (5 - PB);
+  if ((lane & ((32 >> PB) - 1)) == 0 && k < NV) sh[k * 32 + w] = a[0];
 }
 
-// The second half of grid_sum_last, for kernels that write their partials
-// themselves (partials[NV * p + k] for p over the instances' partial ranges
-// seg[i] .. seg[i+1]): every CTA arrives once; the last one sums, for every
-// instance, its partials in FP64 with all its threads (thread t takes the
-// relative partials t, t + blockDim, ...; then a fixed tree) into
-// out[i * NV + k], and returns true after a __syncthreads that makes out
-// visible to all its threads.  The counter is reset.  The caller's partial
-// writes must come from thread 0.
+// Sum of one value over the lanes of a warp, valid in lane 0.
+template <typename T>
+__device__ __forceinline__ T lane_sum(T x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Block-wide sum of NV values of type T (blockDim.x a multiple of 32, <= 1024),
+// value k handed to put(k, total) by lane 0 of one warp; ends with a CTA barrier.
+template <typename T, int NV, typename Put>
+__device__ __forceinline__ void block_sum(const T (&v)[NV], T* sh /* [32*NV] */, Put&& put) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  __syncthreads();
+  warp_sums<T, NV>(v, sh, w);
+  __syncthreads();
+  for (int k = w; k < NV; k += nw) {
+    const T x = lane_sum(lane < nw ? sh[k * 32 + lane] : T(0));
+    if (lane == 0) put(k, x);
+  }
+  __syncthreads();
+}
+
+// Deterministic segmented grid reduction, in three stages: every CTA's total
+// (in the kernel's precision T), the FP64 sum of each group of up to
+// RED_GROUP consecutive CTAs of one instance, and the FP64 sum of an
+// instance's groups.  Groups are counted from the instance's first CTA, so an
+// instance's totals depend only on its own CTAs and their order and are
+// bitwise the same alone and next to other instances.
+//
+// Bound: latency, and in the last stage the FP64 rate (two lanes a clock and
+// SM).  One CTA summing every partial of every instance with block-wide FP64
+// trees took 8-10 us of a 14 us k_bcgv_dot on 140k nodes and most of its 68 us
+// on a batch of eight; with groups each stage is one load and one warp tree
+// a value, spread over the SMs.  A step, before and after: batch of eight
+// requests 37.7 -> 25.6 ms, 16x16x64 tube in FP64 30.4 -> 22.6 ms, refined
+// 64x64x256 tube 32.0 -> 30.5 ms, two-level 16 M-node sac 136.5 -> 133.0 ms.
+constexpr int RED_GROUP = 32;   // one lane per CTA of a group
+
+// the FP64 sum of one group's value k (a warp), written to gpart by lane 0
+template <int NV>
+__device__ __forceinline__ void group_total(const double* __restrict__ partials, double* __restrict__ gpart,
+                                            int first, int gn, int k) {
+  const int lane = threadIdx.x & 31;
+  const double x = lane_sum(lane < gn ? __ldcg(partials + (int64_t)(first + lane) * NV + k) : 0.0);
+  if (lane == 0) gpart[(int64_t)first * NV + k] = x;
+}
+
+// out[i * NV + k] for every instance from the group sums (one warp per value),
+// visible to the whole CTA on return
+template <int NV>
+__device__ __forceinline__ void instance_totals(const double* __restrict__ gpart, const int32_t* __restrict__ seg,
+                                                int nseg, double* __restrict__ out) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  for (int q = w; q < nseg * NV; q += nw) {
+    const int i = q / NV, k = q - NV * i;
+    const int s1 = seg[i + 1];
+    double x = 0.0;
+#pragma unroll 4
+    for (int64_t f = seg[i] + RED_GROUP * lane; f < s1; f += RED_GROUP * 32) x += __ldcg(gpart + f * NV + k);
+    x = lane_sum(x);
+    if (lane == 0) out[(int64_t)i * NV + k] = x;
+  }
+  __threadfence_block();
+  __syncthreads();
+}
+
+// For kernels that write their partials themselves (partials[NV * p + k] for p
+// over the instances' partial ranges seg[i] .. seg[i+1]): every CTA arrives
+// once; the last one forms the group sums and the totals, the same bits as
+// grid_sum_last.  The caller's partial writes must come from thread 0.
+// gpart: as many doubles as partials.
 template <int NV>
 __device__ __forceinline__ bool segment_sums_last(const double* __restrict__ partials, unsigned* __restrict__ counter,
                                                   const int32_t* __restrict__ seg, int nseg,
                                                   double* __restrict__ out) {
-  __shared__ double shd[32 * NV];
   __shared__ bool last;
+  double* gpart = out + (int64_t)nseg * NV;
   if (threadIdx.x == 0) {
     __threadfence();
     unsigned prev = atomicAdd(counter, 1u);
@@ -295,39 +370,58 @@ __device__ __forceinline__ bool segment_sums_last(const double* __restrict__ par
   __syncthreads();
   if (!last) return false;
   __threadfence();
+  const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   for (int i = 0; i < nseg; ++i) {
-    double acc[NV];
-    for (int k = 0; k < NV; ++k) acc[k] = 0.0;
-    for (int64_t b = seg[i] + threadIdx.x; b < seg[i + 1]; b += blockDim.x)
-      for (int k = 0; k < NV; ++k) acc[k] += __ldcg(partials + b * NV + k);
-    block_sum<double, NV>(acc, shd);
-    if (threadIdx.x == 0)
-      for (int k = 0; k < NV; ++k) out[(int64_t)i * NV + k] = acc[k];
+    const int s0 = seg[i], s1 = seg[i + 1], ng = (s1 - s0 + RED_GROUP - 1) / RED_GROUP;
+    for (int q = w; q < ng * NV; q += nw) {
+      const int first = s0 + RED_GROUP * (q / NV);
+      group_total<NV>(partials, gpart, first, min(RED_GROUP, s1 - first), q % NV);
+    }
   }
-  __threadfence_block();
+  __threadfence();
   __syncthreads();
+  instance_totals<NV>(gpart, seg, nseg, out);
   if (threadIdx.x == 0) *counter = 0u;
   return true;
 }
 
-// Deterministic segmented grid reduction.  Every block sums its threads' NV
-// contributions in the kernel's precision T (FP32 kernels: FP32 within the
-// block; the GB300 FP64 rate would otherwise dominate) and writes the block
-// totals in FP64; the last block to arrive sums, for every instance i, the
-// partials of blocks [seg[i], seg[i+1]) in FP64 (segment_sums_last) and
-// stores the totals in out[i * NV + k].  Returns true in that block only,
-// after a __syncthreads that makes out visible to all its threads.  The
-// counter is reset.  An instance's totals depend only on its own blocks and
-// their order, so they are bitwise the same alone and next to other instances.
+// The grid reduction: every thread's NV contributions are summed per instance
+// into out[i * NV + k] (out follows the gridDim.x * NV partials; the group
+// sums follow out).  inst: the instance of this CTA, whose CTAs are
+// seg[inst] .. seg[inst + 1].  counter: 1 + gridDim.x words, zero before
+// and after.  Returns true in the last CTA only, after a barrier that makes
+// out visible to all its threads.
 template <typename T, int NV>
 __device__ __forceinline__ bool grid_sum_last(T (&v)[NV], double* __restrict__ partials,
                                               unsigned* __restrict__ counter, const int32_t* __restrict__ seg,
-                                              int nseg, double* __restrict__ out) {
+                                              int nseg, int inst, double* __restrict__ out) {
   __shared__ T sht[32 * NV];
-  block_sum<T, NV>(v, sht);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < NV; ++k) partials[(int64_t)blockIdx.x * NV + k] = double(v[k]);
-  return segment_sums_last<NV>(partials, counter, seg, nseg, out);
+  __shared__ bool last;
+  double* gpart = out + (int64_t)nseg * NV;
+  block_sum<T, NV>(v, sht, [&](int k, T x) { partials[(int64_t)blockIdx.x * NV + k] = double(x); });
+  const int s0 = seg[inst], s1 = seg[inst + 1];
+  const int first = s0 + (int(blockIdx.x) - s0) / RED_GROUP * RED_GROUP, gn = min(RED_GROUP, s1 - first);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(counter + 1 + first, 1u) == unsigned(gn - 1);
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  for (int k = w; k < NV; k += nw) group_total<NV>(partials, gpart, first, gn, k);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    counter[1 + first] = 0u;
+    __threadfence();
+    last = atomicAdd(counter, unsigned(gn)) + unsigned(gn) == gridDim.x;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  instance_totals<NV>(gpart, seg, nseg, out);
+  if (threadIdx.x == 0) *counter = 0u;
+  return true;
 }
 
 }  // namespace ibg

@@ -927,7 +927,7 @@ __global__ void __launch_bounds__(512) k_poisson_cg(DevGrid g, const T* __restri
   if (!CG) return;
   T v[1] = {acc};
   double* out = partials + (int64_t)gridDim.x;
-  if (!grid_sum_last<T, 1>(v, partials, counter, g.cseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 1>(v, partials, counter, g.cseg, g.ninst, inst, out)) return;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     KState& kk = ks[i];
     if (kk.done) continue;
@@ -1179,7 +1179,7 @@ __global__ void __launch_bounds__(P7_THREADS, 8)
   if (!CG) return;
   float v[1] = {acc};
   double* out = partials + (int64_t)gridDim.x;
-  if (!grid_sum_last<float, 1>(v, partials, counter, g.cseg, g.ninst, out)) return;
+  if (!grid_sum_last<float, 1>(v, partials, counter, g.cseg, g.ninst, inst, out)) return;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     KState& kk = ks[i];
     if (kk.done) continue;
@@ -1388,8 +1388,7 @@ __global__ void __launch_bounds__(P7_THREADS, 6)
     if constexpr (CG) {
       if (h.last) {   // the chunk's p.q partial (zero for an idle instance)
         float v[1] = {acc};
-        block_sum<float, 1>(v, sred);
-        if (t == 0) partials[h.chunk] = double(v[0]);
+        block_sum<float, 1>(v, sred, [&](int, float x) { partials[h.chunk] = double(x); });
         acc = 0.f;
       }
     }
@@ -1636,17 +1635,16 @@ __global__ void __launch_bounds__(512, (sizeof(T) == 4 && OP == OP_MASS && !PB) 
   }
   if (post != POST_CG_ALPHA) return;
   double* out = partials + (int64_t)gridDim.x * NC;
-  if (!grid_sum_last<T, NC>(acc, partials, counter, PB ? g.bseg : g.cseg, g.ninst, out)) return;
-  for (int i = threadIdx.x; i < g.ninst; i += blockDim.x)
-    for (int c = 0; c < NC; ++c) {
-      KState& k = ks[i * NC + c];
-      if (k.done) continue;
-      const double pq = out[i * NC + c];
-      k.pq = pq;
-      if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; k.af = 0.f; continue; }
-      k.alpha = k.rz / pq;
-      k.af = float(k.alpha);
-    }
+  if (!grid_sum_last<T, NC>(acc, partials, counter, PB ? g.bseg : g.cseg, g.ninst, inst, out)) return;
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
+    KState& k = ks[e];
+    if (k.done) continue;
+    const double pq = out[e];
+    k.pq = pq;
+    if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; k.af = 0.f; continue; }
+    k.alpha = k.rz / pq;
+    k.af = float(k.alpha);
+  }
 }
 
 // FP32 momentum operator, 3 components (the inner BiCGStab of the mixed path),

@@ -14,8 +14,8 @@ enum Op : int { OP_POISSON = 0, OP_MASS = 1, OP_COEF = 2 };
 
 // Scratch for deterministic grid reductions.
 struct RedBuf {
-  double* partials = nullptr;   // >= nblocks * 16 + ninst * 16 doubles
-  unsigned* counter = nullptr;  // one zero-initialised word
+  double* partials = nullptr;   // >= 2 * nblocks * 16 + ninst * 16 doubles
+  unsigned* counter = nullptr;  // 1 + nblocks zero-initialised words
 };
 
 // Optional CUDA-event timing of solver kernel launches, by class:

@@ -129,16 +129,15 @@ __global__ void __launch_bounds__(IBB) k_af_apply(IBDev ib, const double* __rest
     }
   if (mode == 0) return;
   double* out = partials + (int64_t)gridDim.x * 3;
-  if (!grid_sum_last<double, 3>(v, partials, counter, ib.seg_w, ib.ninst, out)) return;
-  for (int n = threadIdx.x; n < ib.ninst; n += blockDim.x)
-    for (int c = 0; c < 3; ++c) {
-      KState& k = ks[n * 3 + c];
-      if (k.done) continue;
-      const double pq = out[n * 3 + c];
-      k.pq = pq;
-      if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; continue; }
-      k.alpha = k.rz / pq;
-    }
+  if (!grid_sum_last<double, 3>(v, partials, counter, ib.seg_w, ib.ninst, ib.pinst[(int64_t)blockIdx.x * (IBB / 32)], out)) return;
+  for (int e = threadIdx.x; e < ib.ninst * 3; e += blockDim.x) {
+    KState& k = ks[e];
+    if (k.done) continue;
+    const double pq = out[e];
+    k.pq = pq;
+    if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; continue; }
+    k.alpha = k.rz / pq;
+  }
 }
 
 // CG iteration form of the SpMV: p_new = z + beta p_old (read on the fly for
@@ -180,17 +179,16 @@ __global__ void __launch_bounds__(IBB) k_af_apply_p(IBDev ib, const T* __restric
     }
   }
   double* out = partials + (int64_t)gridDim.x * 3;
-  if (!grid_sum_last<T, 3>(v, partials, counter, ib.seg_g, ib.ninst, out)) return;
-  for (int n = threadIdx.x; n < ib.ninst; n += blockDim.x)
-    for (int c = 0; c < 3; ++c) {
-      KState& k = ks[n * 3 + c];
-      if (k.done) continue;
-      const double pq = out[n * 3 + c];
-      k.pq = pq;
-      if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; k.af = 0.f; continue; }
-      k.alpha = k.rz / pq;
-      k.af = float(k.alpha);
-    }
+  if (!grid_sum_last<T, 3>(v, partials, counter, ib.seg_g, ib.ninst, ib.pinst[(int64_t)blockIdx.x * (IBB / AFL)], out)) return;
+  for (int e = threadIdx.x; e < ib.ninst * 3; e += blockDim.x) {
+    KState& k = ks[e];
+    if (k.done) continue;
+    const double pq = out[e];
+    k.pq = pq;
+    if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; k.af = 0.f; continue; }
+    k.alpha = k.rz / pq;
+    k.af = float(k.alpha);
+  }
 }
 
 // r = b - y (y may be null: zero initial guess), z = D^-1 r, p = 0; skip_os:
@@ -215,24 +213,23 @@ __global__ void __launch_bounds__(IBB) k_af_start(IBDev ib, const T* __restrict_
       v[3 * c + 2] = b[3 * i + c] * b[3 * i + c];
     }
   double* out = partials + (int64_t)gridDim.x * 9;
-  if (!grid_sum_last<T, 9>(v, partials, counter, ib.seg_t, ib.ninst, out)) return;
+  if (!grid_sum_last<T, 9>(v, partials, counter, ib.seg_t, ib.ninst, ib.pinst[(int64_t)blockIdx.x * IBB], out)) return;
   bool any = false;
-  for (int n = threadIdx.x; n < ib.ninst; n += blockDim.x)
-    for (int c = 0; c < 3; ++c) {
-      KState& k = ks[n * 3 + c];
-      const double* t = out + n * 9 + 3 * c;
-      const bool skip = skip_os && skip_os[n].done;
-      k.rz = t[0];
-      k.rr = t[1];
-      k.bb = fmax(t[2], k.rr);
-      k.beta = 0.0;
-      k.bf = 0.f;
-      k.iter = 0;
-      k.status = 0;
-      k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
-      if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
-      any = any || !k.done;
-    }
+  for (int e = threadIdx.x; e < ib.ninst * 3; e += blockDim.x) {
+    KState& k = ks[e];
+    const double* t = out + 3 * e;
+    const bool skip = skip_os && skip_os[e / 3].done;
+    k.rz = t[0];
+    k.rr = t[1];
+    k.bb = fmax(t[2], k.rr);
+    k.beta = 0.0;
+    k.bf = 0.f;
+    k.iter = 0;
+    k.status = 0;
+    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
+    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    any = any || !k.done;
+  }
   any = __syncthreads_or(any ? 1 : 0) != 0;
   if (threadIdx.x == 0) set_cond(cond, any);
 }
@@ -260,23 +257,22 @@ __global__ void __launch_bounds__(IBB) k_af_update(IBDev ib, const T* __restrict
     }
   }
   double* out = partials + (int64_t)gridDim.x * 6;
-  if (!grid_sum_last<T, 6>(v, partials, counter, ib.seg_t, ib.ninst, out)) return;
+  if (!grid_sum_last<T, 6>(v, partials, counter, ib.seg_t, ib.ninst, ib.pinst[(int64_t)blockIdx.x * IBB], out)) return;
   bool any = false;
-  for (int n = threadIdx.x; n < ib.ninst; n += blockDim.x)
-    for (int c = 0; c < 3; ++c) {
-      KState& k = ks[n * 3 + c];
-      if (k.done) continue;
-      k.iter++;
-      k.rr = out[n * 6 + 2 * c + 1];
-      const double rzn = out[n * 6 + 2 * c];
-      if (!isfinite(k.rr)) { k.done = 1; k.status = 5; continue; }
-      if (k.rr <= k.tol2 * k.bb) { k.done = 1; continue; }
-      if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; continue; }
-      k.beta = rzn / k.rz;
-      k.bf = float(k.beta);
-      k.rz = rzn;
-      any = true;
-    }
+  for (int e = threadIdx.x; e < ib.ninst * 3; e += blockDim.x) {
+    KState& k = ks[e];
+    if (k.done) continue;
+    k.iter++;
+    k.rr = out[2 * e + 1];
+    const double rzn = out[2 * e];
+    if (!isfinite(k.rr)) { k.done = 1; k.status = 5; continue; }
+    if (k.rr <= k.tol2 * k.bb) { k.done = 1; continue; }
+    if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; continue; }
+    k.beta = rzn / k.rz;
+    k.bf = float(k.beta);
+    k.rz = rzn;
+    any = true;
+  }
   any = __syncthreads_or(any ? 1 : 0) != 0;
   if (threadIdx.x == 0) set_cond(cond, any);
 }
@@ -382,7 +378,7 @@ __global__ void __launch_bounds__(IBB) k_af_resid_outer(IBDev ib, const double* 
     }
   }
   double* out = partials + (int64_t)gridDim.x * 6;
-  if (!grid_sum_last<double, 6>(w, partials, counter, ib.seg_t, ib.ninst, out)) return;
+  if (!grid_sum_last<double, 6>(w, partials, counter, ib.seg_t, ib.ninst, ib.pinst[(int64_t)blockIdx.x * IBB], out)) return;
   bool any = false;
   for (int n = threadIdx.x; n < ib.ninst; n += blockDim.x) {
     OState& o = os[n];

@@ -106,20 +106,19 @@ __global__ void k_collect_outer(const OState* os, int ninst, SolveRec* rec) {
   R.status = max(R.status, os[i].status);
 }
 
+// Value q (of NQ) of component c of instance i from a grid reduction's totals.
 // Coupled components (one system in NC unknowns per node, the momentum
-// operator of the symmetric viscous form): each component's partial sums
-// become the sums over the components, so the NC states take the same
-// scalars and converge together, which is BiCGStab on the whole vector.
+// operator of the symmetric viscous form) take the sum over the components,
+// so the NC states take the same scalars and converge together, which is
+// BiCGStab on the whole vector.
 template <int NC, int NQ>
-__device__ __forceinline__ void couple_sums(double* o) {
+__device__ __forceinline__ double total_of(const double* out, int i, int c, int q, int coupled) {
+  const double* o = out + (int64_t)i * NC * NQ;
+  if (!coupled) return o[NQ * c + q];
+  double t = 0.0;
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    double t = 0.0;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) t += o[NQ * c + q];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) o[NQ * c + q] = t;
-  }
+  for (int d = 0; d < NC; ++d) t += o[NQ * d + q];
+  return t;
 }
 
 // ---------------------------------------------------------------- CG
@@ -146,27 +145,25 @@ __global__ void __launch_bounds__(512) k_cg_start(DevGrid g, const T* __restrict
     tv[3 * c + 2] = dof ? b[i] * b[i] : T(0);
   }
   double* out = partials + (int64_t)gridDim.x * 3 * NC;
-  if (!grid_sum_last<T, 3 * NC>(tv, partials, counter, g.bseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 3 * NC>(tv, partials, counter, g.bseg, g.ninst, g.binst[blockIdx.x], out)) return;
   bool any = false;
-  for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
-    const bool skip = skip_os && skip_os[i].done;
-    for (int c = 0; c < NC; ++c) {
-      KState& k = ks[i * NC + c];
-      const double* t = out + (int64_t)i * 3 * NC + 3 * c;
-      k.rz = t[0];
-      k.rr = t[1];
-      // reference norm max(||b||, ||r0||): covers a zero right-hand side with a
-      // nonzero Dirichlet lifting as well as warm starts
-      k.bb = fmax(t[2], k.rr);
-      k.iter = 0;
-      k.status = 0;
-      k.alpha = 0.0;
-      k.beta = 0.0;
-      k.af = k.bf = 0.f;
-      k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
-      if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
-      any = any || !k.done;
-    }
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {   // one thread per system: the divisions overlap
+    const bool skip = skip_os && skip_os[e / NC].done;
+    KState& k = ks[e];
+    const double* t = out + (int64_t)3 * e;
+    k.rz = t[0];
+    k.rr = t[1];
+    // reference norm max(||b||, ||r0||): covers a zero right-hand side with a
+    // nonzero Dirichlet lifting as well as warm starts
+    k.bb = fmax(t[2], k.rr);
+    k.iter = 0;
+    k.status = 0;
+    k.alpha = 0.0;
+    k.beta = 0.0;
+    k.af = k.bf = 0.f;
+    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
+    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    any = any || !k.done;
   }
   any = block_any(any);
   if (threadIdx.x == 0) set_cond(cond, any);
@@ -251,23 +248,22 @@ __global__ void __launch_bounds__(512) k_cg_update_vec(DevGrid g, T* __restrict_
     }
   }
   double* out = partials + (int64_t)gridDim.x * 2 * NC;
-  if (!grid_sum_last<T, 2 * NC>(tv, partials, counter, g.scseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 2 * NC>(tv, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
   bool any = false;
-  for (int i = threadIdx.x; i < g.ninst; i += blockDim.x)
-    for (int c = 0; c < NC; ++c) {
-      KState& kk = ks[i * NC + c];
-      if (kk.done) continue;
-      kk.iter++;
-      kk.rr = out[(int64_t)i * 2 * NC + 2 * c + 1];
-      const double rzn = out[(int64_t)i * 2 * NC + 2 * c];
-      if (!isfinite(kk.rr) || !isfinite(rzn)) { kk.done = 1; kk.status = 5; continue; }
-      if (kk.rr <= kk.tol2 * kk.bb) { kk.done = 1; continue; }
-      if (kk.iter >= kk.max_iter) { kk.done = 1; kk.status = 4; continue; }
-      kk.beta = rzn / kk.rz;
-      kk.bf = float(kk.beta);
-      kk.rz = rzn;
-      any = true;
-    }
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
+    KState& kk = ks[e];
+    if (kk.done) continue;
+    kk.iter++;
+    kk.rr = out[2 * (int64_t)e + 1];
+    const double rzn = out[2 * (int64_t)e];
+    if (!isfinite(kk.rr) || !isfinite(rzn)) { kk.done = 1; kk.status = 5; continue; }
+    if (kk.rr <= kk.tol2 * kk.bb) { kk.done = 1; continue; }
+    if (kk.iter >= kk.max_iter) { kk.done = 1; kk.status = 4; continue; }
+    kk.beta = rzn / kk.rz;
+    kk.bf = float(kk.beta);
+    kk.rz = rzn;
+    any = true;
+  }
   any = block_any(any);
   if (threadIdx.x == 0) set_cond(cond, any);
 }
@@ -289,7 +285,7 @@ __global__ void __launch_bounds__(512) k_cg_start_r(DevGrid g, const T* __restri
   r[s] = rv;
   T tv[2] = {dof ? rv * rv : T(0), dof ? b[s] * b[s] : T(0)};
   double* out = partials + (int64_t)gridDim.x * 2;
-  if (!grid_sum_last<T, 2>(tv, partials, counter, g.bseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 2>(tv, partials, counter, g.bseg, g.ninst, g.binst[blockIdx.x], out)) return;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     const bool skip = skip_os && skip_os[i].done;
     KState& k = ks[i];
@@ -350,7 +346,7 @@ __global__ void __launch_bounds__(512) k_cg_update_r(DevGrid g, T* __restrict__ 
     }
   }
   double* out = partials + (int64_t)gridDim.x;
-  if (!grid_sum_last<T, 1>(tv, partials, counter, g.scseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 1>(tv, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     KState& kk = ks[i];
     if (kk.done) continue;
@@ -375,7 +371,7 @@ __global__ void __launch_bounds__(512) k_cg_rz(DevGrid g, const T* __restrict__ 
     for (int64_t s = (int64_t)b0 * DBV + threadIdx.x; s < (int64_t)b1 * DBV; s += blockDim.x)
       if (kdof(g.meta[s], dmask)) tv[0] += r[s] * z[s];
   double* out = partials + (int64_t)gridDim.x;
-  if (!grid_sum_last<T, 1>(tv, partials, counter, g.scseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 1>(tv, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
   bool any = false;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     KState& kk = ks[i];
@@ -414,28 +410,26 @@ __global__ void __launch_bounds__(512) k_bcg_start(DevGrid g, const T* __restric
     tw[2 * c + 1] = dof ? b[i] * b[i] : T(0);
   }
   double* out = partials + (int64_t)gridDim.x * 2 * NC;
-  if (!grid_sum_last<T, 2 * NC>(tw, partials, counter, g.bseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 2 * NC>(tw, partials, counter, g.bseg, g.ninst, g.binst[blockIdx.x], out)) return;
   bool any = false;
-  for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
+    const int i = e / NC, c = e - NC * i;
     const bool skip = skip_os && skip_os[i].done;
-    if (coupled) couple_sums<NC, 2>(out + (int64_t)i * 2 * NC);
-    for (int c = 0; c < NC; ++c) {
-      KState& k = ks[i * NC + c];
-      k.rr = out[(int64_t)i * 2 * NC + 2 * c];
-      k.bb = fmax(out[(int64_t)i * 2 * NC + 2 * c + 1], k.rr);
-      k.rho = k.rr;
-      k.alpha = 1.0;
-      k.omega = 1.0;
-      k.beta = 0.0;
-      k.af = 1.f;
-      k.of = 1.f;
-      k.bf = 0.f;
-      k.iter = 0;
-      k.status = 0;
-      k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
-      if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
-      any = any || !k.done;
-    }
+    KState& k = ks[e];
+    k.rr = total_of<NC, 2>(out, i, c, 0, coupled);
+    k.bb = fmax(total_of<NC, 2>(out, i, c, 1, coupled), k.rr);
+    k.rho = k.rr;
+    k.alpha = 1.0;
+    k.omega = 1.0;
+    k.beta = 0.0;
+    k.af = 1.f;
+    k.of = 1.f;
+    k.bf = 0.f;
+    k.iter = 0;
+    k.status = 0;
+    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
+    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    any = any || !k.done;
   }
   any = block_any(any);
   if (threadIdx.x == 0) set_cond(cond, any);
@@ -541,24 +535,22 @@ __global__ void __launch_bounds__(512) k_bcgv_dot(DevGrid g, const T* __restrict
     }
   }
   double* out = partials + (int64_t)gridDim.x * 2 * NC;
-  if (!grid_sum_last<T, 2 * NC>(tw, partials, counter, g.scseg, g.ninst, out)) return;
-  for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
-    if (coupled) couple_sums<NC, 2>(out + (int64_t)i * 2 * NC);
-    for (int c = 0; c < NC; ++c) {
-      KState& k = ks[i * NC + c];
-      if (k.done) continue;
-      const double t0 = out[(int64_t)i * 2 * NC + 2 * c], t1 = out[(int64_t)i * 2 * NC + 2 * c + 1];
-      if (mode == 0) {
-        k.rv = t0;
-        if (k.rv == 0.0 || !isfinite(k.rv)) { k.done = 1; k.status = 5; k.alpha = 0.0; k.af = 0.f; continue; }
-        k.alpha = k.rho / k.rv;
-        k.af = float(k.alpha);
-      } else {
-        k.ts = t0;
-        k.tt = t1;
-        k.omega = (k.tt > 0.0) ? k.ts / k.tt : 0.0;
-        k.of = float(k.omega);
-      }
+  if (!grid_sum_last<T, 2 * NC>(tw, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
+    const int i = e / NC, c = e - NC * i;
+    KState& k = ks[e];
+    if (k.done) continue;
+    const double t0 = total_of<NC, 2>(out, i, c, 0, coupled), t1 = total_of<NC, 2>(out, i, c, 1, coupled);
+    if (mode == 0) {
+      k.rv = t0;
+      if (k.rv == 0.0 || !isfinite(k.rv)) { k.done = 1; k.status = 5; k.alpha = 0.0; k.af = 0.f; continue; }
+      k.alpha = k.rho / k.rv;
+      k.af = float(k.alpha);
+    } else {
+      k.ts = t0;
+      k.tt = t1;
+      k.omega = (k.tt > 0.0) ? k.ts / k.tt : 0.0;
+      k.of = float(k.omega);
     }
   }
 }
@@ -680,25 +672,23 @@ __global__ void __launch_bounds__(512) k_bcgv_xr(DevGrid g, T* __restrict__ x, T
     }
   }
   double* out = partials + (int64_t)gridDim.x * 2 * NC;
-  if (!grid_sum_last<T, 2 * NC>(tw, partials, counter, g.scseg, g.ninst, out)) return;
+  if (!grid_sum_last<T, 2 * NC>(tw, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
   bool any = false;
-  for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
-    if (coupled) couple_sums<NC, 2>(out + (int64_t)i * 2 * NC);
-    for (int c = 0; c < NC; ++c) {
-      KState& k = ks[i * NC + c];
-      if (k.done) continue;
-      k.iter++;
-      k.rr = out[(int64_t)i * 2 * NC + 2 * c];
-      const double rhon = out[(int64_t)i * 2 * NC + 2 * c + 1];
-      if (!isfinite(k.rr)) { k.done = 1; k.status = 5; continue; }
-      if (k.rr <= k.tol2 * k.bb) { k.done = 1; continue; }
-      if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; continue; }
-      if (k.omega == 0.0 || rhon == 0.0 || !isfinite(rhon)) { k.done = 1; k.status = 5; continue; }
-      k.beta = (rhon / k.rho) * (k.alpha / k.omega);
-      k.bf = float(k.beta);
-      k.rho = rhon;
-      any = true;
-    }
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
+    const int i = e / NC, c = e - NC * i;
+    KState& k = ks[e];
+    if (k.done) continue;
+    k.iter++;
+    k.rr = total_of<NC, 2>(out, i, c, 0, coupled);
+    const double rhon = total_of<NC, 2>(out, i, c, 1, coupled);
+    if (!isfinite(k.rr)) { k.done = 1; k.status = 5; continue; }
+    if (k.rr <= k.tol2 * k.bb) { k.done = 1; continue; }
+    if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; continue; }
+    if (k.omega == 0.0 || rhon == 0.0 || !isfinite(rhon)) { k.done = 1; k.status = 5; continue; }
+    k.beta = (rhon / k.rho) * (k.alpha / k.omega);
+    k.bf = float(k.beta);
+    k.rho = rhon;
+    any = true;
   }
   any = block_any(any);
   if (threadIdx.x == 0) set_cond(cond, any);
@@ -783,7 +773,7 @@ __global__ void __launch_bounds__(512) k_residual_outer(DevGrid g, const double*
     w[2 * c + 1] = sumsq_value(bs[c], bq[c]);
   }
   double* out = partials + (int64_t)gridDim.x * 2 * NC;
-  if (!grid_sum_last<double, 2 * NC>(w, partials, counter, g.scseg, g.ninst, out)) return;
+  if (!grid_sum_last<double, 2 * NC>(w, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
   bool any = false;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     OState& o = os[i];
