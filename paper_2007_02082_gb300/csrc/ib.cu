@@ -6,7 +6,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
+#include "async.cuh"
 #include "ib.hpp"
 #include "krylov.hpp"
 
@@ -277,6 +279,12 @@ __global__ void __launch_bounds__(IBB) k_af_update(IBDev ib, const T* __restrict
   if (threadIdx.x == 0) set_cond(cond, any);
 }
 
+}  // namespace ibg
+
+#include "af_cluster.cuh"
+
+namespace ibg {
+
 // one thread per free support node: u += coef * sum_e W[ent] G[point(ent)]
 __global__ void k_ib_spread(int64_t n, const int32_t* __restrict__ n_dev, const int32_t* __restrict__ sp_slot,
                             const int32_t* __restrict__ sp_off, const int32_t* __restrict__ sp_ent,
@@ -306,6 +314,61 @@ void ib_weights(const IBDev& ib, cudaStream_t st) {
              ib.ihf, ib.W);
 }
 
+template <typename T>
+static cudaLaunchConfig_t afc_config(int ninst, int cl, cudaLaunchAttribute* attr, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(ninst * cl));
+  cfg.blockDim = dim3(AFC_THREADS);
+  cfg.dynamicSmemBytes = AFC_SMEM;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = unsigned(cl);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// The largest cluster of 16 or 8 CTAs this device can hold (a constant of the
+// device, so that results do not depend on what else runs), 0 if none.
+template <typename T>
+static int afc_cluster_size() {
+  if (cudaFuncSetAttribute(k_af_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(k_af_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, AFC_SMEM) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  for (int cl : {AFC_MAX, 8}) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = afc_config<T>(1, cl, attr, nullptr);
+    int nc = 0;
+    if (cudaOccupancyMaxActiveClusters(&nc, k_af_cluster<T>, &cfg) == cudaSuccess && nc > 0) return cl;
+    cudaGetLastError();
+  }
+  return 0;
+}
+
+void ib_choose_solver(IBDev& ib, const int32_t* seg_t) {
+  ib.af_cl32 = afc_cluster_size<float>();
+  ib.af_cl64 = afc_cluster_size<double>();
+  ib.af_big32 = ib.af_big64 = false;
+  for (int n = 0; n < ib.ninst; ++n) {
+    const int64_t rows = int64_t(seg_t[n + 1] - seg_t[n]) * 256;
+    if (!afc_fits<float>(rows, ib.af_cl32)) ib.af_big32 = true;
+    if (!afc_fits<double>(rows, ib.af_cl64)) ib.af_big64 = true;
+  }
+}
+
+// the cluster solve of every problem that fits; x: the iterate (updated), r: its residual
+template <typename T>
+static void af_cluster_solve(const IBDev& ib, int cl, const T* val, const T* dinv, T* x, const T* r, KState* ks,
+                             cudaStream_t st) {
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = afc_config<T>(ib.ninst, cl, attr, st);
+  cudaLaunchKernelEx(&cfg, k_af_cluster<T>, ib, val, dinv, x, r, ks);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+}
+
 void ib_assemble(const IBDev& ib, cudaStream_t st) {
   if (ib.M == 0) return;
   const int64_t th = ib.M * 32;
@@ -326,7 +389,8 @@ cudaError_t ib_solve(const IBDev& ib, const double* BF, double* G, double* work,
   double *r = work, *z = work + L, *p = work + 2 * L, *q = work + 3 * L;
   IBG_LAUNCH(k_init_states, (ib.ninst * 3 + 127) / 128, 128, 0, st, ks, ib.ninst * 3, rtol * rtol, max_iter);
   Cond cond;
-  if (cc && cc->capturing) {
+  const bool cluster = ib.af_cl64 > 0, loop = ib.af_big64;
+  if (loop && cc && cc->capturing) {
     cudaError_t e = cond_handle(st, 0, &cond);
     if (e != cudaSuccess) return e;
   }
@@ -335,6 +399,8 @@ cudaError_t ib_solve(const IBDev& ib, const double* BF, double* G, double* work,
   IBG_LAUNCH(k_af_apply, gw, IBB, 0, st, ib, G, q, 0, ks, rb.partials, rb.counter);
   IBG_LAUNCH((k_af_start<double>), gt, IBB, 0, st, ib, ib.dinv, BF, (const double*)q, r, z, p, ks, rb.partials,
              rb.counter, cond, (const OState*)nullptr);
+  if (cluster) af_cluster_solve<double>(ib, ib.af_cl64, ib.val, ib.dinv, G, r, ks, st);
+  // the problems too large for a cluster (the others are done by now):
   // k_af_start left p = z and beta = 0; the direction ping-pongs between p and
   // p2, two iterations per loop body
   double* p2 = work + 4 * L;
@@ -345,12 +411,14 @@ cudaError_t ib_solve(const IBDev& ib, const double* BF, double* G, double* work,
     IBG_LAUNCH((k_af_update<double>), gt, IBB, 0, s, ib, ib.dinv, G, r, z, (const double*)pnew, (const double*)q,
                ks, rb.partials, rb.counter, c);
   };
-  cudaError_t e = run_loop(cc, st, cond, ks, ks_host, ib.ninst * 3, max_iter, 4, 32,
-                           [&](cudaStream_t s, const Cond& c) {
-    iter(s, c, p, p2);
-    iter(s, c, p2, p);
-  });
-  if (e != cudaSuccess) return e;
+  if (loop) {
+    cudaError_t e = run_loop(cc, st, cond, ks, ks_host, ib.ninst * 3, max_iter, 4, 32,
+                             [&](cudaStream_t s, const Cond& c) {
+      iter(s, c, p, p2);
+      iter(s, c, p2, p);
+    });
+    if (e != cudaSuccess) return e;
+  }
   IBG_LAUNCH(k_collect, (ib.ninst + 127) / 128, 128, 0, st, ks, 3, ib.ninst, rec, (OState*)nullptr);
   return cudaSuccess;
 }
@@ -442,23 +510,27 @@ cudaError_t ib_solve_mixed(const IBDev& ib, const double* BF, double* G, double*
     IBG_LAUNCH(k_init_states, (ib.ninst * 3 + 127) / 128, 128, 0, s, ks, ib.ninst * 3, rtol_inner * rtol_inner,
                max_iter);
     Cond ci;
-    if (cc && cc->capturing) {
+    if (ib.af_big32 && cc && cc->capturing) {
       cudaError_t e = cond_handle(s, 0, &ci);
       if (e != cudaSuccess) return e;
     }
     IBG_LAUNCH((k_af_start<float>), gt, IBB, 0, s, ib, (const float*)ib.dinv32, (const float*)r32,
                (const float*)nullptr, r, z, pa, ks, rb.partials, rb.counter, ci, (const OState*)os);
+    if (ib.af_cl32 > 0) af_cluster_solve<float>(ib, ib.af_cl32, ib.val32, ib.dinv32, e32, r, ks, s);
     auto iter = [&](cudaStream_t s2, const Cond& c2, const float* pold, float* pnew) {
       IBG_LAUNCH((k_af_apply_p<float>), g8, IBB, 0, s2, ib, (const float*)ib.val32, (const float*)z, pold, pnew, q,
                  ks, rb.partials, rb.counter);
       IBG_LAUNCH((k_af_update<float>), gt, IBB, 0, s2, ib, (const float*)ib.dinv32, e32, r, z, (const float*)pnew,
                  (const float*)q, ks, rb.partials, rb.counter, c2);
     };
-    cudaError_t e = run_loop(cc, s, ci, ks, ks_host, ib.ninst * 3, max_iter, 4, 32, [&](cudaStream_t s2, const Cond& c2) {
-      iter(s2, c2, pa, pb);
-      iter(s2, c2, pb, pa);
-    });
-    if (e != cudaSuccess) return e;
+    if (ib.af_big32) {   // the problems too large for a cluster
+      cudaError_t e = run_loop(cc, s, ci, ks, ks_host, ib.ninst * 3, max_iter, 4, 32,
+                               [&](cudaStream_t s2, const Cond& c2) {
+        iter(s2, c2, pa, pb);
+        iter(s2, c2, pb, pa);
+      });
+      if (e != cudaSuccess) return e;
+    }
     IBG_LAUNCH(k_collect, gi, 128, 0, s, (const KState*)ks, 3, ib.ninst, rec, os);
     IBG_LAUNCH(k_af_add, gt, IBB, 0, s, ib, (const float*)e32, G, (const OState*)os);
     return cudaSuccess;

@@ -45,7 +45,15 @@ struct IBDev {
   // device and launches cover sp_cap entries, so a captured step stays valid
   const int32_t* n_sp_dev = nullptr;
   int64_t sp_cap = 0;
+  // force solve (ib_choose_solver): CTAs of the cluster that solves a problem
+  // in one launch (0: no clusters) and whether some problem is too large for one
+  // and takes the launch-per-pass loop, in FP32 and FP64
+  int32_t af_cl32 = 0, af_cl64 = 0;
+  bool af_big32 = true, af_big64 = true;
 };
+
+// Choose each problem's force solver by its padded row count (seg_t, host copy).
+void ib_choose_solver(IBDev& ib, const int32_t* seg_t);
 
 // Eq. 17-18: W[i][a] = phi((x_a - X_i)/hx) phi((y_a - Y_i)/hy) phi((z_a - Z_i)/hz).
 void ib_weights(const IBDev& ib, cudaStream_t st);
