@@ -14,7 +14,7 @@
 // alone and in any batch; problems of a batch run side by side.
 // Bound: latency of the barriers and FP64 scalars at a few hundred rows (5 us an
 // iteration), shared-memory wavefronts of the product at some thousand dense rows
-// (8160 rows of 41 entries: 11 us), in FP64 the FP64 rate of 16 SMs (2000 rows: 13 us).
+// (8160 rows of 41 entries: 12 us), in FP64 the FP64 rate of 16 SMs (2000 rows: 14 us).
 // A step: 8x8x16 tube 22.0 -> 6.5 ms, 16x16x64 tube in FP64 22.6 -> 15.3 ms, dense
 // 32x32x128 tube 22.8 -> 12.0 ms (of which the reductions alone gave a third).
 #pragma once
@@ -22,8 +22,10 @@
 namespace ibg {
 
 constexpr int AFC_THREADS = 1024;
+constexpr int AFC_RPT = 2;                  // rows per thread at most (x stays in registers)
+constexpr int AFC_UNITS = 128;              // 32-row units of a problem that exchanges their sums
 constexpr int AFC_MAX = 16;                 // CTAs per cluster at most
-constexpr int AFC_SMEM = 222 * 1024;        // dynamic shared memory asked for (with the static part below 227 KB)
+constexpr int AFC_SMEM = 218 * 1024;        // dynamic shared memory asked for (with the static part below 227 KB)
 
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t smem, uint32_t rank) {
   uint32_t a;
@@ -34,8 +36,9 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_load3(uint32_t a, float (&v)[3]) {
-  float pad;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(pad) : "r"(a));
+  asm volatile("{\n\t.reg .f32 pad;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, pad}, [%3];\n\t}"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2])
+               : "r"(a));
 }
 __device__ __forceinline__ void cluster_load3(uint32_t a, double (&v)[3]) {
   asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a));
@@ -52,22 +55,33 @@ __device__ __forceinline__ void window_load3(const double* a, double (&v)[3]) {
 __device__ __forceinline__ void cluster_store(uint32_t a, int v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
+__device__ __forceinline__ void cluster_store(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
 __device__ __forceinline__ void cluster_store(uint32_t a, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
+// products that round on their own
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // bytes of shared memory per row: p with 1/diag (four values), q, r and the row's first entry
 template <typename T>
 __host__ __device__ constexpr int afc_row_bytes() { return 10 * int(sizeof(T)) + 4; }
-// Padded rows of a problem that runs in clusters of cl CTAs.  FP32: while its
-// rows take half of the shared memory (at 32,000 rows of 10 entries 14 us an
-// iteration, as the loop; the rest of the range still saves the launches).
+// Padded rows of a problem that runs in clusters of cl CTAs.  FP32: up to where
+// the loop's launches cost the same (32,000 rows of 10 entries: 15.7 us an
+// iteration here, about 16 in the loop; 8160 rows of 41: 11.8 against 22).
 // FP64: while the FP64 rate of 16 SMs costs less than the loop's launches
-// (2000 rows of 40 entries 13 us against 25; 32,000 rows of 10 measured 80 against 50).
+// (2000 rows of 40 entries 14 us against 25; 32,000 rows of 10 measured 80 against 50).
 template <typename T>
-__host__ __device__ constexpr int64_t afc_max_rows(int cl) { return int64_t(cl) * (sizeof(T) == 4 ? 2560 : 384); }
+__host__ __device__ constexpr int64_t afc_max_rows(int cl) { return int64_t(cl) * (sizeof(T) == 4 ? 2048 : 384); }
+static_assert(2048 <= AFC_THREADS * AFC_RPT, "x of a CTA's rows is kept in registers");
 template <typename T>
 __host__ __device__ constexpr bool afc_fits(int64_t n, int cl) { return cl > 0 && n <= afc_max_rows<T>(cl); }
+
+using three = std::integral_constant<int, 3>;
+using six = std::integral_constant<int, 6>;
 
 template <typename T>
 __global__ void __launch_bounds__(AFC_THREADS, 1)
@@ -75,8 +89,8 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
                  const T* __restrict__ r0, KState* __restrict__ ks) {
   KCOUNT();
   extern __shared__ __align__(16) unsigned char afc_sm[];
-  __shared__ double part[2][AFC_MAX][6];   // partial sums of every CTA: p.q, then r.z and r.r
-  __shared__ T red[32 * 6];
+  __shared__ double part[2][AFC_MAX][6];   // sums of every CTA: p.q, then r.z and r.r
+  __shared__ T red[6][AFC_THREADS / 32 * AFC_RPT];
   __shared__ T sal[3], sbe[3];
   __shared__ KState sk[3];
   __shared__ int win, goff[AFC_MAX];
@@ -89,15 +103,19 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   // uniform over the cluster: nothing to do, or too large for a cluster
   if (n == 0 || !afc_fits<T>(n, cl) || (ks[3 * inst].done && ks[3 * inst + 1].done && ks[3 * inst + 2].done)) return;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int rpc = n / int(cl);             // rows of this CTA
-  const int64_t row0 = R0 + int64_t(rank) * rpc;
-  const int e0 = ib.rowptr[row0], ne = ib.rowptr[row0 + rpc] - e0;
-  // lanes per row of the product: four where rows are short (all of the
-  // problem decides, so that its CTAs agree), eight otherwise
-  const int lpr = ib.rowptr[R0 + n] - ib.rowptr[R0] < 20 * n || sizeof(T) == 8 ? 4 : 8;
+  // rows per CTA: FP32 whole units of 32 rows where the problem's units fit the
+  // exchange, else whole blocks of 256 (so that a CTA holds whole blocks
+  // of the sums); FP64 units of 32
+  const bool units = sizeof(T) == 4 && n <= 32 * AFC_UNITS;
+  const int gran = sizeof(T) == 8 || units ? 32 : 256;
+  const int rper = (n / gran + int(cl) - 1) / int(cl) * gran;
+  const int rpc = max(0, min(n - int(rank) * rper, rper));   // rows of this CTA
+  const int64_t row0 = R0 + int64_t(rank) * rper;
+  const int e0 = rpc ? ib.rowptr[row0] : 0, ne = rpc ? ib.rowptr[row0 + rpc] - e0 : 0;
+  constexpr int lpr = AFL / 2;             // threads per row of the product
   // no more warps than the rows need: the others leave (the barriers count
   // the threads that are left)
-  const int nt = min(AFC_THREADS, max(256, lpr * rpc));
+  const int nt = min(AFC_THREADS, max(256, AFL * rper));
   if (t >= nt) return;
   // The rows whose p the CTA's columns need from the others: points listed along
   // the wall need a short run before and after its own.  That window of p
@@ -114,12 +132,15 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     if (need > 0) atomicMax(&win, need);
   }
   __syncthreads();
-  const int own0 = int(rank) * rpc;        // the problem's row of the CTA's first one
-  const int room = AFC_SMEM - 64 - rpc * afc_row_bytes<T>();
+  const int own0 = min(int(rank) * rper, n);   // the problem's row of the CTA's first one
+  const int ubytes = units ? 12 * (n / 32) * int(sizeof(T)) : 0;
+  const int room = AFC_SMEM - 64 - ubytes - rpc * afc_row_bytes<T>();
   const bool fast = win <= room / int(16 * sizeof(T));   // the window takes half the room at most
   const int G = fast ? win : 0;
   const int w0 = max(0, own0 - G), wn = min(n, own0 + rpc + G) - w0;   // window: rows [w0, w0 + wn) of the problem
-  T* pw = reinterpret_cast<T*>(afc_sm);    // [wn][4]: p; the own rows' fourth value is 1/diag
+  // in place of part: the sums of every 32 rows of the problem, [2][6][n / 32]
+  T* unit = reinterpret_cast<T*>(afc_sm);
+  T* pw = reinterpret_cast<T*>(afc_sm + ubytes);   // [wn][4]: p; the own rows' fourth value is 1/diag
   T* p = pw + 4 * (own0 - w0);
   T* q = pw + 4 * wn;                      // [rpc][3]
   T* r = q + 3 * rpc;                      // [rpc][3]
@@ -132,14 +153,15 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   if (t < int(cl)) cluster_store(cluster_addr(smem_u32(&goff[rank]), uint32_t(t)), own0 - w0);
   const uint32_t pbase = smem_u32(pw);
   auto owner = [&](int k) -> uint32_t {    // cluster address of p at row k of the problem
-    const int o = k / rpc;
-    return cluster_addr(pbase + uint32_t(goff[o] + k - o * rpc) * uint32_t(4 * sizeof(T)), uint32_t(o));
+    const int o = k / rper;
+    return cluster_addr(pbase + uint32_t(goff[o] + k - o * rper) * uint32_t(4 * sizeof(T)), uint32_t(o));
   };
   for (int e = t; e < cap; e += nt) {
     cv[e] = val[e0 + e];
     cc[e] = uint16_t(ib.col[e0 + e] - R0 - w0);
   }
-  for (int i = t; i <= rpc; i += nt) rp[i] = ib.rowptr[row0 + i] - e0;
+  if (rpc)
+    for (int i = t; i <= rpc; i += nt) rp[i] = ib.rowptr[row0 + i] - e0;
   for (int i = t; i < rpc; i += nt) {
     p[4 * i + 3] = dinv[row0 + i];
 #pragma unroll
@@ -154,21 +176,85 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   }
   __syncwarp();
   cluster_barrier();
-  const int nact = min(nt / 32, (rpc + 31) / 32);   // warps that hold rows in the row-per-thread passes
   auto wrow = [&](int i) { return i < own0 - w0 ? i : i + rpc; };   // window row of the i-th row of others
   const uint32_t ghost0 = t < wn - rpc ? owner(w0 + wrow(t)) : 0u;
-  // CTA totals of NV values (each thread's v) to every CTA of the cluster
-  auto exchange = [&](auto& v, auto nv, int buf) {
-    constexpr int NV = decltype(nv)::value;
-    if (w < nact) warp_sums<T, NV>(v, red, w);
-    __syncthreads();
-    if (w < NV) {
-      const double s = double(__shfl_sync(0xffffffffu, lane_sum(lane < nact ? red[w * 32 + lane] : T(0)), 0));
-      if (lane < int(cl)) cluster_store(cluster_addr(smem_u32(&part[buf][rank][w]), uint32_t(lane)), s);
-      __syncwarp();
+  // The sums over rows carry the bits of the loop's kernels in FP32, where an
+  // ill-conditioned S makes the number of passes, and whether FP64 takes over,
+  // hang on them: FP32 within the blocks of rows that those kernels sum, in
+  // their order (p.q: 32 rows, four to a warp, then eight warps; r.z and r.r:
+  // 256 rows, 32 to a warp, then eight warps), FP64 beyond.
+  auto unit_sums = [&](auto& v, auto nv, int u) {   // a warp's 32 rows -> red[k][u], in one butterfly (warp_sums)
+    constexpr int NV = decltype(nv)::value, P = NV == 3 ? 4 : 8, PB = NV == 3 ? 2 : 3;
+    constexpr int off[5] = {NV == 3 ? 2 : 16, NV == 3 ? 1 : 8, NV == 3 ? 16 : 4, NV == 3 ? 8 : 2, NV == 3 ? 4 : 1};
+    T a[P];
+    int k = 0;
+#pragma unroll
+    for (int j = 0; j < P; ++j) a[j] = j < NV ? v[j < NV ? j : 0] : T(0);
+#pragma unroll
+    for (int b = 0; b < PB; ++b) {
+      const int h = P >> (b + 1);
+      const bool up = (lane & off[b]) != 0;
+      if (up) k += h;
+#pragma unroll
+      for (int j = 0; j < h; ++j) {
+        const T send = up ? a[j] : a[j + h], keep = up ? a[j + h] : a[j];
+        a[j] = keep + __shfl_xor_sync(0xffffffffu, send, off[b]);
+      }
     }
+    int rest = 0;
+#pragma unroll
+    for (int b = PB; b < 5; ++b) {
+      a[0] += __shfl_xor_sync(0xffffffffu, a[0], off[b]);
+      rest |= off[b];
+    }
+    if ((lane & rest) == 0 && k < NV) red[k][u] = a[0];
+  };
+  // eight warps' sums of a block of 256 rows
+  auto block256 = [](const T* u) {
+    return ((u[0] + u[4]) + (u[2] + u[6])) + ((u[1] + u[5]) + (u[3] + u[7]));
+  };
+  const int nu = rpc / 32;                 // units of this CTA
+  const int clsh = cl == 16 ? 4 : 3;       // clusters of 16 or 8
+  // the CTA's sums to every CTA of the cluster
+  auto exchange = [&](auto nv, int buf) {
+    constexpr int NV = decltype(nv)::value;
+    __syncthreads();
+    if (units) {
+      for (int i = t; i < NV * nu * int(cl); i += nt) {
+        const int o = i & (int(cl) - 1), j = i >> clsh, k = j % NV, u = j / NV;
+        cluster_store(cluster_addr(smem_u32(&unit[(6 * buf + k) * (n / 32) + own0 / 32 + u]), uint32_t(o)), red[k][u]);
+      }
+    } else if (w < NV) {
+      double s = 0.0;
+      if constexpr (NV == 3 || sizeof(T) == 8) {
+        for (int u = lane; u < nu; u += 32) s += double(red[w][u]);
+      } else {
+        for (int u = lane; u < nu / 8; u += 32) s += double(block256(&red[w][8 * u]));
+      }
+      s = __shfl_sync(0xffffffffu, lane_sum(s), 0);
+      if (lane < int(cl)) cluster_store(cluster_addr(smem_u32(&part[buf][rank][w]), uint32_t(lane)), s);
+    }
+    __syncwarp();
     cluster_barrier();
   };
+  // value k summed over the cluster, by a warp (valid in lane 0)
+  auto total = [&](auto nv, int buf, int k) -> double {
+    constexpr int NV = decltype(nv)::value;
+    double s = 0.0;
+    if (!units) {
+      s = lane < int(cl) ? part[buf][lane][k] : 0.0;
+    } else if constexpr (NV == 3) {
+      for (int u = lane; u < n / 32; u += 32) s += double(unit[(6 * buf + k) * (n / 32) + u]);
+    } else {
+      for (int u = lane; u < n / 256; u += 32) s += double(block256(&unit[(6 * buf + k) * (n / 32) + 8 * u]));
+    }
+    return lane_sum(s);
+  };
+  T xr[AFC_RPT][3];                        // this thread's rows of x
+#pragma unroll
+  for (int j = 0; j < AFC_RPT; ++j)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) xr[j][c] = t + j * nt < rpc ? x[3 * (row0 + t + j * nt) + c] : T(0);
   bool live = true;
   while (live) {
     // p = z + beta p, z = D^-1 r
@@ -177,7 +263,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
       for (int i = t; i < rpc; i += nt) {
         const T d = p[4 * i + 3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) p[4 * i + c] = r[3 * i + c] * d + b[c] * p[4 * i + c];
+        for (int c = 0; c < 3; ++c) p[4 * i + c] = fma(b[c], p[4 * i + c], mul_rn(r[3 * i + c], d));
       }
     }
     __syncwarp();
@@ -194,53 +280,64 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     // q = S p
     const int lr = t & (lpr - 1);
     for (int i = t / lpr; i < rpc; i += nt / lpr) {
-      T acc[3] = {T(0), T(0), T(0)};
-      auto add = [&](T a, const T (&v)[3]) {
+      // a thread takes the entries of lanes lr and lr + 4 of the loop's eight
+      T acc[2][3] = {{T(0), T(0), T(0)}, {T(0), T(0), T(0)}};
+      auto add = [&](T (&s)[3], T a, const T (&v)[3]) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c] += a * v[c];
+        for (int c = 0; c < 3; ++c) s[c] = fma(a, v[c], s[c]);
       };
       const int f1 = rp[i + 1], fc = min(f1, cap);
       int f = rp[i] + lr;
-#pragma unroll 4
-      for (; f < fc; f += lpr) {
-        T v[3];
+#pragma unroll 2
+      for (; f + 4 < fc; f += AFL) {
+        T v[3], u[3];
         window_load3(pw + 4 * cc[f], v);
-        add(cv[f], v);
+        window_load3(pw + 4 * cc[f + 4], u);
+        add(acc[0], cv[f], v);
+        add(acc[1], cv[f + 4], u);
       }
-      for (; f < f1; f += lpr) {   // entries that did not fit
-        const int k = int(ib.col[e0 + f] - R0);
-        T v[3];
-        if (fast) window_load3(pw + 4 * (k - w0), v);
-        else cluster_load3(owner(k), v);
-        add(val[e0 + f], v);
+      for (int h = 0; f < f1; f += 4, h ^= 1) {   // the last one, and entries that did not fit
+        T v[3], a;
+        if (f < fc) {
+          a = cv[f];
+          window_load3(pw + 4 * cc[f], v);
+        } else {
+          const int k = int(ib.col[e0 + f] - R0);
+          a = val[e0 + f];
+          if (fast) window_load3(pw + 4 * (k - w0), v);
+          else cluster_load3(owner(k), v);
+        }
+        if (h) add(acc[1], a, v);
+        else add(acc[0], a, v);
       }
       // the three sums over the row's lanes (whole warps get here together: a CTA's
-      // rows are a multiple of 16), two of them in one butterfly step
-      const int h = lpr >> 1;
-      const bool up = (lr & h) != 0;
-      T s0 = (up ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[1], h);
-      T s1 = acc[2] + __shfl_xor_sync(0xffffffffu, acc[2], h);
-      for (int o = h >> 1; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      // rows are a multiple of 32), two of them in one butterfly step
+      T s0, s1;
+      {
+        const T a0 = acc[0][0] + acc[1][0], a1 = acc[0][1] + acc[1][1], a2 = acc[0][2] + acc[1][2];
+        const bool up = (lr & 2) != 0;
+        s0 = (up ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up ? a0 : a1, 2);
+        s1 = a2 + __shfl_xor_sync(0xffffffffu, a2, 2);
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
       }
       if (lr == 0) {
         q[3 * i] = s0;
         q[3 * i + 2] = s1;
-      } else if (lr == h) {
+      } else if (lr == 2) {
         q[3 * i + 1] = s0;
       }
     }
     __syncthreads();
-    {
-      T v[3] = {T(0), T(0), T(0)};
-      for (int i = t; i < rpc; i += nt)
+    for (int i = t; i < rpc; i += nt) {
+      T v[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) v[c] += p[4 * i + c] * q[3 * i + c];
-      exchange(v, std::integral_constant<int, 3>{}, 0);
+      for (int c = 0; c < 3; ++c) v[c] = mul_rn(p[4 * i + c], q[3 * i + c]);
+      unit_sums(v, three{}, i / 32);
     }
+    exchange(three{}, 0);
     if (w < 3) {
-      const double pq = lane_sum(lane < int(cl) ? part[0][lane][w] : 0.0);
+      const double pq = total(three{}, 0, w);
       if (lane == 0) {
         KState& k = sk[w];
         if (!k.done) {
@@ -258,27 +355,28 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
       }
     }
     __syncthreads();
-    {
-      T v[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-      for (int i = t; i < rpc; i += nt) {
-        T* xi = x + 3 * (row0 + i);
-        const T d = p[4 * i + 3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          if (sk[c].done) continue;
-          const T a = sal[c];
-          atomicAdd(xi + c, a * p[4 * i + c]);   // this thread's own element: no load to wait for
-          const T rv = r[3 * i + c] - a * q[3 * i + c];
-          r[3 * i + c] = rv;
-          v[2 * c] += rv * (rv * d);
-          v[2 * c + 1] += rv * rv;
-        }
+    for (int j = 0; j < AFC_RPT; ++j) {
+      const int i = t + j * nt;
+      if (i >= rpc) break;                 // whole warps: a CTA's rows are a multiple of 32
+      const T d = p[4 * i + 3];
+      T v[6];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        v[2 * c] = v[2 * c + 1] = T(0);
+        if (sk[c].done) continue;
+        const T a = sal[c];
+        xr[j][c] = fma(a, p[4 * i + c], xr[j][c]);
+        const T rv = fma(-a, q[3 * i + c], r[3 * i + c]);
+        r[3 * i + c] = rv;
+        v[2 * c] = mul_rn(rv, mul_rn(rv, d));
+        v[2 * c + 1] = mul_rn(rv, rv);
       }
-      exchange(v, std::integral_constant<int, 6>{}, 1);
+      unit_sums(v, six{}, i / 32);
     }
+    exchange(six{}, 1);
     if (w < 3) {
-      const double rzn = lane_sum(lane < int(cl) ? part[1][lane][2 * w] : 0.0);
-      const double rr = lane_sum(lane < int(cl) ? part[1][lane][2 * w + 1] : 0.0);
+      const double rzn = total(six{}, 1, 2 * w), rr = total(six{}, 1, 2 * w + 1);
       KState& k = sk[w];
       if (lane == 0) {
         if (!k.done) {
@@ -299,6 +397,11 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     __syncthreads();
     live = !(sk[0].done && sk[1].done && sk[2].done);
   }
+#pragma unroll
+  for (int j = 0; j < AFC_RPT; ++j)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (t + j * nt < rpc) x[3 * (row0 + t + j * nt) + c] = xr[j][c];
   if (rank == 0 && t < 3) ks[3 * inst + t] = sk[t];
 }
 
