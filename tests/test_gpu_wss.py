@@ -59,3 +59,25 @@ def test_wss_matches_oracle_on_a_refined_run():
     ref, _ = ibfe.wall_shear_stress(m, o.u, X, case["UB"], nrm, case["nu"], case["rho"])
     assert rel_l2(wss, ref) <= 1e-8
     g.close()
+
+
+@pytest.mark.parametrize("M,scale", [(1, 1.0), (31, 1.0), (33, 1e-3), (70, 1e30)])
+def test_wss_point_counts_and_normal_scales(M, scale):
+    """Partly filled CTAs (32 points each), anisotropic spacing, normals of any
+    length: the oracle's formula on the library's own velocity, which it
+    evaluates for the normals as given (t scales with n, t_s with n and n^3)."""
+    from paper_2007_02082_gb300 import IBGrid
+    case = W.cylinder_case(n=(12, 14, 9), length=1.5, M=M, seed=80 + M, nu=0.05, dt=0.01)
+    X = np.asarray(case["X"])
+    g = IBGrid(case, precision="fp64")
+    m = ibfe.build_mesh(case)
+    rng = np.random.default_rng(M)
+    x = m.node_x
+    g.ib_fields_set("U", np.stack([np.sin(2 * x[:, 1]) + x[:, 2], x[:, 0] * x[:, 2], 1 - x[:, 0] ** 2], 1)
+                    + 0.01 * rng.standard_normal(x.shape))
+    nrm = _normals(X) * scale
+    wss, grad = g.ib_wss(nrm, with_grad=True)
+    ref, gref = ibfe.wall_shear_stress(m, g.ib_fields_get("U"), X, case["UB"], nrm, case["nu"], case["rho"])
+    assert rel_l2(grad, gref) <= 1e-10
+    assert rel_l2(wss / scale, ref / scale) <= 1e-10
+    g.close()
