@@ -735,6 +735,7 @@ ib_status engine_build(Engine& E) {
 
   // ---- Poisson multigrid, in the precision of the inner Krylov iterations
   CK(fe_configure());
+  CK(mg_configure());
   {
     // schedule of the persistent staged Poisson stencil: a whole number of
     // CTAs per SM (never more than chunks); CTA c takes the chunks c, c + G, ...

@@ -12,9 +12,9 @@
 //                     sweep;
 //   large levels    : 7-point operator in neighbour-list form, one thread per
 //                     node, one launch per step over all problems;
-//   small levels    : one CTA per problem runs the rest of the cycle (every
-//                     level with at most MG_SMALL_NODES nodes, and the dense
-//                     coarsest solve) with block barriers between steps.
+//   small levels    : one cluster of CTAs per problem runs the rest of the cycle
+//                     (every level with at most MG_SMALL_NODES nodes, and the
+//                     dense coarsest solve) with cluster barriers between steps.
 #include <algorithm>
 
 #include "async.cuh"
@@ -36,27 +36,37 @@ __device__ __forceinline__ bool keep_slot(uint16_t m, uint16_t dmask) {
   return (m & D_VALID) && !(m & (D_HANG | dmask));
 }
 
+// Reads of the level vectors: plain, or past the L1 cache where other CTAs of the
+// same launch write them.
+struct PlainLoad {
+  template <typename T> static __device__ __forceinline__ T ld(const T* p) { return *p; }
+};
+struct FreshLoad {
+  template <typename T> static __device__ __forceinline__ T ld(const T* p) { return __ldcg(p); }
+};
+
 // First two Jacobi steps from zero in one pass: x1 = w D^-1 b is pointwise, so
 // x2 = x1 + w D^-1 (b - A x1) takes the neighbours' x1 from their b and D^-1.
-template <typename T>
+template <typename T, typename Ld = PlainLoad>
 __device__ __forceinline__ T level_jac2(const MGLevelDev<T>& L, T omega, int64_t j) {
-  const T x1 = omega * L.dinv[j] * L.b[j];
+  const T bj = Ld::ld(L.b + j);
+  const T x1 = omega * L.dinv[j] * bj;
   T ax = L.diag[j] * x1;
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
     const int nb = L.nbr[6 * j + d];
-    if (nb >= 0) ax += L.offd[6 * j + d] * (omega * L.dinv[nb] * L.b[nb]);
+    if (nb >= 0) ax += L.offd[6 * j + d] * (omega * L.dinv[nb] * Ld::ld(L.b + nb));
   }
-  return x1 + omega * L.dinv[j] * (L.b[j] - ax);
+  return x1 + omega * L.dinv[j] * (bj - ax);
 }
 
-template <typename T>
-__device__ __forceinline__ T level_ax(const MGLevelDev<T>& L, const T* __restrict__ x, int64_t j) {
-  T v = L.diag[j] * x[j];
+template <typename T, typename Ld = PlainLoad>
+__device__ __forceinline__ T level_ax(const MGLevelDev<T>& L, const T* x, int64_t j) {
+  T v = L.diag[j] * Ld::ld(x + j);
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
     const int nb = L.nbr[6 * j + d];
-    if (nb >= 0) v += L.offd[6 * j + d] * x[nb];
+    if (nb >= 0) v += L.offd[6 * j + d] * Ld::ld(x + nb);
   }
   return v;
 }
@@ -446,16 +456,37 @@ struct SmallArgs {
   int nu;
 };
 
-constexpr int SMALL_THREADS = 1024;
+// The threads that run one problem's small levels: a cluster of CTAs (k_mg_small)
+// or one CTA (k_mg_levels); sync makes the vectors written before it visible to
+// all of them.
+struct CtaTeam {
+  int t = threadIdx.x, n = blockDim.x, rank = 0, ctas = 1;
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+struct ClusterTeam {
+  int t, n, rank, ctas;
+  __device__ ClusterTeam() {
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(ctas));
+    t = rank * int(blockDim.x) + int(threadIdx.x);
+    n = ctas * int(blockDim.x);
+  }
+  __device__ __forceinline__ void sync() const {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+};
 
-// The small levels and the coarsest solve of problem i, by the whole CTA
-// (block barriers between steps); each node's value is computed by one
-// thread, in an order that does not depend on the CTA's size.
-template <typename T>
-__device__ void small_cycle(const SmallArgs<T>& a, int i, const KState* ks) {
+// The small levels and the coarsest solve of problem i, by the whole team;
+// each node's value is computed by one thread, in an order that does not
+// depend on the team.  tile: tile_len values of shared memory for the
+// dense inverse.
+template <typename T, typename Team>
+__device__ void small_cycle(const SmallArgs<T>& a, int i, const KState* ks, const Team& tm, T* tile, int tile_len) {
+  using Ld = FreshLoad;
   if (!a.on[i] || ks[i].done) return;
   const int k0 = a.small[i], K = a.coarsest[i];
-  const int t = threadIdx.x, nt = blockDim.x;
+  const int t = tm.t, nt = tm.n;
   // down: pre-smoothing, residual, restriction
   for (int k = k0; k < K; ++k) {
     const MGLevelDev<T>& L = a.lev[k];
@@ -464,40 +495,58 @@ __device__ void small_cycle(const SmallArgs<T>& a, int i, const KState* ks) {
     T* oth = L.xb;
     int s0 = 1;
     if (a.nu >= 2) {   // the first two steps in one pass, result in xb
-      for (int j = j0 + t; j < j1; j += nt) L.xb[j] = level_jac2(L, a.omega, j);
+      for (int j = j0 + t; j < j1; j += nt) L.xb[j] = level_jac2<T, Ld>(L, a.omega, j);
       cur = L.xb;
       oth = L.xa;
       s0 = 2;
     } else {
-      for (int j = j0 + t; j < j1; j += nt) L.xa[j] = a.omega * L.dinv[j] * L.b[j];
+      for (int j = j0 + t; j < j1; j += nt) L.xa[j] = a.omega * L.dinv[j] * Ld::ld(L.b + j);
     }
-    __syncthreads();
+    tm.sync();
     for (int s = s0; s < a.nu; ++s) {
-      for (int j = j0 + t; j < j1; j += nt) oth[j] = cur[j] + a.omega * L.dinv[j] * (L.b[j] - level_ax(L, cur, j));
-      __syncthreads();
+      for (int j = j0 + t; j < j1; j += nt)
+        oth[j] = Ld::ld(cur + j) + a.omega * L.dinv[j] * (Ld::ld(L.b + j) - level_ax<T, Ld>(L, cur, j));
+      tm.sync();
       T* tmp = cur; cur = oth; oth = tmp;
     }
-    for (int j = j0 + t; j < j1; j += nt) L.res[j] = L.b[j] - level_ax(L, cur, j);
-    __syncthreads();
+    for (int j = j0 + t; j < j1; j += nt) L.res[j] = Ld::ld(L.b + j) - level_ax<T, Ld>(L, cur, j);
+    tm.sync();
     const MGLevelDev<T>& C = a.lev[k + 1];
     for (int j = C.noff[i] + t; j < C.noff[i + 1]; j += nt) {
       T v = T(0);
-      for (int e = C.rptr[j]; e < C.rptr[j + 1]; ++e) v += C.rw[e] * L.res[C.rcol[e]];
+      for (int e = C.rptr[j]; e < C.rptr[j + 1]; ++e) v += C.rw[e] * Ld::ld(L.res + C.rcol[e]);
       C.b[j] = v;
     }
-    __syncthreads();
+    tm.sync();
   }
-  // coarsest: x = A^-1 b with the (symmetrised) dense inverse, read by columns
+  // coarsest: x = A^-1 b with the (symmetrised) dense inverse, by columns; each
+  // CTA takes a range of rows and stages their entries in shared memory (a
+  // row's sum is one chain of n terms: from memory its loads would wait in turn)
   {
     const MGLevelDev<T>& L = a.lev[K];
     const int j0 = L.noff[i], n = L.noff[i + 1] - j0;
     const T* Ai = a.cinv + a.cinv_off[i];
-    for (int r = t; r < n; r += nt) {
+    const int nr = (n + tm.ctas - 1) / tm.ctas, r0 = min(tm.rank * nr, n), rows = min(nr, n - r0);
+    const int ct = max(1, tile_len / (nr + 1));   // columns of a tile, after their entries of b
+    for (int rb = 0; rb < rows; rb += int(blockDim.x)) {
+      const int m = min(rows - rb, int(blockDim.x));
       T v = T(0);
-      for (int c = 0; c < n; ++c) v += Ai[(int64_t)c * n + r] * L.b[j0 + c];
-      L.xa[j0 + r] = v;
+      for (int c0 = 0; c0 < n; c0 += ct) {
+        const int nc = min(ct, n - c0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nc * m; e += blockDim.x) {
+          const int c = e / m;
+          tile[nc + e] = Ai[(int64_t)(c0 + c) * n + r0 + rb + (e - c * m)];
+        }
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) tile[c] = Ld::ld(L.b + j0 + c0 + c);
+        __syncthreads();
+        if (int(threadIdx.x) < m)
+#pragma unroll 8
+          for (int c = 0; c < nc; ++c) v += tile[nc + c * m + threadIdx.x] * tile[c];
+      }
+      if (int(threadIdx.x) < m) L.xa[j0 + r0 + rb + threadIdx.x] = v;
     }
-    __syncthreads();
+    tm.sync();
   }
   // up: prolongation, post-smoothing; each level's result ends in xa
   for (int k = K - 1; k >= k0; --k) {
@@ -507,24 +556,52 @@ __device__ void small_cycle(const SmallArgs<T>& a, int i, const KState* ks) {
     T* cur = (a.nu % 2 == 1) ? L.xa : L.xb;          // pre-smoothed iterate
     T* y = (a.nu % 2 == 0) ? L.xa : L.xb;
     for (int j = j0 + t; j < j1; j += nt) {
-      T v = cur[j];
-      for (int e = C.pptr[j]; e < C.pptr[j + 1]; ++e) v += C.pw[e] * C.xa[C.pcol[e]];
+      T v = Ld::ld(cur + j);
+      for (int e = C.pptr[j]; e < C.pptr[j + 1]; ++e) v += C.pw[e] * Ld::ld(C.xa + C.pcol[e]);
       y[j] = v;
     }
-    __syncthreads();
+    tm.sync();
     T* o = (y == L.xa) ? L.xb : L.xa;
     for (int s = 0; s < a.nu; ++s) {
-      for (int j = j0 + t; j < j1; j += nt) o[j] = y[j] + a.omega * L.dinv[j] * (L.b[j] - level_ax(L, y, j));
-      __syncthreads();
+      for (int j = j0 + t; j < j1; j += nt)
+        o[j] = Ld::ld(y + j) + a.omega * L.dinv[j] * (Ld::ld(L.b + j) - level_ax<T, Ld>(L, y, j));
+      if (k > k0 || s + 1 < a.nu) tm.sync();
       T* tmp = y; y = o; o = tmp;
     }
   }
 }
 
+// The small levels of one problem by a cluster of SMALL_CTAS CTAs: the steps are
+// a chain of about 6 per level over at most 8192 nodes and a dense product, bound by
+// the latency of each step; a cluster's threads take one or two nodes each
+// and its hardware barrier costs what a CTA's does.  One CTA of 1024 threads took
+// 41-60 us a cycle, the cluster 24-32 us (same bits).
+constexpr int SMALL_CTAS = 8;
+constexpr int SMALL_THREADS = 512;
+constexpr int SMALL_TILE = 96 * 1024;   // bytes of shared memory for the dense inverse's tile
 template <typename T>
 __global__ void __launch_bounds__(SMALL_THREADS) k_mg_small(SmallArgs<T> a, const KState* ks) {
   KCOUNT();
-  small_cycle(a, blockIdx.x, ks);
+  extern __shared__ __align__(16) unsigned char small_sm[];
+  const ClusterTeam tm;
+  small_cycle(a, int(blockIdx.x) / tm.ctas, ks, tm, reinterpret_cast<T*>(small_sm), SMALL_TILE / int(sizeof(T)));
+}
+
+template <typename T>
+void launch_small(const SmallArgs<T>& a, int ninst, const KState* ks, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(ninst * SMALL_CTAS));
+  cfg.blockDim = dim3(SMALL_THREADS);
+  cfg.dynamicSmemBytes = SMALL_TILE;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = SMALL_CTAS;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_mg_small<T>, a, ks);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
 // ---------------------------------------------------------------- persistent coarse levels
@@ -539,6 +616,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_mg_small(SmallArgs<T> a, cons
 // (cooperative launch); each barrier wait is bounded in wall-clock time, and
 // on expiry the CTA records ASYNC_TIMEOUT for every problem and returns.
 constexpr int LV_THREADS = 512;
+constexpr int LV_TILE = 4096;   // values of shared memory for the dense inverse
 
 template <typename T>
 struct LevelsArgs {
@@ -626,7 +704,11 @@ __global__ void __launch_bounds__(LV_THREADS) k_mg_levels(LevelsArgs<T> a, const
     if (!grid_barrier(a.bar, a.ninst, a.aerr)) return;
   }
   // small levels and the coarsest solve, a CTA per problem
-  for (int i = blockIdx.x; i < a.ninst; i += gridDim.x) small_cycle(S, i, ks);
+  __shared__ T tile[LV_TILE];
+  for (int i = blockIdx.x; i < a.ninst; i += gridDim.x) {
+    __syncthreads();
+    small_cycle(S, i, ks, CtaTeam(), tile, LV_TILE);
+  }
   if (!grid_barrier(a.bar, a.ninst, a.aerr)) return;
   // levels up: prolongation, post-smoothing; each level's result ends in xa
   for (int k = a.max_big - 1; k >= 0; --k) {
@@ -727,8 +809,8 @@ void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T*
     IBG_LAUNCH(k_mg_l_restrict<T>, nblk256(mg.lev[k + 1].n), 256, 0, st, mg.lev[k + 1], (const T*)L.res, k, mg.on,
                mg.small, ks);
   }
-  // small levels and the coarsest solve, one CTA per problem
-  IBG_LAUNCH(k_mg_small<T>, mg.ninst, SMALL_THREADS, 0, st, sa, ks);
+  // small levels and the coarsest solve, one cluster per problem
+  launch_small(sa, mg.ninst, ks, st);
   // large levels, up
   for (int k = mg.max_big - 1; k >= 0; --k) {
     const MGLevelDev<T>& L = mg.lev[k];
@@ -758,6 +840,12 @@ void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T*
     fe_expand2<T>(g, 1, o, (T*)nullptr, st);
     T* tmp = y; y = o; o = tmp;
   }
+}
+
+cudaError_t mg_configure() {
+  cudaError_t e = cudaFuncSetAttribute(k_mg_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMALL_TILE);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_mg_small<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMALL_TILE);
 }
 
 template <typename T>

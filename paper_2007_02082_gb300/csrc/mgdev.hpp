@@ -83,6 +83,8 @@ struct MGDev {
 // the composite Jacobi inverse.  Problems whose KState is done are skipped.
 // With prof set, launches are timed by class: pcls + 0 the composite stencil
 // applies, pcls + 1 the composite smoothing updates, pcls + 2 the rest.
+// kernel attributes (shared memory), once per device
+cudaError_t mg_configure();
 // CTAs of the cooperative coarse-level kernel that fit on the device at once
 // (at most two per SM), 0 if the query fails
 template <typename T>
