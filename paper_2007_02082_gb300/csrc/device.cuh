@@ -385,20 +385,15 @@ __device__ __forceinline__ bool segment_sums_last(const double* __restrict__ par
   return true;
 }
 
-// The grid reduction: every thread's NV contributions are summed per instance
-// into out[i * NV + k] (out follows the gridDim.x * NV partials; the group
-// sums follow out).  inst: the instance of this CTA, whose CTAs are
-// seg[inst] .. seg[inst + 1].  counter: 1 + gridDim.x words, zero before
-// and after.  Returns true in the last CTA only, after a barrier that makes
-// out visible to all its threads.
-template <typename T, int NV>
-__device__ __forceinline__ bool grid_sum_last(T (&v)[NV], double* __restrict__ partials,
-                                              unsigned* __restrict__ counter, const int32_t* __restrict__ seg,
-                                              int nseg, int inst, double* __restrict__ out) {
-  __shared__ T sht[32 * NV];
+// The stages after the CTA totals: this CTA's partials[NV * blockIdx.x + k] have
+// been written (by any of its threads).
+template <int NV>
+__device__ __forceinline__ bool grid_finish(double* __restrict__ partials, unsigned* __restrict__ counter,
+                                            const int32_t* __restrict__ seg, int nseg, int inst,
+                                            double* __restrict__ out) {
   __shared__ bool last;
   double* gpart = out + (int64_t)nseg * NV;
-  block_sum<T, NV>(v, sht, [&](int k, T x) { partials[(int64_t)blockIdx.x * NV + k] = double(x); });
+  __syncthreads();
   const int s0 = seg[inst], s1 = seg[inst + 1];
   const int first = s0 + (int(blockIdx.x) - s0) / RED_GROUP * RED_GROUP, gn = min(RED_GROUP, s1 - first);
   if (threadIdx.x == 0) {
@@ -422,6 +417,21 @@ __device__ __forceinline__ bool grid_sum_last(T (&v)[NV], double* __restrict__ p
   instance_totals<NV>(gpart, seg, nseg, out);
   if (threadIdx.x == 0) *counter = 0u;
   return true;
+}
+
+// The grid reduction: every thread's NV contributions are summed per instance
+// into out[i * NV + k] (out follows the gridDim.x * NV partials; the group
+// sums follow out).  inst: the instance of this CTA, whose CTAs are
+// seg[inst] .. seg[inst + 1].  counter: 1 + gridDim.x words, zero before
+// and after.  Returns true in the last CTA only, after a barrier that makes
+// out visible to all its threads.
+template <typename T, int NV>
+__device__ __forceinline__ bool grid_sum_last(T (&v)[NV], double* __restrict__ partials,
+                                              unsigned* __restrict__ counter, const int32_t* __restrict__ seg,
+                                              int nseg, int inst, double* __restrict__ out) {
+  __shared__ T sht[32 * NV];
+  block_sum<T, NV>(v, sht, [&](int k, T x) { partials[(int64_t)blockIdx.x * NV + k] = double(x); });
+  return grid_finish<NV>(partials, counter, seg, nseg, inst, out);
 }
 
 }  // namespace ibg

@@ -961,19 +961,20 @@ __global__ void __launch_bounds__(512) k_poisson_cg(DevGrid g, const T* __restri
 // of the 256 incident-cell masks in shared memory.  The arithmetic is that of
 // k_poisson_cg, in the same order.
 // ring depth: the apply (3.5 KB per brick from memory) keeps 4 bricks ahead,
-// eight CTAs per SM; the CG form (6.5 KB per brick, twice the stage) 3 ahead,
-// six CTAs per SM
-template <int NV>
-__host__ __device__ constexpr int p7_stages() { return NV == 2 ? 4 : 5; }
+// eight CTAs per SM; the CG form (6.5 KB per brick, twice the stage) and the
+// smoothing form (8.5 KB) 3 ahead, six CTAs per SM
+template <int NV, int NX = 0>
+__host__ __device__ constexpr int p7_stages() { return NV == 2 || NX ? 4 : 5; }
 constexpr int P7_THREADS = 128;
 constexpr int P7_CHUNK = 8;    // bricks per chunk at most (the chunk table's)
-template <int NV>   // input vectors: 2 (z and p_old) for the CG form, 1 for the apply
-struct P7Stage {
+template <int NV, int NX = 0>   // input vectors: 2 (z and p_old) for the CG form, 1 for the apply
+struct P7Stage {               // and own values only (r and 1/diag of the smoothing form)
   // per vector 896 floats: the brick's own 512 values, then the face halos,
   // face f (-x, +x, -y, +y, -z, +z) at 512 + 64 f, its element (u, v) at 8 v + u
   static constexpr int VEC = 896;
   static constexpr int META = NV * VEC * 4;       // 512 x uint16
-  static constexpr int BYTES = META + 1024;
+  static constexpr int OWN = META + 1024;         // NX x 512 values
+  static constexpr int BYTES = OWN + NX * 2048;
 };
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src, bool fill) {
@@ -1019,17 +1020,20 @@ __device__ __forceinline__ P7Copies p7_copies(int t) {
 // Fill one stage with brick i of the chunk (every thread calls it): warp 0
 // issues the bulk copies, every thread its face copies.  nbf[6 i + f] is the
 // neighbour brick across face f.
-template <int NV>
+template <int NV, int NX = 0>
 __device__ __forceinline__ void p7_issue(const DevGrid& g, unsigned char* stage, uint64_t* bar, int b,
                                          const int* nbf, int i, const float* v0, const float* v1,
-                                         const P7Copies& c) {
+                                         const P7Copies& c, const float* x0 = nullptr, const float* x1 = nullptr) {
   const int t = threadIdx.x;
   float* sv = reinterpret_cast<float*>(stage);
   if (t < 32) {
-    if (t == 0) mbar_arrive_expect_tx(bar, uint32_t(NV * 2048 + 1024));
+    if (t == 0) mbar_arrive_expect_tx(bar, uint32_t((NV + NX) * 2048 + 1024));
     __syncwarp();
     if (t < NV) bulk_g2s(sv + t * P7Stage<NV>::VEC, (t ? v1 : v0) + (int64_t)b * DBV, 2048u, bar);
     else if (t == NV) bulk_g2s(stage + P7Stage<NV>::META, g.meta + (int64_t)b * DBV, 1024u, bar);
+    else if (t <= NV + NX)
+      bulk_g2s(stage + P7Stage<NV, NX>::OWN + 2048 * (t - NV - 1), (t == NV + 1 ? x0 : x1) + (int64_t)b * DBV, 2048u,
+               bar);
   }
   const int na = nbf[6 * i + c.fa];
   const int64_t sa = na >= 0 ? (int64_t)na * DBV + c.ha : 0;
@@ -1048,16 +1052,27 @@ __device__ __forceinline__ void p7_issue(const DevGrid& g, unsigned char* stage,
   cp_async_commit();
 }
 
-template <bool CG>
-__global__ void __launch_bounds__(P7_THREADS, 8)
+//
+// SMOOTH: one damped-Jacobi sweep of the V-cycle in the same pass, z_out =
+// z + omega D^-1 (r - K z), with the arithmetic of the apply followed by
+// k_mg_c_smooth (pold: r, pnew: z_out).  Its stage also takes r and 1/diag of the
+// brick's own nodes, so K z is neither written nor read again: 18 bytes a
+// node instead of 32.  Nodes whose K z is an interface sum are left to
+// k_mg_if_smooth: q receives the level's part at interface and hanging nodes
+// only.  Bound by the stages in flight, as the apply.  A sweep of the 16 M-node
+// sac with its interface nodes: 98 -> 74 us (apply, sums, update -> one pass, interface nodes).
+template <bool CG, bool SMOOTH = false>
+__global__ void __launch_bounds__(P7_THREADS, SMOOTH ? 6 : 8)
     k_poisson7_staged(DevGrid g, const float* __restrict__ z, const float* __restrict__ pold,
                       float* __restrict__ pnew, float* __restrict__ q, uint16_t dmask, KState* __restrict__ ks,
-                      double* __restrict__ partials, unsigned* __restrict__ counter, const uint8_t* __restrict__ on) {
+                      double* __restrict__ partials, unsigned* __restrict__ counter, const uint8_t* __restrict__ on,
+                      const float* __restrict__ dinv = nullptr, float omega = 0.f) {
   KCOUNT();
   constexpr int NV = CG ? 2 : 1;
+  constexpr int NX = SMOOTH ? 2 : 0;
   constexpr int VEC = P7Stage<NV>::VEC;
-  using S = P7Stage<NV>;
-  constexpr int P7_STAGES = p7_stages<NV>();
+  using S = P7Stage<NV, NX>;
+  constexpr int P7_STAGES = p7_stages<NV, NX>();
   extern __shared__ unsigned char p7_dyn[];
   __shared__ __align__(8) uint64_t full[P7_STAGES];
   __shared__ int nbf[6 * P7_CHUNK];
@@ -1100,7 +1115,7 @@ __global__ void __launch_bounds__(P7_THREADS, 8)
     const int ozm = lz > 0 ? o - 64 : DBV + 256 + 8 * ly + 4 * seg, ozp = lz < 7 ? o + 64 : DBV + 320 + 8 * ly + 4 * seg;
     const int oxl = seg ? o - 1 : DBV + 8 * lz + ly, oxr = seg ? DBV + 64 + 8 * lz + ly : o + 4;
     for (int k = 0; k < P7_STAGES - 1; ++k) {
-      if (k < n) p7_issue<NV>(g, sm + k * S::BYTES, &full[k], b0 + k, nbf, k, z, pold, cc);
+      if (k < n) p7_issue<NV, NX>(g, sm + k * S::BYTES, &full[k], b0 + k, nbf, k, z, pold, cc, pold, dinv);
       else cp_async_commit();
     }
     for (int i = 0; i < n; ++i) {
@@ -1110,7 +1125,7 @@ __global__ void __launch_bounds__(P7_THREADS, 8)
       __syncthreads();   // stage k complete and visible; every thread is past brick i - 1
       {
         const int ir = i + P7_STAGES - 1, kr = ir % P7_STAGES;   // the stage of brick i - 1
-        if (ir < n) p7_issue<NV>(g, sm + kr * S::BYTES, &full[kr], b0 + ir, nbf, ir, z, pold, cc);
+        if (ir < n) p7_issue<NV, NX>(g, sm + kr * S::BYTES, &full[kr], b0 + ir, nbf, ir, z, pold, cc, pold, dinv);
         else cp_async_commit();
       }
       const unsigned char* st = sm + k * S::BYTES;
@@ -1168,7 +1183,25 @@ __global__ void __launch_bounds__(P7_THREADS, 8)
         if (m[j] & dmask) out[j] = 0.f;
       // brick padding: the inputs are zero there, so are p and the output
       const int64_t s = (int64_t)(b0 + i) * DBV + o;
-      *reinterpret_cast<float4*>(q + s) = make_float4(out[0], out[1], out[2], out[3]);
+      if constexpr (SMOOTH) {
+        const float4 rv = *reinterpret_cast<const float4*>(st + S::OWN + 4 * o);
+        const float4 dv = *reinterpret_cast<const float4*>(st + S::OWN + 2048 + 4 * o);
+        const float re[4] = {rv.x, rv.y, rv.z, rv.w}, de[4] = {dv.x, dv.y, dv.z, dv.w};
+        float zo[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool keep = (m[j] & D_VALID) && !(m[j] & (D_HANG | dmask));
+          zo[j] = keep ? float(pv[j] + omega * de[j] * (re[j] - out[j])) : 0.f;
+        }
+        *reinterpret_cast<float4*>(pnew + s) = make_float4(zo[0], zo[1], zo[2], zo[3]);
+        if ((m[0] | m[1] | m[2] | m[3]) & (D_IFACE | D_HANG)) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (m[j] & (D_IFACE | D_HANG)) q[s + j] = out[j];
+        }
+      } else {
+        *reinterpret_cast<float4*>(q + s) = make_float4(out[0], out[1], out[2], out[3]);
+      }
       if constexpr (CG) {
         *reinterpret_cast<float4*>(pnew + s) = pc;
 #pragma unroll
@@ -1191,8 +1224,8 @@ __global__ void __launch_bounds__(P7_THREADS, 8)
   }
 }
 
-template <int NV>
-static constexpr size_t p7_smem() { return size_t(p7_stages<NV>()) * P7Stage<NV>::BYTES + 128; }
+template <int NV, int NX = 0>
+static constexpr size_t p7_smem() { return size_t(p7_stages<NV, NX>()) * P7Stage<NV, NX>::BYTES + 128; }
 
 // ---------------------------------------------------------------- persistent Poisson stencil
 // A launch choice (IB_TUNE_POISSON_KERNEL = 3): the staged kernel above made
@@ -1442,7 +1475,7 @@ static bool launch_p7(const DevGrid& g, const T* z, const T* pold, T* pnew, T* q
       return true;
     }
     IBG_LAUNCH((k_poisson7_staged<CG>), g.nchunks, P7_THREADS, p7_smem<CG ? 2 : 1>(), st, g, z, pold, pnew, q, dmask,
-               ks, partials, counter, on);
+               ks, partials, counter, on, (const float*)nullptr, 0.f);
     return true;
   }
 }
@@ -1813,6 +1846,22 @@ void fe_poisson_apply(const DevGrid& g, const T* x, T* q, uint16_t dmask, KState
                (double*)nullptr, (unsigned*)nullptr, on);
 }
 
+// The fused sweep is an instance of the staged kernel: FP32 on 16-byte
+// boundaries, not under the launch choices of the other two stencil kernels.
+template <typename T>
+bool fe_poisson_smooth(const DevGrid& g, const T* z, T* zout, const T* r, T* q, const T* dinv, T omega,
+                       uint16_t dmask, KState* ks, const uint8_t* on, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    if (g.poisson_kernel > 1 || !a16(z) || !a16(zout) || !a16(r) || !a16(dinv)) return false;
+    IBG_LAUNCH((k_poisson7_staged<false, true>), g.nchunks, P7_THREADS, (p7_smem<1, 2>()), st, g, z, r, zout, q, dmask,
+               ks, (double*)nullptr, (unsigned*)nullptr, on, dinv, omega);
+    return true;
+  } else {
+    return false;
+  }
+}
+
 template <typename T>
 void fe_sync(const DevGrid& g, int nc, T* y, uint16_t dmask, cudaStream_t st) {
   if (g.n_if == 0) return;
@@ -1894,15 +1943,17 @@ cudaError_t fe_configure() {
   cudaError_t e = cudaFuncSetAttribute(k_apply15_mom32<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        int(cudaSharedmemCarveoutMaxShared));
   if (e != cudaSuccess) return e;
-  for (auto k : {k_poisson7_staged<true>, k_poisson7_staged<false>, k_poisson7_persist<true>,
-                 k_poisson7_persist<false>}) {
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  int(cudaSharedmemCarveoutMaxShared))) != cudaSuccess)
-      return e;
-    const size_t mx = std::max(std::max(p7_smem<1>(), p7_smem<2>()), std::max(p7p_smem<1>(), p7p_smem<2>()));
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(mx))) != cudaSuccess)
-      return e;
-  }
+  auto staged = [&](auto k, size_t smem) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  };
+  staged(k_poisson7_staged<true>, p7_smem<2>());
+  staged(k_poisson7_staged<false>, p7_smem<1>());
+  staged(k_poisson7_staged<false, true>, p7_smem<1, 2>());
+  staged(k_poisson7_persist<true>, p7p_smem<2>());
+  staged(k_poisson7_persist<false>, p7p_smem<1>());
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_apply15_mom32<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               int(cudaSharedmemCarveoutMaxShared));
 }
@@ -1962,6 +2013,10 @@ template void fe_apply_local<double>(const DevGrid&, const OpDesc<double>&, int,
                                      cudaStream_t);
 template void fe_poisson_apply<float>(const DevGrid&, const float*, float*, uint16_t, KState*, const uint8_t*,
                                       cudaStream_t);
+template bool fe_poisson_smooth<float>(const DevGrid&, const float*, float*, const float*, float*, const float*, float,
+                                      uint16_t, KState*, const uint8_t*, cudaStream_t);
+template bool fe_poisson_smooth<double>(const DevGrid&, const double*, double*, const double*, double*,
+                                       const double*, double, uint16_t, KState*, const uint8_t*, cudaStream_t);
 template void fe_poisson_apply<double>(const DevGrid&, const double*, double*, uint16_t, KState*, const uint8_t*,
                                        cudaStream_t);
 template void fe_sync<double>(const DevGrid&, int, double*, uint16_t, cudaStream_t);

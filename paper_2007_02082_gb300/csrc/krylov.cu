@@ -302,25 +302,29 @@ __global__ void __launch_bounds__(512) k_cg_start_r(DevGrid g, const T* __restri
   }
 }
 
-// k_cg_update_vec without the preconditioner: x += alpha p, r -= alpha q
-// (q interface-summed), ||r||^2 -> convergence and iteration cap
+// k_cg_update_vec with the preconditioner's first step in its place: x += alpha p,
+// r -= alpha q (q interface-summed), z = w D^-1 r (w = omega with multigrid, 1
+// without: the V-cycle's first smoothing step, which would read r
+// again), ||r||^2 -> convergence and iteration cap
 template <typename T>
 __global__ void __launch_bounds__(512) k_cg_update_r(DevGrid g, T* __restrict__ x, T* __restrict__ r,
                                                      const T* __restrict__ p, const T* __restrict__ q,
-                                                     uint16_t dmask, KState* ks, double* partials,
-                                                     unsigned* counter) {
+                                                     T* __restrict__ z, const T* __restrict__ dinv,
+                                                     const uint8_t* __restrict__ on, T omega, uint16_t dmask,
+                                                     KState* ks, double* partials, unsigned* counter) {
   KCOUNT();
   using V = typename Vec16<T>::type;
   using MT = typename Vec16<T>::mt;
   constexpr int W = Vec16<T>::W;
   const int b0 = g.scbrick[blockIdx.x], b1 = g.scbrick[blockIdx.x + 1];
-  const KState& k = ks[g.binst[b0]];
+  const int inst = g.binst[b0];
+  const KState& k = ks[inst];
   T tv[1] = {T(0)};
   if (!k.done) {
-    const T a = k_alpha<T>(k);
+    const T a = k_alpha<T>(k), w = on[inst] ? omega : T(1);
     const int64_t s1 = (int64_t)b1 * DBV;
-  #pragma unroll 2
-  for (int64_t s = (int64_t)b0 * DBV + threadIdx.x * W; s < s1; s += (int64_t)blockDim.x * W) {
+#pragma unroll 2
+    for (int64_t s = (int64_t)b0 * DBV + threadIdx.x * W; s < s1; s += (int64_t)blockDim.x * W) {
       const MT mv = *reinterpret_cast<const MT*>(g.meta + s);
       const uint16_t* mm = reinterpret_cast<const uint16_t*>(&mv);
       if (!(vec_or_n<W>(mm) & D_VALID)) continue;   // brick padding: always zero, never read or written
@@ -328,10 +332,14 @@ __global__ void __launch_bounds__(512) k_cg_update_r(DevGrid g, T* __restrict__ 
       V rv = *reinterpret_cast<const V*>(r + s);
       V pv = *reinterpret_cast<const V*>(p + s);
       V qv = *reinterpret_cast<const V*>(q + s);
+      const V dv = *reinterpret_cast<const V*>(dinv + s);
+      V zv;
       T* xe = reinterpret_cast<T*>(&xv);
       T* re = reinterpret_cast<T*>(&rv);
       T* pe = reinterpret_cast<T*>(&pv);
       T* qe = reinterpret_cast<T*>(&qv);
+      T* ze = reinterpret_cast<T*>(&zv);
+      const T* de = reinterpret_cast<const T*>(&dv);
 #pragma unroll
       for (int j = 0; j < W; ++j) {
         const uint16_t m = mm[j];
@@ -339,10 +347,12 @@ __global__ void __launch_bounds__(512) k_cg_update_r(DevGrid g, T* __restrict__ 
         if (m & D_VALID) xe[j] += a * pe[j];
         const T rn = kkeep(m, dmask) ? T(re[j] - a * qq) : T(0);
         re[j] = rn;
+        ze[j] = T(w * de[j] * rn);   // zero where r is
         if (kdof(m, dmask)) tv[0] += rn * rn;
       }
       *reinterpret_cast<V*>(x + s) = xv;
       *reinterpret_cast<V*>(r + s) = rv;
+      *reinterpret_cast<V*>(z + s) = zv;
     }
   }
   double* out = partials + (int64_t)gridDim.x;
@@ -358,20 +368,55 @@ __global__ void __launch_bounds__(512) k_cg_update_r(DevGrid g, T* __restrict__ 
   }
 }
 
-// r.z over DOF slots -> beta (0 on the first pass), rz; loop condition
+// r.z over DOF slots -> beta (0 on the first pass), rz; loop condition.  Every
+// thread takes W consecutive nodes of each brick of the chunk with 16-byte loads (a
+// CTA of 512 / W threads); the W sums of a thread stand for W threads
+// of one node each and are added in the order of their trees, so that the
+// bits are those of a 512-thread CTA with a node a thread.  Bound by HBM:
+// 2V + 2 bytes a slot (16 M-node sac: 61 us with one value a load, 36 here).
 template <typename T>
 __global__ void __launch_bounds__(512) k_cg_rz(DevGrid g, const T* __restrict__ r, const T* __restrict__ z,
                                                uint16_t dmask, KState* ks, double* partials, unsigned* counter,
                                                Cond cond, int first) {
   KCOUNT();
+  using V = typename Vec16<T>::type;
+  using MT = typename Vec16<T>::mt;
+  constexpr int W = Vec16<T>::W, TW = 32 / W;   // TW threads stand for a warp
+  __shared__ T sh[16];
   const int b0 = g.scbrick[blockIdx.x], b1 = g.scbrick[blockIdx.x + 1];
-  const KState& k = ks[g.binst[b0]];
-  T tv[1] = {T(0)};
-  if (!k.done)
-    for (int64_t s = (int64_t)b0 * DBV + threadIdx.x; s < (int64_t)b1 * DBV; s += blockDim.x)
-      if (kdof(g.meta[s], dmask)) tv[0] += r[s] * z[s];
+  const int inst = g.binst[b0];
+  T a[W];
+#pragma unroll
+  for (int j = 0; j < W; ++j) a[j] = T(0);
+  if (!ks[inst].done)
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) {
+      const int64_t s = (int64_t)b * DBV + threadIdx.x * W;
+      const MT mv = *reinterpret_cast<const MT*>(g.meta + s);
+      const V rv = *reinterpret_cast<const V*>(r + s), zv = *reinterpret_cast<const V*>(z + s);
+      const uint16_t* mm = reinterpret_cast<const uint16_t*>(&mv);
+      const T* re = reinterpret_cast<const T*>(&rv);
+      const T* ze = reinterpret_cast<const T*>(&zv);
+#pragma unroll
+      for (int j = 0; j < W; ++j)
+        if (kdof(mm[j], dmask)) a[j] += re[j] * ze[j];
+    }
+#pragma unroll
+  for (int o = TW / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < W; ++j) a[j] += __shfl_xor_sync(0xffffffffu, a[j], o);
+#pragma unroll
+  for (int o = W / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < o; ++j) a[j] += a[j + o];
+  if (threadIdx.x % TW == 0) sh[threadIdx.x / TW] = a[0];
+  __syncthreads();
   double* out = partials + (int64_t)gridDim.x;
-  if (!grid_sum_last<T, 1>(tv, partials, counter, g.scseg, g.ninst, g.binst[b0], out)) return;
+  if (threadIdx.x < 32) {
+    const T v = lane_sum(threadIdx.x < 16 ? sh[threadIdx.x] : T(0));
+    if (threadIdx.x == 0) partials[blockIdx.x] = double(v);
+  }
+  if (!grid_finish<1>(partials, counter, g.scseg, g.ninst, inst, out)) return;
   bool any = false;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
     KState& kk = ks[i];
@@ -930,18 +975,18 @@ static cudaError_t cg_mg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const M
   IBG_LAUNCH(k_cg_start_r<T>, g.nbricks, DBV, 0, st, g, b, x_zero ? (const T*)nullptr : (const T*)w.q, w.r, A.dmask,
              a.ks, rb.partials, rb.counter, skip_os);
   mg_vcycle<T>(g, mg, w.r, w.z, zs, w.q, A.dinv, A.dmask, a.ks, st, a.prof, 9);
-  IBG_LAUNCH(k_cg_rz<T>, g.nschunks, DBV, 0, st, g, w.r, w.z, A.dmask, a.ks, rb.partials, rb.counter, cond, 1);
+  IBG_LAUNCH(k_cg_rz<T>, g.nschunks, DBV / Vec16<T>::W, 0, st, g, w.r, w.z, A.dmask, a.ks, rb.partials, rb.counter, cond, 1);
   auto iter = [&](cudaStream_t s, const Cond& c, T* pold, T* pnew) {
     pbegin(a.prof, a.pbase + 0, s);
     fe_apply_cg<T>(g, A, 1, w.z, pold, pnew, w.q, a.ks, rb, s);
     pend(a.prof, s);
     fe_sync<T>(g, 1, w.q, A.dmask, s);
     pbegin(a.prof, a.pbase + 1, s);
-    IBG_LAUNCH(k_cg_update_r<T>, g.nschunks, DBV, 0, s, g, x, w.r, pnew, w.q, A.dmask, a.ks, rb.partials,
-               rb.counter);
+    IBG_LAUNCH(k_cg_update_r<T>, g.nschunks, DBV, 0, s, g, x, w.r, pnew, w.q, w.z, A.dinv, mg.on, mg.omega,
+               A.dmask, a.ks, rb.partials, rb.counter);
     pend(a.prof, s);
-    mg_vcycle<T>(g, mg, w.r, w.z, zs, w.q, A.dinv, A.dmask, a.ks, s, a.prof, 9);
-    IBG_LAUNCH(k_cg_rz<T>, g.nschunks, DBV, 0, s, g, w.r, w.z, A.dmask, a.ks, rb.partials, rb.counter, c, 0);
+    mg_vcycle<T>(g, mg, w.r, w.z, zs, w.q, A.dinv, A.dmask, a.ks, s, a.prof, 9, true);
+    IBG_LAUNCH(k_cg_rz<T>, g.nschunks, DBV / Vec16<T>::W, 0, s, g, w.r, w.z, A.dmask, a.ks, rb.partials, rb.counter, c, 0);
   };
   return run_loop(cc, st, cond, a.ks, a.ks_host, g.ninst, a.max_iter, 1, 4, [&](cudaStream_t s, const Cond& c) {
     iter(s, c, w.pa, w.pb);

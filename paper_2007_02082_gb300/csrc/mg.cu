@@ -149,6 +149,31 @@ __global__ void __launch_bounds__(512) k_mg_c_smooth(DevGrid g, const T* __restr
   }
 }
 
+// The same at interface nodes after the fused sweep (fe_poisson_smooth): K z is the
+// sum of both copies' parts and half of each hanging child's, as k_sync forms it.
+template <typename T>
+__global__ void k_mg_if_smooth(DevGrid g, const T* __restrict__ zin, T* __restrict__ zout, const T* __restrict__ r,
+                               const T* __restrict__ q, const T* __restrict__ dinv, uint16_t dmask,
+                               const uint8_t* __restrict__ on, T omega, const KState* ks) {
+  KCOUNT();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= g.n_if) return;
+  const int32_t s[2] = {g.if_c[e], g.if_f[e]};
+  const int32_t k0 = g.if_off[e], k1 = g.if_off[e + 1];
+  const int inst = g.binst[s[0] / DBV];
+  const uint16_t m[2] = {g.meta[s[0]], g.meta[s[1]]};
+  T z[2], rv[2], d[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) z[j] = zin[s[j]], rv[j] = r[s[j]], d[j] = dinv[s[j]];
+  T tot = q[s[0]] + q[s[1]];
+  for (int k = k0; k < k1; ++k) tot += T(0.5) * q[g.if_kid[k]];
+  if (m[0] & dmask) tot = T(0);
+  if (ks[inst].done || !on[inst]) return;
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+    zout[s[j]] = keep_slot(m[j], dmask) ? T(z[j] + omega * d[j] * (rv[j] - tot)) : T(0);
+}
+
 // Composite <-> G0 transfers.  The weights are those of P1 interpolation on
 // the G0 Kuhn tetrahedron holding a composite node (multiples of 2^-l, exact
 // in floating point), computed per node from lattice positions instead of
@@ -741,7 +766,7 @@ inline unsigned nblk256(int64_t n) { return unsigned((n + 255) / 256); }
 
 template <typename T>
 void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T* q, const T* dinv, uint16_t dmask,
-               const KState* ks, cudaStream_t st, Prof* prof, int pcls) {
+               const KState* ks, cudaStream_t st, Prof* prof, int pcls, bool z_started) {
   const int nu = mg.nu;
   const T w = mg.omega;
   KState* ksm = const_cast<KState*>(ks);
@@ -756,21 +781,32 @@ void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T*
     timed(0, [&] { fe_poisson_apply<T>(g, x, q, dmask, ksm, mg.on, st); });
     fe_sync<T>(g, 1, q, dmask, st);
   };
-  auto smooth = [&](const T* zin, T* zout) {
-    timed(1, [&] {
-      IBG_LAUNCH(k_mg_c_smooth<T>, g.nschunks, DBV, 0, st, g, zin, zout, r, q, dinv, dmask, mg.on, w, ks);
-    });
+  // one sweep: the fused stencil and update, then its interface nodes; or (FP64, other
+  // launch choices) the apply with its sums, then the update
+  auto sweep = [&](const T* zin, T* zout) {
+    bool fused = false;
+    timed(0, [&] { fused = fe_poisson_smooth<T>(g, zin, zout, r, q, dinv, w, dmask, ksm, mg.on, st); });
+    if (fused) {
+      if (g.n_if)
+        IBG_LAUNCH(k_mg_if_smooth<T>, (g.n_if + 255) / 256, 256, 0, st, g, zin, zout, r, (const T*)q, dinv, dmask, mg.on,
+                   w, ks);
+    } else {
+      apply(zin);
+      timed(1, [&] {
+        IBG_LAUNCH(k_mg_c_smooth<T>, g.nschunks, DBV, 0, st, g, zin, zout, r, q, dinv, dmask, mg.on, w, ks);
+      });
+    }
+    fe_expand2<T>(g, 1, zout, (T*)nullptr, st);
   };
   // composite pre-smoothing
-  timed(2, [&] { IBG_LAUNCH(k_mg_c_jac0<T>, g.nschunks, DBV, 0, st, g, r, z, dinv, dmask, mg.on, w, ks); });
+  if (!z_started)
+    timed(2, [&] { IBG_LAUNCH(k_mg_c_jac0<T>, g.nschunks, DBV, 0, st, g, r, z, dinv, dmask, mg.on, w, ks); });
   fe_expand2<T>(g, 1, z, (T*)nullptr, st);
   if (!mg.any) return;
   T* cur = z;
   T* oth = zs;
   for (int s = 1; s < nu; ++s) {
-    apply(cur);
-    smooth(cur, oth);
-    fe_expand2<T>(g, 1, oth, (T*)nullptr, st);
+    sweep(cur, oth);
     T* tmp = cur; cur = oth; oth = tmp;
   }
   apply(cur);
@@ -835,9 +871,7 @@ void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T*
   fe_expand2<T>(g, 1, y, (T*)nullptr, st);
   T* o = (y == z) ? zs : z;
   for (int s = 0; s < nu; ++s) {
-    apply(y);
-    smooth(y, o);
-    fe_expand2<T>(g, 1, o, (T*)nullptr, st);
+    sweep(y, o);
     T* tmp = y; y = o; o = tmp;
   }
 }
@@ -861,8 +895,8 @@ template int mg_levels_ctas<float>();
 template int mg_levels_ctas<double>();
 
 template void mg_vcycle<float>(const DevGrid&, const MGDev<float>&, const float*, float*, float*, float*,
-                               const float*, uint16_t, const KState*, cudaStream_t, Prof*, int);
+                               const float*, uint16_t, const KState*, cudaStream_t, Prof*, int, bool);
 template void mg_vcycle<double>(const DevGrid&, const MGDev<double>&, const double*, double*, double*, double*,
-                                const double*, uint16_t, const KState*, cudaStream_t, Prof*, int);
+                                const double*, uint16_t, const KState*, cudaStream_t, Prof*, int, bool);
 
 }  // namespace ibg
