@@ -6,17 +6,18 @@
 // launches an iteration is two launches and two grid reductions, all latency
 // (15-25 us whatever the size).  Here a cluster of up to 16 CTAs (co-scheduled
 // by the hardware, so its barriers end) runs the whole loop of one problem: rows
-// in equal contiguous ranges, p of the rows around a CTA's own copied once an
-// iteration through distributed shared memory, S kept in shared memory as far
-// as it fits (16-bit columns into that window), partial sums stored straight
-// into every CTA, three hardware barriers an iteration (about 500 cycles each).
+// in equal contiguous ranges, p of the rows around a CTA's own formed in every CTA
+// that needs it from the owners' residuals (distributed shared memory), S
+// kept in shared memory as far as it fits (16-bit columns into that window), partial
+// sums stored straight into every CTA, two hardware barriers an iteration
+// (about 500 cycles each).
 // A problem's arithmetic depends on its own rows only, so it keeps its bits
 // alone and in any batch; problems of a batch run side by side.
-// Bound: latency of the barriers and FP64 scalars at a few hundred rows (5 us an
+// Bound: latency of the barriers and scalars at a few hundred rows (4.2 us an
 // iteration), shared-memory wavefronts of the product at some thousand dense rows
-// (8160 rows of 41 entries: 12 us), in FP64 the FP64 rate of 16 SMs (2000 rows: 14 us).
-// A step: 8x8x16 tube 22.0 -> 6.5 ms, 16x16x64 tube in FP64 22.6 -> 15.3 ms, dense
-// 32x32x128 tube 22.8 -> 12.0 ms (of which the reductions alone gave a third).
+// (8160 rows of 41 entries: 10 us), in FP64 the FP64 rate of 16 SMs (2000 rows: 11.5 us).
+// A step: 8x8x16 tube 21.6 -> 5.8 ms, 16x16x64 tube in FP64 31.6 -> 14.8 ms, dense
+// 32x32x128 tube 25.4 -> 12.0 ms (of which the reductions alone gave a third).
 #pragma once
 
 namespace ibg {
@@ -44,6 +45,15 @@ __device__ __forceinline__ void cluster_load3(uint32_t a, double (&v)[3]) {
   asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a));
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[2]) : "r"(a + 16));
 }
+__device__ __forceinline__ void cluster_load4(uint32_t a, float (&v)[4]) {
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "r"(a));
+}
+__device__ __forceinline__ void cluster_load4(uint32_t a, double (&v)[4]) {
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a));
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "r"(a + 16));
+}
 __device__ __forceinline__ void window_load3(const float* a, float (&v)[3]) {
   const float4 x = *reinterpret_cast<const float4*>(a);
   v[0] = x.x, v[1] = x.y, v[2] = x.z;
@@ -66,16 +76,35 @@ __device__ __forceinline__ void cluster_store(uint32_t a, double v) {
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
-// bytes of shared memory per row: p with 1/diag (four values), q, r and the row's first entry
+// a / b as T.  FP32: rounded from the quotient to about 2^-46, by one correction
+// of an FP32 division (an FP64 division is a chain of a dozen FP64
+// instructions, and every row waits for it), FP64 where FP32 could not hold
+// the operands.
+__device__ __forceinline__ float quotient(double a, double b, float) {
+  const unsigned ea = (unsigned(__double2hiint(a)) >> 20) & 0x7FFu, eb = (unsigned(__double2hiint(b)) >> 20) & 0x7FFu;
+  if (ea - 923u > 200u || eb - 923u > 200u) return float(a / b);   // outside 2^-100 .. 2^100
+  const float inv = __frcp_rn(float(b));
+  const float q = __fmul_rn(float(a), inv);
+  return fmaf(float(fma(-double(q), b, a)), inv, q);
+}
+__device__ __forceinline__ double quotient(double a, double b, double) { return a / b; }
+// sum over the first `width` lanes (a power of two), valid in lane 0
+__device__ __forceinline__ double lanes_sum(double x, int width) {
+  for (int o = width >> 1; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// bytes of shared memory per row: p (four values), r with 1/diag, q and the row's first entry
 template <typename T>
-__host__ __device__ constexpr int afc_row_bytes() { return 10 * int(sizeof(T)) + 4; }
+__host__ __device__ constexpr int afc_row_bytes() { return 11 * int(sizeof(T)) + 4; }
 // Padded rows of a problem that runs in clusters of cl CTAs.  FP32: up to where
-// the loop's launches cost the same (32,000 rows of 10 entries: 15.7 us an
-// iteration here, about 16 in the loop; 8160 rows of 41: 11.8 against 22).
+// the loop's launches cost the same (32,000 rows of 10 entries: 14 us an
+// iteration here, about 16 in the loop; 8160 rows of 41: 10 against 22).
 // FP64: while the FP64 rate of 16 SMs costs less than the loop's launches
-// (2000 rows of 40 entries 14 us against 25; 32,000 rows of 10 measured 80 against 50).
+// (2000 rows of 40 entries 11.5 us against 25; 32,000 rows of 10 measured 80 against 50).
 template <typename T>
 __host__ __device__ constexpr int64_t afc_max_rows(int cl) { return int64_t(cl) * (sizeof(T) == 4 ? 2048 : 384); }
+static_assert(AFC_UNITS == 128, "16 blocks of 256 rows at most");
 static_assert(2048 <= AFC_THREADS * AFC_RPT, "x of a CTA's rows is kept in registers");
 template <typename T>
 __host__ __device__ constexpr bool afc_fits(int64_t n, int cl) { return cl > 0 && n <= afc_max_rows<T>(cl); }
@@ -93,7 +122,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   __shared__ T red[6][AFC_THREADS / 32 * AFC_RPT];
   __shared__ T sal[3], sbe[3];
   __shared__ KState sk[3];
-  __shared__ int win, goff[AFC_MAX];
+  __shared__ int win, goff[AFC_MAX];       // goff: where every CTA's own rows start in its window, -1: no window
   uint32_t rank, cl;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cl));
@@ -112,7 +141,9 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   const int rpc = max(0, min(n - int(rank) * rper, rper));   // rows of this CTA
   const int64_t row0 = R0 + int64_t(rank) * rper;
   const int e0 = rpc ? ib.rowptr[row0] : 0, ne = rpc ? ib.rowptr[row0 + rpc] - e0 : 0;
-  constexpr int lpr = AFL / 2;             // threads per row of the product
+  // threads per row of the product: four with two chains each in FP32; two in
+  // FP64, whose rate pays for every idle lane of a row's last round
+  constexpr int lpr = sizeof(T) == 8 ? 2 : AFL / 2;
   // no more warps than the rows need: the others leave (the barriers count
   // the threads that are left)
   const int nt = min(AFC_THREADS, max(256, AFL * rper));
@@ -134,27 +165,27 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   __syncthreads();
   const int own0 = min(int(rank) * rper, n);   // the problem's row of the CTA's first one
   const int ubytes = units ? 12 * (n / 32) * int(sizeof(T)) : 0;
-  const int room = AFC_SMEM - 64 - ubytes - rpc * afc_row_bytes<T>();
+  const int room = AFC_SMEM - 64 - ubytes - rper * afc_row_bytes<T>();
   const bool fast = win <= room / int(16 * sizeof(T));   // the window takes half the room at most
   const int G = fast ? win : 0;
   const int w0 = max(0, own0 - G), wn = min(n, own0 + rpc + G) - w0;   // window: rows [w0, w0 + wn) of the problem
   // in place of part: the sums of every 32 rows of the problem, [2][6][n / 32]
   T* unit = reinterpret_cast<T*>(afc_sm);
-  T* pw = reinterpret_cast<T*>(afc_sm + ubytes);   // [wn][4]: p; the own rows' fourth value is 1/diag
+  T* r = reinterpret_cast<T*>(afc_sm + ubytes);   // [rper][4]: r and 1/diag, at the same place in every CTA
+  T* pw = r + 4 * rper;                    // [wn][4]: p
   T* p = pw + 4 * (own0 - w0);
   T* q = pw + 4 * wn;                      // [rpc][3]
-  T* r = q + 3 * rpc;                      // [rpc][3]
-  T* cv = r + 3 * rpc;                     // cached values of S ...
+  T* cv = q + 3 * rpc;                     // cached values of S ...
   const int cap = fast ? min(ne, (room - (wn - rpc) * int(4 * sizeof(T))) / int(sizeof(T) + 2)) / 2 * 2 : 0;
   uint16_t* cc = reinterpret_cast<uint16_t*>(cv + cap);   // ... and their columns' places in the window
   int* rp = reinterpret_cast<int*>(cc + cap);             // [rpc + 1] entries relative to e0
-  // where every CTA's own rows start in its window (once every CTA runs)
-  cluster_barrier();
-  if (t < int(cl)) cluster_store(cluster_addr(smem_u32(&goff[rank]), uint32_t(t)), own0 - w0);
-  const uint32_t pbase = smem_u32(pw);
-  auto owner = [&](int k) -> uint32_t {    // cluster address of p at row k of the problem
+  cluster_barrier();                       // every CTA runs
+  if (t < int(cl)) cluster_store(cluster_addr(smem_u32(&goff[rank]), uint32_t(t)), fast ? own0 - w0 : -1);
+  const uint32_t rbase = smem_u32(r), pbase = smem_u32(pw);
+  // cluster address of r at row k of the problem
+  auto owner = [&](int k) -> uint32_t {
     const int o = k / rper;
-    return cluster_addr(pbase + uint32_t(goff[o] + k - o * rper) * uint32_t(4 * sizeof(T)), uint32_t(o));
+    return cluster_addr(rbase + uint32_t(k - o * rper) * uint32_t(4 * sizeof(T)), uint32_t(o));
   };
   for (int e = t; e < cap; e += nt) {
     cv[e] = val[e0 + e];
@@ -163,19 +194,24 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   if (rpc)
     for (int i = t; i <= rpc; i += nt) rp[i] = ib.rowptr[row0 + i] - e0;
   for (int i = t; i < rpc; i += nt) {
-    p[4 * i + 3] = dinv[row0 + i];
+    r[4 * i + 3] = dinv[row0 + i];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      r[3 * i + c] = r0[3 * (row0 + i) + c];
-      p[4 * i + c] = T(0);
-    }
+    for (int c = 0; c < 3; ++c) r[4 * i + c] = r0[3 * (row0 + i) + c];
   }
+  for (int i = t; i < 4 * wn; i += nt) pw[i] = T(0);
   if (t < 3) {
     sk[t] = ks[3 * inst + t];
     sbe[t] = T(0);
   }
   __syncwarp();
   cluster_barrier();
+  bool all_fast = true;
+  for (int o = 0; o < int(cl); ++o) all_fast = all_fast && goff[o] >= 0;
+  // p at row k of the problem, from its owner
+  auto column3 = [&](int k, T (&v)[3]) {
+    const int o = k / rper, at = max(goff[o], 0) + k - o * rper;
+    cluster_load3(cluster_addr(pbase + uint32_t(at) * uint32_t(4 * sizeof(T)), uint32_t(o)), v);
+  };
   auto wrow = [&](int i) { return i < own0 - w0 ? i : i + rpc; };   // window row of the i-th row of others
   const uint32_t ghost0 = t < wn - rpc ? owner(w0 + wrow(t)) : 0u;
   // The sums over rows carry the bits of the loop's kernels in FP32, where an
@@ -183,7 +219,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   // hang on them: FP32 within the blocks of rows that those kernels sum, in
   // their order (p.q: 32 rows, four to a warp, then eight warps; r.z and r.r:
   // 256 rows, 32 to a warp, then eight warps), FP64 beyond.
-  auto unit_sums = [&](auto& v, auto nv, int u) {   // a warp's 32 rows -> red[k][u], in one butterfly (warp_sums)
+  auto unit_sums = [&](auto& v, auto nv, int u, int buf) {   // a warp's 32 rows, in one butterfly (warp_sums)
     constexpr int NV = decltype(nv)::value, P = NV == 3 ? 4 : 8, PB = NV == 3 ? 2 : 3;
     constexpr int off[5] = {NV == 3 ? 2 : 16, NV == 3 ? 1 : 8, NV == 3 ? 16 : 4, NV == 3 ? 8 : 2, NV == 3 ? 4 : 1};
     T a[P];
@@ -201,38 +237,43 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
         a[j] = keep + __shfl_xor_sync(0xffffffffu, send, off[b]);
       }
     }
-    int rest = 0;
 #pragma unroll
-    for (int b = PB; b < 5; ++b) {
-      a[0] += __shfl_xor_sync(0xffffffffu, a[0], off[b]);
-      rest |= off[b];
+    for (int b = PB; b < 5; ++b) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off[b]);
+    // value k is in every lane with k's bits: lane o of those stores it to CTA o, ...
+    int place = 0;   // the lane's number among the holders of its value
+#pragma unroll
+    for (int b = PB; b < 5; ++b) place = 2 * place + ((lane & off[b]) != 0);
+    if (k < NV) {
+      if (units) {
+        for (int o = place; o < int(cl); o += 32 / P)
+          cluster_store(cluster_addr(smem_u32(&unit[(6 * buf + k) * (n / 32) + own0 / 32 + u]), uint32_t(o)), a[0]);
+      } else if (place == 0) {
+        red[k][u] = a[0];
+      }
     }
-    if ((lane & rest) == 0 && k < NV) red[k][u] = a[0];
   };
   // eight warps' sums of a block of 256 rows
   auto block256 = [](const T* u) {
     return ((u[0] + u[4]) + (u[2] + u[6])) + ((u[1] + u[5]) + (u[3] + u[7]));
   };
   const int nu = rpc / 32;                 // units of this CTA
-  const int clsh = cl == 16 ? 4 : 3;       // clusters of 16 or 8
-  // the CTA's sums to every CTA of the cluster
+  // the CTA's sums to every CTA of the cluster (units: each warp has sent its own)
   auto exchange = [&](auto nv, int buf) {
     constexpr int NV = decltype(nv)::value;
-    __syncthreads();
-    if (units) {
-      for (int i = t; i < NV * nu * int(cl); i += nt) {
-        const int o = i & (int(cl) - 1), j = i >> clsh, k = j % NV, u = j / NV;
-        cluster_store(cluster_addr(smem_u32(&unit[(6 * buf + k) * (n / 32) + own0 / 32 + u]), uint32_t(o)), red[k][u]);
+    if (!units) {
+      __syncthreads();
+      if (w < NV) {
+        double s = 0.0;
+        if constexpr (NV == 3 || sizeof(T) == 8) {
+          for (int u = lane; u < nu; u += 32) s += double(red[w][u]);
+          s = lanes_sum(s, nu > 16 ? 32 : 16);
+        } else {
+          for (int u = lane; u < nu / 8; u += 32) s += double(block256(&red[w][8 * u]));
+          s = lanes_sum(s, 8);
+        }
+        s = __shfl_sync(0xffffffffu, s, 0);
+        if (lane < int(cl)) cluster_store(cluster_addr(smem_u32(&part[buf][rank][w]), uint32_t(lane)), s);
       }
-    } else if (w < NV) {
-      double s = 0.0;
-      if constexpr (NV == 3 || sizeof(T) == 8) {
-        for (int u = lane; u < nu; u += 32) s += double(red[w][u]);
-      } else {
-        for (int u = lane; u < nu / 8; u += 32) s += double(block256(&red[w][8 * u]));
-      }
-      s = __shfl_sync(0xffffffffu, lane_sum(s), 0);
-      if (lane < int(cl)) cluster_store(cluster_addr(smem_u32(&part[buf][rank][w]), uint32_t(lane)), s);
     }
     __syncwarp();
     cluster_barrier();
@@ -243,12 +284,15 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     double s = 0.0;
     if (!units) {
       s = lane < int(cl) ? part[buf][lane][k] : 0.0;
-    } else if constexpr (NV == 3) {
-      for (int u = lane; u < n / 32; u += 32) s += double(unit[(6 * buf + k) * (n / 32) + u]);
-    } else {
-      for (int u = lane; u < n / 256; u += 32) s += double(block256(&unit[(6 * buf + k) * (n / 32) + 8 * u]));
+      return lanes_sum(s, int(cl));
     }
-    return lane_sum(s);
+    if constexpr (NV == 3) {
+      for (int u = lane; u < n / 32; u += 32) s += double(unit[(6 * buf + k) * (n / 32) + u]);
+      return lanes_sum(s, n > 512 ? 32 : 16);
+    } else {
+      if (lane < n / 256) s = double(block256(&unit[(6 * buf + k) * (n / 32) + 8 * lane]));
+      return lanes_sum(s, 16);
+    }
   };
   T xr[AFC_RPT][3];                        // this thread's rows of x
 #pragma unroll
@@ -257,46 +301,64 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     for (int c = 0; c < 3; ++c) xr[j][c] = t + j * nt < rpc ? x[3 * (row0 + t + j * nt) + c] : T(0);
   bool live = true;
   while (live) {
-    // p = z + beta p, z = D^-1 r
+    // p = z + beta p, z = D^-1 r.  Every CTA forms p of its whole window, the
+    // others' rows from their r: the same values as their owners', without a
+    // barrier in between.
     {
       const T b[3] = {sbe[0], sbe[1], sbe[2]};
-      for (int i = t; i < rpc; i += nt) {
-        const T d = p[4 * i + 3];
+      auto direct = [&](int j, const T (&v)[4]) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) p[4 * i + c] = fma(b[c], p[4 * i + c], mul_rn(r[3 * i + c], d));
+        for (int c = 0; c < 3; ++c) pw[4 * j + c] = fma(b[c], pw[4 * j + c], mul_rn(v[c], v[3]));
+      };
+      T gh[4] = {T(0), T(0), T(0), T(0)};
+      if (t < wn - rpc) cluster_load4(ghost0, gh);
+      for (int i = t; i < rpc; i += nt) {
+        T v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = r[4 * i + c];
+        direct(own0 - w0 + i, v);
+      }
+      for (int i = t; i < wn - rpc; i += nt) {
+        const int j = wrow(i);
+        if (i != t) cluster_load4(owner(w0 + j), gh);
+        direct(j, gh);
       }
     }
-    __syncwarp();
-    cluster_barrier();
-    // the others' rows of the window
-    for (int i = t; i < wn - rpc; i += nt) {
-      const int j = wrow(i);
-      T v[3];
-      cluster_load3(i == t ? ghost0 : owner(w0 + j), v);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) pw[4 * j + c] = v[c];
+    if (all_fast) {
+      __syncthreads();
+    } else {
+      __syncwarp();
+      cluster_barrier();
     }
-    __syncthreads();
     // q = S p
     const int lr = t & (lpr - 1);
     for (int i = t / lpr; i < rpc; i += nt / lpr) {
-      // a thread takes the entries of lanes lr and lr + 4 of the loop's eight
       T acc[2][3] = {{T(0), T(0), T(0)}, {T(0), T(0), T(0)}};
       auto add = [&](T (&s)[3], T a, const T (&v)[3]) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) s[c] = fma(a, v[c], s[c]);
       };
       const int f1 = rp[i + 1], fc = min(f1, cap);
-      int f = rp[i] + lr;
+      int f = rp[i] + lr, h = 0;
+      if constexpr (sizeof(T) == 8) {
+#pragma unroll 4
+        for (; f < fc; f += lpr) {
+          T v[3];
+          window_load3(pw + 4 * cc[f], v);
+          add(acc[0], cv[f], v);
+        }
+      } else {
+        // a thread takes the entries of lanes lr and lr + 4 of the loop's eight
 #pragma unroll 2
-      for (; f + 4 < fc; f += AFL) {
-        T v[3], u[3];
-        window_load3(pw + 4 * cc[f], v);
-        window_load3(pw + 4 * cc[f + 4], u);
-        add(acc[0], cv[f], v);
-        add(acc[1], cv[f + 4], u);
+        for (; f + 4 < fc; f += AFL) {
+          T v[3], u[3];
+          window_load3(pw + 4 * cc[f], v);
+          window_load3(pw + 4 * cc[f + 4], u);
+          add(acc[0], cv[f], v);
+          add(acc[1], cv[f + 4], u);
+        }
       }
-      for (int h = 0; f < f1; f += 4, h ^= 1) {   // the last one, and entries that did not fit
+      for (; f < f1; f += lpr, h ^= 1) {   // the last one, and entries that did not fit
         T v[3], a;
         if (f < fc) {
           a = cv[f];
@@ -304,27 +366,32 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
         } else {
           const int k = int(ib.col[e0 + f] - R0);
           a = val[e0 + f];
-          if (fast) window_load3(pw + 4 * (k - w0), v);
-          else cluster_load3(owner(k), v);
+          if (unsigned(k - w0) < unsigned(wn)) window_load3(pw + 4 * (k - w0), v);
+          else column3(k, v);
         }
-        if (h) add(acc[1], a, v);
+        if (h && sizeof(T) == 4) add(acc[1], a, v);
         else add(acc[0], a, v);
       }
       // the three sums over the row's lanes (whole warps get here together: a CTA's
       // rows are a multiple of 32), two of them in one butterfly step
+      constexpr int hb = lpr / 2;
+      const bool up = (lr & hb) != 0;
       T s0, s1;
       {
-        const T a0 = acc[0][0] + acc[1][0], a1 = acc[0][1] + acc[1][1], a2 = acc[0][2] + acc[1][2];
-        const bool up = (lr & 2) != 0;
-        s0 = (up ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up ? a0 : a1, 2);
-        s1 = a2 + __shfl_xor_sync(0xffffffffu, a2, 2);
-        s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+        const T a0 = sizeof(T) == 8 ? acc[0][0] : acc[0][0] + acc[1][0],
+                a1 = sizeof(T) == 8 ? acc[0][1] : acc[0][1] + acc[1][1],
+                a2 = sizeof(T) == 8 ? acc[0][2] : acc[0][2] + acc[1][2];
+        s0 = (up ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up ? a0 : a1, hb);
+        s1 = a2 + __shfl_xor_sync(0xffffffffu, a2, hb);
+        if constexpr (lpr == 4) {
+          s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+          s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+        }
       }
       if (lr == 0) {
         q[3 * i] = s0;
         q[3 * i + 2] = s1;
-      } else if (lr == 2) {
+      } else if (lr == hb) {
         q[3 * i + 1] = s0;
       }
     }
@@ -333,7 +400,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
       T v[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) v[c] = mul_rn(p[4 * i + c], q[3 * i + c]);
-      unit_sums(v, three{}, i / 32);
+      unit_sums(v, three{}, i / 32, 0);
     }
     exchange(three{}, 0);
     if (w < 3) {
@@ -342,16 +409,15 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
         KState& k = sk[w];
         if (!k.done) {
           k.pq = pq;
+          T al = T(0);
           if (!(pq > 0.0) || !isfinite(pq)) {
             k.done = 1;
             k.status = 5;
-            k.alpha = 0.0;
           } else {
-            k.alpha = k.rz / pq;
+            al = quotient(k.rz, pq, T(0));
           }
-          k.af = float(k.alpha);
+          sal[w] = al;
         }
-        sal[w] = k_alpha<T>(k);
       }
     }
     __syncthreads();
@@ -359,7 +425,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     for (int j = 0; j < AFC_RPT; ++j) {
       const int i = t + j * nt;
       if (i >= rpc) break;                 // whole warps: a CTA's rows are a multiple of 32
-      const T d = p[4 * i + 3];
+      const T d = r[4 * i + 3];
       T v[6];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -367,18 +433,19 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
         if (sk[c].done) continue;
         const T a = sal[c];
         xr[j][c] = fma(a, p[4 * i + c], xr[j][c]);
-        const T rv = fma(-a, q[3 * i + c], r[3 * i + c]);
-        r[3 * i + c] = rv;
+        const T rv = fma(-a, q[3 * i + c], r[4 * i + c]);
+        r[4 * i + c] = rv;
         v[2 * c] = mul_rn(rv, mul_rn(rv, d));
         v[2 * c + 1] = mul_rn(rv, rv);
       }
-      unit_sums(v, six{}, i / 32);
+      unit_sums(v, six{}, i / 32, 1);
     }
     exchange(six{}, 1);
     if (w < 3) {
       const double rzn = total(six{}, 1, 2 * w), rr = total(six{}, 1, 2 * w + 1);
       KState& k = sk[w];
       if (lane == 0) {
+        T be = T(0);
         if (!k.done) {
           k.iter++;
           k.rr = rr;
@@ -386,12 +453,11 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
           else if (rr <= k.tol2 * k.bb) k.done = 1;
           else if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; }
           else {
-            k.beta = rzn / k.rz;
-            k.bf = float(k.beta);
+            be = quotient(rzn, k.rz, T(0));
             k.rz = rzn;
           }
         }
-        sbe[w] = k.done ? T(0) : k_beta<T>(k);
+        sbe[w] = be;
       }
     }
     __syncthreads();

@@ -34,11 +34,20 @@ def _residual(g, case):
     return float(np.max(np.linalg.norm(B - y, axis=0) / np.where(nb > 0, nb, 1.0)))
 
 
+def _shuffled():
+    """Points in random order: no CTA's columns fit a window of neighbouring rows."""
+    c = W.cylinder_refined_64x64x256(n=(48, 48, 192), M=18000)
+    k = np.random.default_rng(5).permutation(len(c["X"]))
+    c["X"], c["dS"], c["UB"] = (np.ascontiguousarray(c[f][k]) for f in ("X", "dS", "UB"))
+    return c
+
+
 CASES = {
     "one_block": lambda: W.cylinder_case(n=(8, 8, 16), length=2.0, M=30, seed=71, nu=0.1, dt=0.01),
     "two_blocks": lambda: W.cylinder_case(n=(8, 8, 16), length=2.0, M=270, seed=72, nu=0.1, dt=0.01),
     "dense": lambda: W.cylinder_uniform_16x16x64(),
     "uncached": lambda: W.cylinder_refined_64x64x256(),
+    "shuffled": _shuffled,
 }
 
 
