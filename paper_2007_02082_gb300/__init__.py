@@ -186,6 +186,7 @@ class IBGrid:
 
     def ib_set_boundary(self, X, dS, UB, inside):
         self._keep = (X, dS, UB, inside)
+        self._sizes = None
         s = self.lib.ib_set_boundary(self.h, int(X.shape[0]), X.ctypes.data, dS.ctypes.data,
                                      UB.ctypes.data if UB is not None else None,
                                      inside.ctypes.data if inside is not None else None)
@@ -199,9 +200,16 @@ class IBGrid:
         self._check("ib_grid_info", self.lib.ib_grid_info(self.h, C.byref(info)))
         return info.as_dict()
 
+    _sizes = None   # (nodes, points) since the last ib_set_boundary, which alone changes them
+
+    def _nodes_points(self):
+        if self._sizes is None:
+            info = self.ib_grid_info()
+            self._sizes = info["n_nodes"], info["n_points"]
+        return self._sizes
+
     def _shape(self, field):
-        info = self.ib_grid_info()
-        N, M = info["n_nodes"], info["n_points"]
+        N, M = self._nodes_points()
         n = self.case["n"]
         return {
             "U": ((N, 3), np.float64), "U_TENT": ((N, 3), np.float64), "U_IB": ((N, 3), np.float64),
@@ -281,7 +289,7 @@ class IBGrid:
         """Wall shear stress at the Lagrangian points (Sec. 2.6) from the
         current velocity; normals (M, 3) unit outward.  Returns wss (M,) and,
         with with_grad, the velocity gradient (M, 3, 3), [p, i, j] = d u_i / d x_j."""
-        M = self.ib_grid_info()["n_points"]
+        M = self._nodes_points()[1]
         n = np.ascontiguousarray(normals, dtype=np.float64).reshape(M, 3)
         w = np.empty(M)
         g = np.empty((M, 3, 3)) if with_grad else None

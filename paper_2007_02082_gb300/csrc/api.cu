@@ -1242,10 +1242,7 @@ void fill_info(const HostGrid& H, const MGHost* mg, const Engine* E, int64_t dev
   for (double v : H.dS) mdS += v;
   mdS = H.M ? mdS / double(H.M) : 0.0;
   for (int a = 0; a < 3; ++a) I.a_ratio[a] = std::sqrt(mdS) / H.hf[a];
-  int64_t nv = 0;
-  for (uint16_t m : H.meta)
-    if (m & M_VALID) nv++;
-  I.n_valid_slots = nv;
+  I.n_valid_slots = H.n_valid;   // counted once at set-up: the metadata are 2 bytes a slot
   I.device_bytes = dev_bytes;
   I.kernel_launches = int64_t(fe_kcount() + krylov_kcount() + ib_kcount() + mg_kcount() + move_kcount() + wss_kcount());
   if (E) {
@@ -1373,6 +1370,8 @@ ib_status ib_set_boundary(ib_grid* g, int64_t M, const double* X, const double* 
   g->ready = false;
   ib_status s = build_host_grid(g->d, M, X, dS, UB, inside, g->H, g->err);
   if (s != IB_OK) return s;
+  g->H.n_valid = 0;
+  for (uint16_t m : g->H.meta) g->H.n_valid += (m & M_VALID) ? 1 : 0;
   g->mg = MGHost();
   if (g->d.poisson_pc == IB_PC_MULTIGRID)
     build_mg(g->H, g->mg, g->d.tune[IB_TUNE_MG_SMALL] > 0 ? g->d.tune[IB_TUNE_MG_SMALL] : MG_SMALL_NODES);

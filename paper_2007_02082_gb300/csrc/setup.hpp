@@ -76,6 +76,7 @@ struct HostGrid {
   std::vector<int32_t> canon_q;       // [N][3] finest coordinates
   std::vector<uint8_t> canon_flags;   // [N]
   int64_t n_dof = 0;
+  int64_t n_valid = 0;              // stored node copies, all levels (valid slots)
   // inlet Dirichlet entries (every stored copy)
   std::vector<int32_t> inlet_slot;
   std::vector<int32_t> inlet_port;
