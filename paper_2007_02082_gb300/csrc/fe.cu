@@ -35,6 +35,15 @@ std::atomic<long long> g_launches{0};
 __constant__ int8_t c_sten[15][3];
 __constant__ int16_t c_toff[15];               // tile offset of each stencil slot
 __constant__ int8_t c_slot_of_rel[27];
+// Weights of every incident-cell mask for bodies with a run-time mask; the lanes
+// of a warp hold few different masks, so the rows stay in L1.
+// Transpose couplings, row [mask][k], byte 3 i + j (signed), for the FP64 momentum
+// operator of the symmetric form (33x33x131 tube: 288 -> 259 us; in FP32 the loads
+// cost more than forming the weights, 43 against 35 us)
+__device__ uint4 g_transw[256 * 15];
+// mass, off-diagonal weights 4 bits each (neighbour k at 4 (k - 1)), half the
+// diagonal weight in the top byte, for the FP32 operator (16 M-node sac: 238 -> 229 us)
+__device__ unsigned long long g_massw[256];
 
 static const int8_t h_sten[15][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
                                      {0, 0, 1},  {0, 0, -1}, {1, 1, 0},  {-1, -1, 0}, {0, 1, 1},
@@ -52,6 +61,20 @@ cudaError_t fe_init_tables() {
   if ((e = cudaMemcpyToSymbol(c_sten, h_sten, sizeof(h_sten))) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_toff, toff, sizeof(toff))) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_slot_of_rel, slot_of_rel, sizeof(slot_of_rel))) != cudaSuccess) return e;
+  std::vector<uint4> tw(256 * 15);
+  unsigned long long mw[256];
+  for (int mk = 0; mk < 256; ++mk) {
+    for (int k = 0; k < 15; ++k) {
+      int8_t b[16] = {};
+      for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) b[3 * i + j] = int8_t(trans_weight(mk, k, i, j));
+      std::memcpy(&tw[mk * 15 + k], b, 16);
+    }
+    mw[mk] = (unsigned long long)(mass_weight(mk, 0) / 2) << 56;
+    for (int k = 1; k < 15; ++k) mw[mk] |= (unsigned long long)mass_weight(mk, k) << (4 * k - 4);
+  }
+  if ((e = cudaMemcpyToSymbol(g_transw, tw.data(), tw.size() * sizeof(uint4))) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(g_massw, mw, sizeof(mw))) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
@@ -106,6 +129,12 @@ __device__ __forceinline__ constexpr bool const_mask() {
 // x_j(neighbour k), the transpose-gradient couplings (grad u^T, grad v) per
 // Kuhn tetrahedron (kuhn_weights.hpp), F_ij = (V/6)/(h_i h_j) from the
 // stencil factors.  xk(k, v) loads the three components at neighbour k.
+// (Couplings that are zero for every mask, 36 of 135, are left out of the run-time
+// body too: FP64 333 -> 288 us on the 33x33x131 tube.)
+__host__ __device__ constexpr bool trans_couples(int k, int i, int j) {   // some mask gives (k, i, j) a weight
+  constexpr int t[15] = {0x1ff, 0x0ef, 0x0ef, 0x0fe, 0x0fe, 0x1ee, 0x1ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee};
+  return (t[k] >> (3 * i + j)) & 1;
+}
 template <typename T, typename MK, typename XK>
 __device__ __forceinline__ void add_transpose(MK mk, const T* F, T dtnu, XK&& xk, T (&out)[3]) {
   T acc[3][3];
@@ -117,12 +146,26 @@ __device__ __forceinline__ void add_transpose(MK mk, const T* F, T dtnu, XK&& xk
   for (int k = 0; k < 15; ++k) {
     T v[3];
     xk(k, v);
+    uint4 row = make_uint4(0u, 0u, 0u, 0u);
+    if constexpr (!const_mask<MK>() && sizeof(T) == 8) row = g_transw[15 * int(mk) + k];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        const int w = trans_weight(mk, k, i, j);
-        if (!const_mask<MK>() || w != 0) acc[i][j] += wconv<T>(w) * v[j];
+        if constexpr (const_mask<MK>()) {
+          const int w = trans_weight(mk, k, i, j);
+          if (w != 0) acc[i][j] += wconv<T>(w) * v[j];
+        } else if (trans_couples(k, i, j)) {
+          int w;
+          if constexpr (sizeof(T) == 8) {
+            const int e = 3 * i + j;
+            const unsigned word = e < 4 ? row.x : e < 8 ? row.y : row.z;
+            w = int((word >> (8 * (e & 3)) & 0xFFu) ^ 0x80u) - 128;
+          } else {
+            w = trans_weight(mk, k, i, j);
+          }
+          acc[i][j] += wconv<T>(w) * v[j];
+        }
       }
   }
   const T fij[3][3] = {{F[0], F[8], F[10]}, {F[8], F[1], F[9]}, {F[10], F[9], F[2]}};
@@ -1066,7 +1109,7 @@ __global__ void __launch_bounds__(P7_THREADS, SMOOTH ? 6 : 8)
     k_poisson7_staged(DevGrid g, const float* __restrict__ z, const float* __restrict__ pold,
                       float* __restrict__ pnew, float* __restrict__ q, uint16_t dmask, KState* __restrict__ ks,
                       double* __restrict__ partials, unsigned* __restrict__ counter, const uint8_t* __restrict__ on,
-                      const float* __restrict__ dinv = nullptr, float omega = 0.f) {
+                      const float* __restrict__ dinv, float omega, int split) {
   KCOUNT();
   constexpr int NV = CG ? 2 : 1;
   constexpr int NX = SMOOTH ? 2 : 0;
@@ -1079,7 +1122,11 @@ __global__ void __launch_bounds__(P7_THREADS, SMOOTH ? 6 : 8)
   __shared__ float fac[3 * P7_CHUNK];   // stencil factors (V/6)/h_a^2 of each brick
   __shared__ uint32_t ecnt[256];        // per mask: edge counts, 4 bits each, (+x, -x, +y, -y, +z, -z)
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p7_dyn) + 127) & ~uintptr_t(127));
-  const int b0 = g.cbrick[blockIdx.x], b1 = g.cbrick[blockIdx.x + 1];
+  // the CTA's bricks: a chunk, or one of `split` parts of it (forms without sums)
+  const int ch = CG ? int(blockIdx.x) : int(blockIdx.x) / split, part = CG ? 0 : int(blockIdx.x) - ch * split;
+  const int c0 = g.cbrick[ch], c1 = g.cbrick[ch + 1], per = CG ? P7_CHUNK : P7_CHUNK / split;
+  const int b0 = c0 + part * per, b1 = min(c1, b0 + per);
+  if (b0 >= b1) return;
   const int inst = g.binst[b0];
   const bool done = ks ? ks[inst].done != 0 : false;
   float acc = 0.f;
@@ -1456,6 +1503,17 @@ int fe_p7_ctas_per_sm() {
   return std::min(a, b);
 }
 
+// Parts a chunk of eight bricks is cut into for the forms without sums: while
+// the chunks are fewer than two CTAs per SM a CTA's walk through its bricks is the
+// kernel's time (8x8x16 tube, 2 chunks: sweep 4.6 -> 2.4 us); beyond that the parts'
+// own start (tables, ring fill) costs more than the shorter walk gives
+// (312 chunks in four parts: 8.6 -> 9.9 us).
+static int p7_split(const DevGrid& g) {
+  int s = 1;
+  while (s < P7_CHUNK && int64_t(g.nchunks) * s * 2 <= 152 * 2) s *= 2;
+  return s;
+}
+
 // The staged kernels serve FP32 vectors on 16-byte boundaries (every vector of
 // the library; the bulk and 16-byte copies need it) over the chunks of at most
 // P7_CHUNK bricks (the persistent one also needs its schedule and at most
@@ -1474,8 +1532,9 @@ static bool launch_p7(const DevGrid& g, const T* z, const T* pold, T* pnew, T* q
                  dmask, ks, partials, counter, on);
       return true;
     }
-    IBG_LAUNCH((k_poisson7_staged<CG>), g.nchunks, P7_THREADS, p7_smem<CG ? 2 : 1>(), st, g, z, pold, pnew, q, dmask,
-               ks, partials, counter, on, (const float*)nullptr, 0.f);
+    const int split = CG ? 1 : p7_split(g);
+    IBG_LAUNCH((k_poisson7_staged<CG>), g.nchunks * split, P7_THREADS, p7_smem<CG ? 2 : 1>(), st, g, z, pold, pnew, q,
+               dmask, ks, partials, counter, on, (const float*)nullptr, 0.f, split);
     return true;
   }
 }
@@ -1615,9 +1674,16 @@ __global__ void __launch_bounds__(512, (sizeof(T) == 4 && OP == OP_MASS && !PB) 
         // M x = (V/120) sum_k w_k x_k with integer weights w_k
         with_mask(act ? (m & 0xFF) : 0, [&](auto mk) {
           if (!act) return;
+          unsigned long long mw = 0;
+          if constexpr (sizeof(T) == 4 && !const_mask<decltype(mk)>()) mw = g_massw[int(mk)];
 #pragma unroll
           for (int k = 0; k < 15; ++k) {
-            const T wk = wconv<T>(mass_weight(mk, k));
+            T wk;
+            if constexpr (sizeof(T) == 4 && !const_mask<decltype(mk)>())
+              wk = __uint_as_float(0x4B000000u | unsigned(k == 0 ? 2u * unsigned(mw >> 56)
+                                                                  : unsigned(mw >> (4 * k - 4)) & 15u)) - 8388608.f;
+            else
+              wk = wconv<T>(mass_weight(mk, k));
             if constexpr (V4) {
               const float4 v = tile4[ti + c_toff[k]];
               out[0] += wk * v.x;
@@ -1779,13 +1845,30 @@ __global__ void k_natural_bterm(DevGrid g, const T* __restrict__ x, T* __restric
   const int inst = g.binst[a / DBV];
   const T* w = sizeof(T) == 4 ? reinterpret_cast<const T*>(g.nat_w32) : reinterpret_cast<const T*>(g.nat_w64);
   T acc[3] = {T(0), T(0), T(0)};
-  for (int e = g.nat_off[r]; e < g.nat_off[r + 1]; ++e) {
-    const int ij = g.nat_comp[e];
-    const int i = ij / 3, j = ij - 3 * (ij / 3);
-    const T v = w[e] * x[(int64_t)j * g.nslots + g.nat_ent[e]];
-    if (i == 0) acc[0] += v;
-    else if (i == 1) acc[1] += v;
-    else acc[2] += v;
+  // a row's entries eight at a time: their indices, then their values, are in
+  // flight together; each component's sum runs in the order of the entries
+  // (11.2 -> 7.6 us on the 33x33x131 tube)
+  constexpr int U = 8;
+  const int e1 = g.nat_off[r + 1];
+  for (int e0 = g.nat_off[r]; e0 < e1; e0 += U) {
+    int ij[U];
+    T we[U], xe[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int e = min(e0 + k, e1 - 1);
+      ij[k] = g.nat_comp[e];
+      we[k] = w[e];
+      xe[k] = x[(int64_t)(ij[k] % 3) * g.nslots + g.nat_ent[e]];
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (e0 + k >= e1) break;
+      const int i = ij[k] / 3;
+      const T v = we[k] * xe[k];
+      if (i == 0) acc[0] += v;
+      else if (i == 1) acc[1] += v;
+      else acc[2] += v;
+    }
   }
   const T dtnu = T(g.pdt[inst] * g.pnu[inst]);
 #pragma unroll
@@ -1854,8 +1937,9 @@ bool fe_poisson_smooth(const DevGrid& g, const T* z, T* zout, const T* r, T* q, 
   if constexpr (sizeof(T) == 4) {
     auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     if (g.poisson_kernel > 1 || !a16(z) || !a16(zout) || !a16(r) || !a16(dinv)) return false;
-    IBG_LAUNCH((k_poisson7_staged<false, true>), g.nchunks, P7_THREADS, (p7_smem<1, 2>()), st, g, z, r, zout, q, dmask,
-               ks, (double*)nullptr, (unsigned*)nullptr, on, dinv, omega);
+    const int split = p7_split(g);
+    IBG_LAUNCH((k_poisson7_staged<false, true>), g.nchunks * split, P7_THREADS, (p7_smem<1, 2>()), st, g, z, r, zout, q,
+               dmask, ks, (double*)nullptr, (unsigned*)nullptr, on, dinv, omega, split);
     return true;
   } else {
     return false;
