@@ -13,10 +13,10 @@
 // (about 500 cycles each).
 // A problem's arithmetic depends on its own rows only, so it keeps its bits
 // alone and in any batch; problems of a batch run side by side.
-// Bound: latency of the barriers and scalars at a few hundred rows (4.2 us an
+// Bound: latency of the barriers and scalars at a few hundred rows (3.8 us an
 // iteration), shared-memory wavefronts of the product at some thousand dense rows
 // (8160 rows of 41 entries: 10 us), in FP64 the FP64 rate of 16 SMs (2000 rows: 11.5 us).
-// A step: 8x8x16 tube 21.6 -> 5.8 ms, 16x16x64 tube in FP64 31.6 -> 14.8 ms, dense
+// A step: 8x8x16 tube 21.6 -> 5.2 ms, 16x16x64 tube in FP64 31.6 -> 14.4 ms, dense
 // 32x32x128 tube 25.4 -> 12.0 ms (of which the reductions alone gave a third).
 #pragma once
 
@@ -176,9 +176,10 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   T* p = pw + 4 * (own0 - w0);
   T* q = pw + 4 * wn;                      // [rpc][3]
   T* cv = q + 3 * rpc;                     // cached values of S ...
-  const int cap = fast ? min(ne, (room - (wn - rpc) * int(4 * sizeof(T))) / int(sizeof(T) + 2)) / 2 * 2 : 0;
-  uint16_t* cc = reinterpret_cast<uint16_t*>(cv + cap);   // ... and their columns' places in the window
-  int* rp = reinterpret_cast<int*>(cc + cap);             // [rpc + 1] entries relative to e0
+  const int cap = fast ? min(ne, (room - (wn - rpc) * int(4 * sizeof(T))) / int(sizeof(T) + 2) / 2 * 2) : 0;
+  const int capr = (cap + 1) / 2 * 2;      // (an even number of 16-bit places)
+  uint16_t* cc = reinterpret_cast<uint16_t*>(cv + capr);   // ... and their columns' places in the window
+  int* rp = reinterpret_cast<int*>(cc + capr);             // [rpc + 1] entries relative to e0
   cluster_barrier();                       // every CTA runs
   if (t < int(cl)) cluster_store(cluster_addr(smem_u32(&goff[rank]), uint32_t(t)), fast ? own0 - w0 : -1);
   const uint32_t rbase = smem_u32(r), pbase = smem_u32(pw);
@@ -201,10 +202,13 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   for (int i = t; i < 4 * wn; i += nt) pw[i] = T(0);
   if (t < 3) {
     sk[t] = ks[3 * inst + t];
+    sk[t].tt = sk[t].tol2 * sk[t].bb;      // the square norm to reach
     sbe[t] = T(0);
   }
   __syncwarp();
   cluster_barrier();
+  // small problems in FP32: a thread for each of the loop's eight lanes of a row
+  const bool wide = sizeof(T) == 4 && nt >= AFL * rper && fast && cap == ne;
   bool all_fast = true;
   for (int o = 0; o < int(cl); ++o) all_fast = all_fast && goff[o] >= 0;
   // p at row k of the problem, from its owner
@@ -278,20 +282,28 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     __syncwarp();
     cluster_barrier();
   };
-  // value k summed over the cluster, by a warp (valid in lane 0)
+  // a value summed over the cluster by a warp: p.q with all lanes (valid in lane
+  // 0), r.z and r.r with half of them each (k by lane; valid in lanes 0 and 16)
   auto total = [&](auto nv, int buf, int k) -> double {
     constexpr int NV = decltype(nv)::value;
     double s = 0.0;
-    if (!units) {
+    if constexpr (NV == 3) {
+      if (units) {
+        for (int u = lane; u < n / 32; u += 32) s += double(unit[(6 * buf + k) * (n / 32) + u]);
+        return lanes_sum(s, n > 512 ? 32 : 16);
+      }
       s = lane < int(cl) ? part[buf][lane][k] : 0.0;
       return lanes_sum(s, int(cl));
-    }
-    if constexpr (NV == 3) {
-      for (int u = lane; u < n / 32; u += 32) s += double(unit[(6 * buf + k) * (n / 32) + u]);
-      return lanes_sum(s, n > 512 ? 32 : 16);
     } else {
-      if (lane < n / 256) s = double(block256(&unit[(6 * buf + k) * (n / 32) + 8 * lane]));
-      return lanes_sum(s, 16);
+      const int l = lane & 15;
+      if (units) {
+        if (l < n / 256) s = double(block256(&unit[(6 * buf + k) * (n / 32) + 8 * l]));
+      } else if (l < int(cl)) {
+        s = part[buf][l][k];
+      }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, 16);
+      return s;
     }
   };
   T xr[AFC_RPT][3];                        // this thread's rows of x
@@ -299,6 +311,10 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   for (int j = 0; j < AFC_RPT; ++j)
 #pragma unroll
     for (int c = 0; c < 3; ++c) xr[j][c] = t + j * nt < rpc ? x[3 * (row0 + t + j * nt) + c] : T(0);
+  // r of the first of this thread's rows of others; fetched while the scalars are formed
+  T gh[4] = {T(0), T(0), T(0), T(0)};
+  const bool ghosts = t < wn - rpc;
+  if (ghosts) cluster_load4(ghost0, gh);
   bool live = true;
   while (live) {
     // p = z + beta p, z = D^-1 r.  Every CTA forms p of its whole window, the
@@ -310,8 +326,6 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
 #pragma unroll
         for (int c = 0; c < 3; ++c) pw[4 * j + c] = fma(b[c], pw[4 * j + c], mul_rn(v[c], v[3]));
       };
-      T gh[4] = {T(0), T(0), T(0), T(0)};
-      if (t < wn - rpc) cluster_load4(ghost0, gh);
       for (int i = t; i < rpc; i += nt) {
         T v[4];
 #pragma unroll
@@ -331,8 +345,37 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
       cluster_barrier();
     }
     // q = S p
+    if (wide) {
+      const int i = t / AFL, l = t & (AFL - 1);
+      if (i < rpc) {                       // whole warps
+        T acc[3] = {T(0), T(0), T(0)};
+        const int f1 = rp[i + 1];
+#pragma unroll 4
+        for (int f = rp[i] + l; f < f1; f += AFL) {
+          T v[3];
+          window_load3(pw + 4 * cc[f], v);
+          const T a = cv[f];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) acc[c] = fma(a, v[c], acc[c]);
+        }
+        const bool up = (l & 4) != 0;
+        T s0 = (up ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[1], 4);
+        T s1 = acc[2] + __shfl_xor_sync(0xffffffffu, acc[2], 4);
+#pragma unroll
+        for (int o = 2; o > 0; o >>= 1) {
+          s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        }
+        if (l == 0) {
+          q[3 * i] = s0;
+          q[3 * i + 2] = s1;
+        } else if (l == 4) {
+          q[3 * i + 1] = s0;
+        }
+      }
+    }
     const int lr = t & (lpr - 1);
-    for (int i = t / lpr; i < rpc; i += nt / lpr) {
+    for (int i = wide ? rpc : t / lpr; i < rpc; i += nt / lpr) {
       T acc[2][3] = {{T(0), T(0), T(0)}, {T(0), T(0), T(0)}};
       auto add = [&](T (&s)[3], T a, const T (&v)[3]) {
 #pragma unroll
@@ -441,8 +484,11 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
       unit_sums(v, six{}, i / 32, 1);
     }
     exchange(six{}, 1);
+    if (ghosts) cluster_load4(ghost0, gh);
     if (w < 3) {
-      const double rzn = total(six{}, 1, 2 * w), rr = total(six{}, 1, 2 * w + 1);
+      // r.z in the lower lanes, r.r in the upper ones
+      const double sum = total(six{}, 1, 2 * w + (lane >> 4));
+      const double rzn = sum, rr = __shfl_sync(0xffffffffu, sum, 16);
       KState& k = sk[w];
       if (lane == 0) {
         T be = T(0);
@@ -450,7 +496,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
           k.iter++;
           k.rr = rr;
           if (!isfinite(rr)) { k.done = 1; k.status = 5; }
-          else if (rr <= k.tol2 * k.bb) k.done = 1;
+          else if (rr <= k.tt) k.done = 1;
           else if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; }
           else {
             be = quotient(rzn, k.rz, T(0));
@@ -463,6 +509,11 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
     __syncthreads();
     live = !(sk[0].done && sk[1].done && sk[2].done);
   }
+  // no CTA leaves while another still reads its rows: the last fetch has arrived
+  // (its values are used) before this CTA's arrival
+  if (ghosts) pw[4 * wrow(t) + 3] = gh[0] + gh[1] + gh[2] + gh[3];
+  __syncwarp();
+  cluster_barrier();
 #pragma unroll
   for (int j = 0; j < AFC_RPT; ++j)
 #pragma unroll
