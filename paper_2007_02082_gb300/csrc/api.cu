@@ -124,7 +124,7 @@ struct Engine {
   // mixed path, gradient viscous form: the lo parts of the momentum
   // coefficient pairs (coef32 holds the hi parts); coef64 is not held then
   float* coeflo32 = nullptr;
-  float *r32 = nullptr, *e32 = nullptr, *w32 = nullptr;
+  float *e32 = nullptr, *w32 = nullptr;
   double *X = nullptr, *dS = nullptr, *UB = nullptr, *BF = nullptr, *Gf = nullptr, *ibw = nullptr;
   double* ib_y64 = nullptr;       // mixed force solve: FP64 S G
   float* ib_w32 = nullptr;        // mixed force solve: FP32 work (7 x 3 M)
@@ -728,7 +728,6 @@ ib_status engine_build(Engine& E) {
     TRY(dalloc(E, &E.dK32, ns, true));
     TRY(dalloc(E, &E.dM32, ns, true));
     TRY(dalloc(E, &E.dA32, ns, true));
-    TRY(dalloc(E, &E.r32, 3 * ns, true));
     TRY(dalloc(E, &E.e32, 3 * ns, true));
     TRY(dalloc(E, &E.w32, 8 * 3 * ns, true));
   }
@@ -939,7 +938,6 @@ SolveArgs solve_args(Engine& E, int op, bool bicg, int nc, uint16_t dmask, const
   a.w32 = E.w32;
   a.y64 = E.y64;
   a.r64 = E.r64;
-  a.r32 = E.r32;
   a.e32 = E.e32;
   a.ks = E.ks;
   a.os = E.os;

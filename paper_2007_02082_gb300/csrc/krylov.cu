@@ -126,8 +126,7 @@ template <typename T, int NC>
 __global__ void __launch_bounds__(512) k_cg_start(DevGrid g, const T* __restrict__ b, const T* __restrict__ y,
                                                   T* __restrict__ r, T* __restrict__ z, T* __restrict__ p,
                                                   const T* __restrict__ dinv, uint16_t dmask, KState* ks,
-                                                  double* partials, unsigned* counter, Cond cond,
-                                                  const OState* skip_os) {
+                                                  double* partials, unsigned* counter, Cond cond) {
   KCOUNT();
   const int64_t s = (int64_t)blockIdx.x * DBV + threadIdx.x;
   const uint16_t m = g.meta[s];
@@ -135,7 +134,7 @@ __global__ void __launch_bounds__(512) k_cg_start(DevGrid g, const T* __restrict
   for (int c = 0; c < NC; ++c) {
     const bool dof = kdof(m, dmask, c), keep = kkeep(m, dmask, c);
     const int64_t i = c * g.nslots + s;
-    T rv = keep ? (y ? T(b[i] - y[i]) : b[i]) : T(0);
+    T rv = keep ? T(b[i] - y[i]) : T(0);
     T zv = rv * dinv[s];
     r[i] = rv;
     z[i] = zv;
@@ -148,7 +147,6 @@ __global__ void __launch_bounds__(512) k_cg_start(DevGrid g, const T* __restrict
   if (!grid_sum_last<T, 3 * NC>(tv, partials, counter, g.bseg, g.ninst, g.binst[blockIdx.x], out)) return;
   bool any = false;
   for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {   // one thread per system: the divisions overlap
-    const bool skip = skip_os && skip_os[e / NC].done;
     KState& k = ks[e];
     const double* t = out + (int64_t)3 * e;
     k.rz = t[0];
@@ -161,8 +159,8 @@ __global__ void __launch_bounds__(512) k_cg_start(DevGrid g, const T* __restrict
     k.alpha = 0.0;
     k.beta = 0.0;
     k.af = k.bf = 0.f;
-    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
-    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    k.done = k.rr <= k.tol2 * k.bb ? 1 : 0;
+    if (!isfinite(k.rr)) { k.done = 1; k.status = 5; }
     any = any || !k.done;
   }
   any = block_any(any);
@@ -276,18 +274,17 @@ __global__ void __launch_bounds__(512) k_cg_update_vec(DevGrid g, T* __restrict_
 template <typename T>
 __global__ void __launch_bounds__(512) k_cg_start_r(DevGrid g, const T* __restrict__ b, const T* __restrict__ y,
                                                     T* __restrict__ r, uint16_t dmask, KState* ks,
-                                                    double* partials, unsigned* counter, const OState* skip_os) {
+                                                    double* partials, unsigned* counter) {
   KCOUNT();
   const int64_t s = (int64_t)blockIdx.x * DBV + threadIdx.x;
   const uint16_t m = g.meta[s];
   const bool dof = kdof(m, dmask), keep = kkeep(m, dmask);
-  const T rv = keep ? (y ? T(b[s] - y[s]) : b[s]) : T(0);
+  const T rv = keep ? T(b[s] - y[s]) : T(0);
   r[s] = rv;
   T tv[2] = {dof ? rv * rv : T(0), dof ? b[s] * b[s] : T(0)};
   double* out = partials + (int64_t)gridDim.x * 2;
   if (!grid_sum_last<T, 2>(tv, partials, counter, g.bseg, g.ninst, g.binst[blockIdx.x], out)) return;
   for (int i = threadIdx.x; i < g.ninst; i += blockDim.x) {
-    const bool skip = skip_os && skip_os[i].done;
     KState& k = ks[i];
     k.rr = out[(int64_t)i * 2];
     k.bb = fmax(out[(int64_t)i * 2 + 1], k.rr);
@@ -297,8 +294,8 @@ __global__ void __launch_bounds__(512) k_cg_start_r(DevGrid g, const T* __restri
     k.alpha = 0.0;
     k.beta = 0.0;
     k.af = k.bf = 0.f;
-    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
-    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    k.done = k.rr <= k.tol2 * k.bb ? 1 : 0;
+    if (!isfinite(k.rr)) { k.done = 1; k.status = 5; }
   }
 }
 
@@ -437,8 +434,7 @@ template <typename T, int NC>
 __global__ void __launch_bounds__(512) k_bcg_start(DevGrid g, const T* __restrict__ b, const T* __restrict__ y,
                                                    T* __restrict__ r, T* __restrict__ rh, T* __restrict__ p,
                                                    T* __restrict__ v, uint16_t dmask, KState* ks,
-                                                   double* partials, unsigned* counter, Cond cond,
-                                                   const OState* skip_os, int coupled) {
+                                                   double* partials, unsigned* counter, Cond cond, int coupled) {
   KCOUNT();
   const int64_t s = (int64_t)blockIdx.x * DBV + threadIdx.x;
   const uint16_t m = g.meta[s];
@@ -446,7 +442,7 @@ __global__ void __launch_bounds__(512) k_bcg_start(DevGrid g, const T* __restric
   for (int c = 0; c < NC; ++c) {
     const bool dof = kdof(m, dmask, c), keep = kkeep(m, dmask, c);
     const int64_t i = c * g.nslots + s;
-    T rv = keep ? (y ? T(b[i] - y[i]) : b[i]) : T(0);
+    T rv = keep ? T(b[i] - y[i]) : T(0);
     r[i] = rv;
     rh[i] = rv;
     p[i] = T(0);
@@ -459,7 +455,6 @@ __global__ void __launch_bounds__(512) k_bcg_start(DevGrid g, const T* __restric
   bool any = false;
   for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
     const int i = e / NC, c = e - NC * i;
-    const bool skip = skip_os && skip_os[i].done;
     KState& k = ks[e];
     k.rr = total_of<NC, 2>(out, i, c, 0, coupled);
     k.bb = fmax(total_of<NC, 2>(out, i, c, 1, coupled), k.rr);
@@ -472,8 +467,8 @@ __global__ void __launch_bounds__(512) k_bcg_start(DevGrid g, const T* __restric
     k.bf = 0.f;
     k.iter = 0;
     k.status = 0;
-    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
-    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    k.done = k.rr <= k.tol2 * k.bb ? 1 : 0;
+    if (!isfinite(k.rr)) { k.done = 1; k.status = 5; }
     any = any || !k.done;
   }
   any = block_any(any);
@@ -747,7 +742,7 @@ __global__ void __launch_bounds__(512) k_bcgv_xr(DevGrid g, T* __restrict__ x, T
 // squares (scale, sum: no FP64 instruction per element, no underflow for
 // entries above 2^-126) that it hands to the FP64 grid sum as scale^2 sum;
 // per component the power of two that brings ||r|| into [0.5, 1) (sexp), by
-// which k_scale_residual divides r when it rounds it to FP32 as the inner
+// which k_start32 divides r when it rounds it to FP32 as the inner
 // right-hand side, so that the FP32 iterations never see values whose
 // squares leave the FP32 range (a problem in SI units has velocity
 // residuals near 1e-20).  Sets the outer loop condition and the condition of
@@ -851,39 +846,171 @@ __global__ void __launch_bounds__(512) k_residual_outer(DevGrid g, const double*
   }
 }
 
-// r32 = r * 2^-sexp, rounded to FP32: the scaled inner right-hand side (only
-// instances whose outer loop is still running); r comes as the pair (hi, lo)
-// that k_residual_outer stored in place of an FP64 value
-__global__ void k_scale_residual(DevGrid g, const double* __restrict__ r64, float* __restrict__ r32, int nc,
-                                 const OState* os) {
-  KCOUNT();
-  const OState& o = os[g.binst[blockIdx.x]];
-  if (o.done) return;
-  const int64_t s = (int64_t)blockIdx.x * DBV + threadIdx.x;
-  const float2* rp = reinterpret_cast<const float2*>(r64);
-  for (int c = 0; c < nc; ++c) {
-    const float2 p = rp[c * g.nslots + s];
-    // a power of two applied in at most two exact steps (the scale may leave
-    // the normal FP32 range; the scaled values do not)
-    const int e = -o.sexp[c];
-    const int e1 = e > 126 ? 126 : (e < -126 ? -126 : e);
-    const int e2 = max(-126, min(126, e - e1));
-    const float v = __fadd_rn(p.x, p.y);
-    r32[c * g.nslots + s] = __fmul_rn(__fmul_rn(v, __int_as_float((127 + e1) << 23)), __int_as_float((127 + e2) << 23));
-  }
-}
-
 // x += e * 2^sexp (the inner solution of the scaled right-hand side), only
 // for instances whose outer loop is still running
 // (e exactly in FP64 from its bits, the power of two on the exponent field:
-// one FP64 instruction per element, the addition)
-__global__ void k_add_f2d_active(DevGrid g, const float* __restrict__ e, double* __restrict__ x, int nc,
-                                 const OState* os) {
+// one FP64 instruction per element, the addition).  Two slots a thread and
+// step; bound by HBM: 20 bytes a slot and component (16 M-node sac 170 us a
+// pass, a mean over one- and three-component passes).
+__global__ void __launch_bounds__(512) k_add_f2d_active(DevGrid g, const float* __restrict__ e, double* __restrict__ x,
+                                                        int nc, const OState* os) {
   KCOUNT();
-  const OState& o = os[g.binst[blockIdx.x]];
+  const int b0 = g.scbrick[blockIdx.x], b1 = g.scbrick[blockIdx.x + 1];
+  const OState& o = os[g.binst[b0]];
   if (o.done) return;
-  const int64_t s = (int64_t)blockIdx.x * DBV + threadIdx.x;
-  for (int c = 0; c < nc; ++c) x[c * g.nslots + s] += scale2(f2d(e[c * g.nslots + s]), o.sexp[c]);
+  const int64_t s1 = (int64_t)b1 * DBV;
+#pragma unroll 2
+  for (int64_t s = (int64_t)b0 * DBV + threadIdx.x * 2; s < s1; s += (int64_t)blockDim.x * 2) {
+    const uint32_t mv = *reinterpret_cast<const uint32_t*>(g.meta + s);
+    if (!((mv | (mv >> 16)) & D_VALID)) continue;   // brick padding stays zero
+    for (int c = 0; c < nc; ++c) {
+      const int64_t i = c * g.nslots + s;
+      const float2 ev = *reinterpret_cast<const float2*>(e + i);
+      double2 xv = *reinterpret_cast<const double2*>(x + i);
+      xv.x += scale2(f2d(ev.x), o.sexp[c]);
+      xv.y += scale2(f2d(ev.y), o.sexp[c]);
+      *reinterpret_cast<double2*>(x + i) = xv;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- starts of the inner solves
+// The right-hand side of an inner solve is the outer residual r * 2^-sexp
+// rounded to FP32 (r as the pairs (hi, lo) that k_residual_outer stored in place
+// of FP64 values), formed here where the solve starts from it: the correction
+// starts from zero, so the residual is the right-hand side and nothing else reads it.
+// MG CG: r; Jacobi CG: r, z = p = D^-1 r; BiCGStab: r, rh = r, p = v = 0; and the
+// sums the states start from.  A CTA of four groups of 128 threads takes a
+// chunk, a brick a group and step, four nodes a thread with 16-byte accesses; each
+// brick's sums are formed in the order of a 512-thread CTA with a node a thread
+// (sixteen warps of 32 nodes), then in FP64.  Bound by HBM.  16 M-node sac,
+// the scaling pass it replaces included: Jacobi CG 678 -> 447 us; the whole
+// step 110.0 -> 108.4 ms.
+enum StartKind : int { START_MG = 0, START_JACOBI = 1, START_BCG = 2 };
+
+template <int KIND, int NC>
+__global__ void __launch_bounds__(512) k_start32(DevGrid g, const double* __restrict__ r64, float* __restrict__ r,
+                                                 float* __restrict__ z, float* __restrict__ p, float* __restrict__ v,
+                                                 const float* __restrict__ dinv, uint16_t dmask, KState* ks,
+                                                 double* partials, unsigned* counter, Cond cond, const OState* os,
+                                                 int coupled) {
+  KCOUNT();
+  constexpr int NS = KIND == START_JACOBI ? 3 : 2, NV = NS * NC;
+  __shared__ float sh[4][NV][16];
+  __shared__ double gs[4][NV];
+  const int b0 = g.scbrick[blockIdx.x], b1 = g.scbrick[blockIdx.x + 1];
+  const int inst = g.binst[b0];
+  const OState& o = os[inst];
+  const int grp = threadIdx.x >> 7, lt = threadIdx.x & 127, lane = threadIdx.x & 31, gw = lt >> 5;
+  double sum[(NV + 3) / 4];   // lane 0 of the group's warps: values gw, gw + 4, ...
+#pragma unroll
+  for (int q = 0; q < (NV + 3) / 4; ++q) sum[q] = 0.0;
+  if (!o.done)
+    for (int b = b0 + grp; b < b1; b += 4) {
+      const int64_t s = (int64_t)b * DBV + 4 * lt;
+      const uint2 mv = *reinterpret_cast<const uint2*>(g.meta + s);
+      const uint16_t* mm = reinterpret_cast<const uint16_t*>(&mv);
+      const bool any = ((mm[0] | mm[1] | mm[2] | mm[3]) & D_VALID) != 0;
+      float a[NV][4];
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[k][j] = 0.f;
+      if (any) {   // brick padding stays zero
+        float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (KIND == START_JACOBI) dv = *reinterpret_cast<const float4*>(dinv + s);
+        const float de[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const int64_t i = c * g.nslots + s;
+          const float4 h0 = *reinterpret_cast<const float4*>(r64 + i), h1 = *reinterpret_cast<const float4*>(r64 + i + 2);
+          const float hi[4] = {h0.x, h0.z, h1.x, h1.z}, lo[4] = {h0.y, h0.w, h1.y, h1.w};
+          // a power of two applied in at most two exact steps (the scale may leave
+          // the normal FP32 range; the scaled values do not)
+          const int e = -o.sexp[c];
+          const int e1 = e > 126 ? 126 : (e < -126 ? -126 : e);
+          const int e2 = max(-126, min(126, e - e1));
+          const float f1 = __int_as_float((127 + e1) << 23), f2 = __int_as_float((127 + e2) << 23);
+          float rv[4], zv[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float bv = __fmul_rn(__fmul_rn(__fadd_rn(hi[j], lo[j]), f1), f2);
+            const bool dof = kdof(mm[j], dmask, c), keep = kkeep(mm[j], dmask, c);
+            rv[j] = keep ? bv : 0.f;
+            zv[j] = __fmul_rn(rv[j], de[j]);
+            if (dof) {
+              if (KIND == START_JACOBI) a[NS * c][j] = __fmul_rn(rv[j], zv[j]);
+              a[NS * c + NS - 2][j] = __fmul_rn(rv[j], rv[j]);
+              a[NS * c + NS - 1][j] = __fmul_rn(bv, bv);
+            }
+          }
+          const float4 r4 = make_float4(rv[0], rv[1], rv[2], rv[3]), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+          *reinterpret_cast<float4*>(r + i) = r4;
+          if (KIND == START_JACOBI) {
+            const float4 z4 = make_float4(zv[0], zv[1], zv[2], zv[3]);
+            *reinterpret_cast<float4*>(z + i) = z4;
+            *reinterpret_cast<float4*>(p + i) = z4;
+          } else if (KIND == START_BCG) {   // z: rh
+            *reinterpret_cast<float4*>(z + i) = r4;
+            *reinterpret_cast<float4*>(p + i) = zero;
+            *reinterpret_cast<float4*>(v + i) = zero;
+          }
+        }
+      }
+      // the 32 nodes of eight threads, as a warp's tree
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+#pragma unroll
+        for (int q = 4; q > 0; q >>= 1)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) a[k][j] += __shfl_xor_sync(0xffffffffu, a[k][j], q);
+        const float t = (a[k][0] + a[k][2]) + (a[k][1] + a[k][3]);
+        if ((lane & 7) == 0) sh[grp][k][lt >> 3] = t;
+      }
+      asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory");
+#pragma unroll
+      for (int q = 0; q < (NV + 3) / 4; ++q) {
+        const int k = gw + 4 * q;
+        if (k < NV) {
+          const float t = lane_sum(lane < 16 ? sh[grp][k][lane] : 0.f);
+          sum[q] += double(t);
+        }
+      }
+      asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory");
+    }
+#pragma unroll
+  for (int q = 0; q < (NV + 3) / 4; ++q)
+    if (lane == 0 && gw + 4 * q < NV) gs[grp][gw + 4 * q] = sum[q];
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    const int k = threadIdx.x;
+    partials[(int64_t)blockIdx.x * NV + k] = (gs[0][k] + gs[1][k]) + (gs[2][k] + gs[3][k]);
+  }
+  double* out = partials + (int64_t)gridDim.x * NV;
+  if (!grid_finish<NV>(partials, counter, g.scseg, g.ninst, inst, out)) return;
+  bool live = false;
+  for (int e = threadIdx.x; e < g.ninst * NC; e += blockDim.x) {
+    const int i = e / NC, c = e - NC * i;
+    const bool skip = os[i].done != 0;
+    KState& k = ks[e];
+    k.rr = total_of<NC, NS>(out, i, c, NS - 2, coupled);
+    // reference norm max(||b||, ||r0||)
+    k.bb = fmax(total_of<NC, NS>(out, i, c, NS - 1, coupled), k.rr);
+    k.rz = KIND == START_JACOBI ? out[(int64_t)NV * i + NS * c] : 0.0;
+    k.rho = k.rr;
+    k.alpha = KIND == START_BCG ? 1.0 : 0.0;
+    k.omega = KIND == START_BCG ? 1.0 : 0.0;
+    k.beta = 0.0;
+    k.af = k.of = KIND == START_BCG ? 1.f : 0.f;
+    k.bf = 0.f;
+    k.iter = 0;
+    k.status = 0;
+    k.done = (skip || k.rr <= k.tol2 * k.bb) ? 1 : 0;
+    if (!skip && !isfinite(k.rr)) { k.done = 1; k.status = 5; }
+    live = live || !k.done;
+  }
+  live = block_any(live);
+  if (KIND != START_MG && threadIdx.x == 0) set_cond(cond, live);
 }
 
 // ---------------------------------------------------------------- drivers
@@ -916,8 +1043,8 @@ static inline void pend(Prof* p, cudaStream_t s) { if (p && p->on) p->end(s); }
 
 // one CG solve of A x = b in precision T (x: initial guess in, solution out)
 template <typename T, int NC>
-static cudaError_t cg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const T* b, T* x, T* work, cudaStream_t st,
-                              CaptureCtx* cc, double rtol, const OState* skip_os, bool x_zero) {
+static cudaError_t cg_enqueue(const SolveArgs& a, const OpDesc<T>& A, T* x, T* work, cudaStream_t st,
+                              CaptureCtx* cc, double rtol, const OState* os) {
   const DevGrid& g = *a.g;
   const int64_t L = int64_t(NC) * g.nslots;
   Work<T> w = carve(work, L);
@@ -929,9 +1056,14 @@ static cudaError_t cg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const T* b
     cudaError_t e = cond_handle(st, 0, &cond);
     if (e != cudaSuccess) return e;
   }
-  if (!x_zero) fe_apply<T>(g, A, NC, x, w.q, st);
-  IBG_LAUNCH((k_cg_start<T, NC>), g.nbricks, DBV, 0, st, g, b, x_zero ? (const T*)nullptr : (const T*)w.q, w.r,
-             w.z, w.pa, A.dinv, A.dmask, a.ks, rb.partials, rb.counter, cond, skip_os);
+  if constexpr (sizeof(T) == 4) {   // a correction of the mixed path
+    IBG_LAUNCH((k_start32<START_JACOBI, NC>), g.nschunks, DBV, 0, st, g, (const double*)a.r64, w.r, w.z, w.pa,
+               (float*)nullptr, A.dinv, A.dmask, a.ks, rb.partials, rb.counter, cond, os, 0);
+  } else {
+    fe_apply<T>(g, A, NC, x, w.q, st);
+    IBG_LAUNCH((k_cg_start<T, NC>), g.nbricks, DBV, 0, st, g, a.b, (const T*)w.q, w.r, w.z, w.pa, A.dinv, A.dmask,
+               a.ks, rb.partials, rb.counter, cond);
+  }
   fe_expand2<T>(g, NC, w.z, w.pa, st);
   auto iter = [&](cudaStream_t s, const Cond& c, T* pold, T* pnew) {
     pbegin(a.prof, a.pbase + 0, s);
@@ -957,9 +1089,8 @@ static const MGDev<T>* mg_of(const SolveArgs& a) {
 
 // CG with the multigrid V-cycle as preconditioner (Poisson, one component)
 template <typename T>
-static cudaError_t cg_mg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const MGDev<T>& mg, const T* b, T* x,
-                                 T* work, cudaStream_t st, CaptureCtx* cc, double rtol, const OState* skip_os,
-                                 bool x_zero) {
+static cudaError_t cg_mg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const MGDev<T>& mg, T* x, T* work,
+                                 cudaStream_t st, CaptureCtx* cc, double rtol, const OState* os) {
   const DevGrid& g = *a.g;
   const int64_t L = g.nslots;
   Work<T> w = carve(work, L);
@@ -971,9 +1102,15 @@ static cudaError_t cg_mg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const M
     cudaError_t e = cond_handle(st, 0, &cond);
     if (e != cudaSuccess) return e;
   }
-  if (!x_zero) fe_apply<T>(g, A, 1, x, w.q, st);
-  IBG_LAUNCH(k_cg_start_r<T>, g.nbricks, DBV, 0, st, g, b, x_zero ? (const T*)nullptr : (const T*)w.q, w.r, A.dmask,
-             a.ks, rb.partials, rb.counter, skip_os);
+  if constexpr (sizeof(T) == 4) {   // a correction of the mixed path
+    IBG_LAUNCH((k_start32<START_MG, 1>), g.nschunks, DBV, 0, st, g, (const double*)a.r64, w.r, (float*)nullptr,
+               (float*)nullptr, (float*)nullptr, (const float*)nullptr, A.dmask, a.ks, rb.partials, rb.counter, Cond(),
+               os, 0);
+  } else {
+    fe_apply<T>(g, A, 1, x, w.q, st);
+    IBG_LAUNCH(k_cg_start_r<T>, g.nbricks, DBV, 0, st, g, a.b, (const T*)w.q, w.r, A.dmask, a.ks, rb.partials,
+               rb.counter);
+  }
   mg_vcycle<T>(g, mg, w.r, w.z, zs, w.q, A.dinv, A.dmask, a.ks, st, a.prof, 9);
   IBG_LAUNCH(k_cg_rz<T>, g.nschunks, DBV / Vec16<T>::W, 0, st, g, w.r, w.z, A.dmask, a.ks, rb.partials, rb.counter, cond, 1);
   auto iter = [&](cudaStream_t s, const Cond& c, T* pold, T* pnew) {
@@ -995,8 +1132,8 @@ static cudaError_t cg_mg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const M
 }
 
 template <typename T, int NC>
-static cudaError_t bcg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const T* b, T* x, T* work, cudaStream_t st,
-                               CaptureCtx* cc, double rtol, const OState* skip_os, bool x_zero) {
+static cudaError_t bcg_enqueue(const SolveArgs& a, const OpDesc<T>& A, T* x, T* work, cudaStream_t st,
+                               CaptureCtx* cc, double rtol, const OState* os) {
   const DevGrid& g = *a.g;
   const int64_t L = int64_t(NC) * g.nslots;
   Work<T> w = carve(work, L);
@@ -1007,10 +1144,15 @@ static cudaError_t bcg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const T* 
     cudaError_t e = cond_handle(st, 0, &cond);
     if (e != cudaSuccess) return e;
   }
-  if (!x_zero) fe_apply<T>(g, A, NC, x, w.tv, st);
   const int cpl = a.coupled ? 1 : 0;
-  IBG_LAUNCH((k_bcg_start<T, NC>), g.nbricks, DBV, 0, st, g, b, x_zero ? (const T*)nullptr : (const T*)w.tv, w.r,
-             w.rh, w.p, w.v, A.dmask, a.ks, rb.partials, rb.counter, cond, skip_os, cpl);
+  if constexpr (sizeof(T) == 4) {   // a correction of the mixed path
+    IBG_LAUNCH((k_start32<START_BCG, NC>), g.nschunks, DBV, 0, st, g, (const double*)a.r64, w.r, w.rh, w.p, w.v,
+               (const float*)nullptr, A.dmask, a.ks, rb.partials, rb.counter, cond, os, cpl);
+  } else {
+    fe_apply<T>(g, A, NC, x, w.tv, st);
+    IBG_LAUNCH((k_bcg_start<T, NC>), g.nbricks, DBV, 0, st, g, a.b, (const T*)w.tv, w.r, w.rh, w.p, w.v, A.dmask, a.ks,
+               rb.partials, rb.counter, cond, cpl);
+  }
   // v and t hold the interface-summed operator outputs (the start kernel set v = 0)
   return run_loop(cc, st, cond, a.ks, a.ks_host, g.ninst * NC, a.max_iter, 1, 8, [&](cudaStream_t s, const Cond& c) {
     pbegin(a.prof, a.pbase + 2, s);
@@ -1038,19 +1180,20 @@ static cudaError_t bcg_enqueue(const SolveArgs& a, const OpDesc<T>& A, const T* 
   });
 }
 
-// x_zero: the initial guess is zero (the mixed path's corrections), so its
-// operator product is not formed and the residual starts as b
+// One Krylov solve in precision T.  FP64: A x = a.b from the guess in x.  FP32: a
+// correction of the mixed path, A x = the scaled outer residual a.r64 of the
+// outer state os, from zero (x holds zeros).
 template <typename T>
-static cudaError_t inner_enqueue(const SolveArgs& a, const OpDesc<T>& A, const T* b, T* x, T* work, cudaStream_t st,
-                                 CaptureCtx* cc, double rtol, const OState* skip_os, bool x_zero) {
-  if (a.bicg) return a.nc == 1 ? bcg_enqueue<T, 1>(a, A, b, x, work, st, cc, rtol, skip_os, x_zero)
-                               : bcg_enqueue<T, 3>(a, A, b, x, work, st, cc, rtol, skip_os, x_zero);
+static cudaError_t inner_enqueue(const SolveArgs& a, const OpDesc<T>& A, T* x, T* work, cudaStream_t st,
+                                 CaptureCtx* cc, double rtol, const OState* os) {
+  if (a.bicg) return a.nc == 1 ? bcg_enqueue<T, 1>(a, A, x, work, st, cc, rtol, os)
+                               : bcg_enqueue<T, 3>(a, A, x, work, st, cc, rtol, os);
   if (a.nc == 1 && a.op == OP_POISSON) {
     const MGDev<T>* mg = mg_of<T>(a);
-    if (mg && mg->any) return cg_mg_enqueue<T>(a, A, *mg, b, x, work, st, cc, rtol, skip_os, x_zero);
+    if (mg && mg->any) return cg_mg_enqueue<T>(a, A, *mg, x, work, st, cc, rtol, os);
   }
-  return a.nc == 1 ? cg_enqueue<T, 1>(a, A, b, x, work, st, cc, rtol, skip_os, x_zero)
-                   : cg_enqueue<T, 3>(a, A, b, x, work, st, cc, rtol, skip_os, x_zero);
+  return a.nc == 1 ? cg_enqueue<T, 1>(a, A, x, work, st, cc, rtol, os)
+                   : cg_enqueue<T, 3>(a, A, x, work, st, cc, rtol, os);
 }
 
 cudaError_t solve_enqueue(const SolveArgs& a, cudaStream_t st, CaptureCtx* cc) {
@@ -1058,7 +1201,7 @@ cudaError_t solve_enqueue(const SolveArgs& a, cudaStream_t st, CaptureCtx* cc) {
   OpDesc<double> A64{a.op, a.coef64, a.dmask, a.dinv64, a.prof, a.pbase};
   const int ib = (g.ninst + 127) / 128;
   if (!a.mixed) {
-    cudaError_t e = inner_enqueue<double>(a, A64, a.b, a.x, a.w64, st, cc, a.rtol, nullptr, false);
+    cudaError_t e = inner_enqueue<double>(a, A64, a.x, a.w64, st, cc, a.rtol, nullptr);
     if (e != cudaSuccess) return e;
     IBG_LAUNCH(k_collect, ib, 128, 0, st, a.ks, a.nc, g.ninst, a.rec, (OState*)nullptr);
     return cudaSuccess;
@@ -1076,11 +1219,10 @@ cudaError_t solve_enqueue(const SolveArgs& a, cudaStream_t st, CaptureCtx* cc) {
                  a.rb.counter, cl, cb);
   };
   auto correction = [&](cudaStream_t s) {
-    IBG_LAUNCH(k_scale_residual, g.nbricks, DBV, 0, s, g, (const double*)a.r64, a.r32, a.nc, (const OState*)a.os);
     // the correction starts from zero (k_residual_outer cleared e32)
-    cudaError_t e = inner_enqueue<float>(a, A32, a.r32, a.e32, a.w32, s, cc, a.rtol_inner, a.os, true);
+    cudaError_t e = inner_enqueue<float>(a, A32, a.e32, a.w32, s, cc, a.rtol_inner, a.os);
     IBG_LAUNCH(k_collect, ib, 128, 0, s, a.ks, a.nc, g.ninst, a.rec, a.os);
-    IBG_LAUNCH(k_add_f2d_active, g.nbricks, DBV, 0, s, g, a.e32, a.x, a.nc, (const OState*)a.os);
+    IBG_LAUNCH(k_add_f2d_active, g.nschunks, DBV, 0, s, g, a.e32, a.x, a.nc, (const OState*)a.os);
     // the FP32 correction carries hanging values rounded in FP32: restore the
     // constraint (hanging = mean of parents) in FP64
     fe_expand<double>(g, a.nc, a.x, s);
