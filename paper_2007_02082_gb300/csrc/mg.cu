@@ -19,6 +19,7 @@
 
 #include "async.cuh"
 #include "fe.hpp"
+#include "ib.h"
 #include "mgdev.hpp"
 
 namespace ibg {
@@ -202,12 +203,17 @@ __global__ void k_mg_fp_gather(MGLevelDev<T> L0, const uint8_t* __restrict__ on,
 // and all of a thread's loads of one pass are in flight together.  The
 // set-up data is read before the wait for the previous kernel (programmatic
 // dependent launch), so the first wave's reads overlap that kernel's tail.
+// Bound by the latency of its dependent rounds (chunk, values, footprint) at
+// three CTAs an SM, not by HBM (8 bytes a node).  A node's place in its cell, and so its four footprint entries and weights, depend on the thread
+// and the level alone (a G0 cell is no wider than a brick: three levels at most)
+// unless the brick reaches the last lattice plane; they are formed once per
+// level of the chunk.  16 M-node sac 105 -> 90 us, 64x64x256 L1 tube 27 -> 24.
 template <typename T>
-__global__ void __launch_bounds__(512, 3) k_mg_c_prolong(DevGrid g, MGLevelDev<T> L0, const T* __restrict__ zin,
-                                                      T* __restrict__ zout, uint16_t dmask,
-                                                      const uint8_t* __restrict__ on, const KState* ks) {
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 3 : 2)
+    k_mg_c_prolong(DevGrid g, MGLevelDev<T> L0, const T* __restrict__ zin, T* __restrict__ zout, uint16_t dmask,
+                   const uint8_t* __restrict__ on, const KState* ks) {
   constexpr int CH = 8;
-  __shared__ int sl[CH], sq[CH][3], sc0[CH][3];
+  __shared__ int sl[CH], sq[CH][3], sc0[CH][3], same[CH];
   __shared__ int64_t sfb[CH];
   // set-up data (the chunk, its instance, the metadata and the bricks'
   // lattice constants) before the wait for the previous kernel; then this
@@ -222,14 +228,17 @@ __global__ void __launch_bounds__(512, 3) k_mg_c_prolong(DevGrid g, MGLevelDev<T
   for (int i = 0; i < CH; ++i) m[i] = i < nb ? g.meta[(int64_t)(b0 + i) * DBV + t] : uint16_t(0);
   if (t < nb) {
     const int b = b0 + t, l = g.blev[b], sc = 1 << l;
+    bool inner = true;   // the last lattice plane lies beyond the brick
     sl[t] = l;
     sfb[t] = L0.fbase[b];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const int nla = L0.lat_n[3 * inst + a];
-      sq[t][a] = L0.bco[3 * b + a] * DBS;                                  // brick origin, level lattice
-      sc0[t][a] = l ? min(L0.bco[3 * b + a] * DBS / sc, nla - 2) : 0;     // the footprint's first G0 node
+      const int nla = L0.lat_n[3 * inst + a], q = L0.bco[3 * b + a] * DBS;
+      sq[t][a] = q;                                  // brick origin, level lattice
+      sc0[t][a] = l ? min(q / sc, nla - 2) : 0;      // the footprint's first G0 node
+      inner = inner && ((q + DBS - 1) >> l) <= nla - 2;
     }
+    same[t] = inner ? 1 : 0;
   }
   KCOUNT();
 #pragma unroll
@@ -239,49 +248,57 @@ __global__ void __launch_bounds__(512, 3) k_mg_c_prolong(DevGrid g, MGLevelDev<T
   if (skip) return;
   const int nl[3] = {L0.lat_n[3 * inst], L0.lat_n[3 * inst + 1], L0.lat_n[3 * inst + 2]};
   const int lt[3] = {t & 7, (t >> 3) & 7, t >> 6};
-  // every brick's value first, the stores after: no store stands between
-  // two bricks' footprint loads, so all of them are in flight together
-  T out[CH];
+  int lev = -1;   // the level that e and w are for; -1: of one brick only
+  int e[4] = {0, 0, 0, 0};
+  T w[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
   for (int i = 0; i < CH; ++i) {
-    out[i] = T(0);
-    if (i >= nb || !keep_slot(m[i], dmask)) continue;
+    if (i >= nb) break;
     const T* fp = L0.fp + sfb[i];
     const int l = sl[i];
+    const bool keep = keep_slot(m[i], dmask);
     if (l == 0) {   // a G0 node itself: weight 1 on its own footprint entry
-      out[i] = z[i] + T(1) * fp[t];
+      z[i] = keep ? z[i] + T(1) * fp[t] : T(0);
       continue;
     }
-    const int sc = 1 << l, nt = (6 + sc) / sc + 1;
-    int c[3], f[3];
+    if (l != lev || !same[i]) {
+      const int sc = 1 << l, nt = (6 + sc) / sc + 1;
+      int c[3], f[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int p = sq[i][a] + lt[a];
-      c[a] = min(p >> l, nl[a] - 2);   // the last cell holds the far lattice plane
-      f[a] = p - (c[a] << l);
-      c[a] -= sc0[i][a];
-    }
-    // axes by decreasing offset, ties in axis order: a stable three-element
-    // sort (swaps on strict inequality only)
-    int a0 = 0, a1 = 1, a2 = 2, f0 = f[0], f1 = f[1], f2 = f[2];
-    if (f1 > f0) { int x = a0; a0 = a1; a1 = x; x = f0; f0 = f1; f1 = x; }
-    if (f2 > f1) { int x = a1; a1 = a2; a2 = x; x = f1; f1 = f2; f2 = x; }
-    if (f1 > f0) { int x = a0; a0 = a1; a1 = x; x = f0; f0 = f1; f1 = x; }
-    const int vb[4] = {0, 1 << a0, (1 << a0) | (1 << a1), 7};
-    const int wn[4] = {sc - f0, f0 - f1, f1 - f2, f2};
-    const T inv = T(1) / T(sc);   // a power of two: exact
-    T v = z[i];
+      for (int a = 0; a < 3; ++a) {
+        const int p = sq[i][a] + lt[a];
+        c[a] = min(p >> l, nl[a] - 2);   // the last cell holds the far lattice plane
+        f[a] = p - (c[a] << l);
+        c[a] -= sc0[i][a];
+      }
+      // axes by decreasing offset, ties in axis order: a stable three-element
+      // sort (swaps on strict inequality only)
+      int a0 = 0, a1 = 1, a2 = 2, f0 = f[0], f1 = f[1], f2 = f[2];
+      if (f1 > f0) { int x = a0; a0 = a1; a1 = x; x = f0; f0 = f1; f1 = x; }
+      if (f2 > f1) { int x = a1; a1 = a2; a2 = x; x = f1; f1 = f2; f2 = x; }
+      if (f1 > f0) { int x = a0; a0 = a1; a1 = x; x = f0; f0 = f1; f1 = x; }
+      const int vb[4] = {0, 1 << a0, (1 << a0) | (1 << a1), 7};
+      const int wn[4] = {sc - f0, f0 - f1, f1 - f2, f2};
+      const T inv = T(1) / T(sc);   // a power of two: exact
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (wn[k] == 0) continue;
-      const int e = ((c[2] + ((vb[k] >> 2) & 1)) * nt + (c[1] + ((vb[k] >> 1) & 1))) * nt + (c[0] + (vb[k] & 1));
-      v += (T(wn[k]) * inv) * fp[e];   // a Dirichlet G0 node's entry is zero
+      for (int k = 0; k < 4; ++k) {
+        w[k] = T(wn[k]) * inv;
+        e[k] = ((c[2] + ((vb[k] >> 2) & 1)) * nt + (c[1] + ((vb[k] >> 1) & 1))) * nt + (c[0] + (vb[k] & 1));
+      }
+      lev = same[i] ? l : -1;
     }
-    out[i] = v;
+    T v = T(0);
+    if (keep) {
+      v = z[i];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)   // a Dirichlet G0 node's entry is zero
+        if (w[k] != T(0)) v += w[k] * fp[e[k]];
+    }
+    z[i] = v;
   }
 #pragma unroll
   for (int i = 0; i < CH; ++i)   // brick padding stays zero: no store
-    if (i < nb && (m[i] & D_VALID)) zout[(int64_t)(b0 + i) * DBV + t] = out[i];
+    if (i < nb && (m[i] & D_VALID)) zout[(int64_t)(b0 + i) * DBV + t] = z[i];
 }
 
 // b0 = R0 (r - A z), R0 = P0^T over owner slots, in two passes.
@@ -294,7 +311,7 @@ __global__ void __launch_bounds__(512, 3) k_mg_c_prolong(DevGrid g, MGLevelDev<T
 // +-(0,1,1), +-(1,0,1), +-(1,1,1)) with weight 1/2; its transpose gathers, for
 // a coarse node at fine position 2t, the value there plus half of its 14
 // Kuhn neighbours.  An array of w nodes per axis becomes one of w / 2 + 1
-// (8 -> 5 -> 3 -> 2), each sum in a fixed order.
+// (8 -> 5 -> 3 -> 2, three levels at most), each sum in a fixed order.
 constexpr int R0_GROUP = 128;                    // threads per brick of the restriction
 constexpr int R0_BRICKS = 4;                     // bricks per CTA
 constexpr int R0_THREADS = R0_GROUP * R0_BRICKS;
@@ -307,24 +324,31 @@ __device__ __forceinline__ void kuhn_dir(int k, int& dx, int& dy, int& dz) {
 }
 
 // One level of the restriction for the 128 threads of a brick group (lt =
-// the thread's index in the group).
-template <typename T>
-__device__ __forceinline__ void restrict_one_level(const T* in, int w, T* out, int wo, int lt) {
-  for (int j = lt; j < wo * wo * wo; j += R0_GROUP) {
-    const int tx = j % wo, ty = (j / wo) % wo, tz = j / (wo * wo);
-    const int cx = 2 * tx, cy = 2 * ty, cz = 2 * tz;
-    auto at = [&](int x, int y, int z) -> T {
-      return (x >= 0 && x < w && y >= 0 && y < w && z >= 0 && z < w) ? in[(z * w + y) * w + x] : T(0);
-    };
-    T acc = at(cx, cy, cz);
+// the thread's index in the group): W nodes per axis to W / 2 + 1.  in: rows and
+// planes RestrictPitch apart with zeros behind each row (they also stand before
+// the next), behind each plane and before the first, so that no neighbour is
+// tested; put(x, y, z, value) takes each sum.
+template <int W>
+constexpr int RestrictPitch = 2 * (W / 2 + 1);
+template <int W>   // the zeros before the first node, on an even number of elements
+constexpr int RestrictLead = (RestrictPitch<W> * RestrictPitch<W> + RestrictPitch<W> + 2) & ~1;
+template <int W>
+constexpr int RestrictSize = RestrictLead<W> + RestrictPitch<W> * RestrictPitch<W> * RestrictPitch<W>;
+
+template <int W, typename T, typename Put>
+__device__ __forceinline__ void restrict_one_level(const T* in, int lt, Put put) {
+  constexpr int WO = W / 2 + 1, P = RestrictPitch<W>;
+  for (int j = lt; j < WO * WO * WO; j += R0_GROUP) {
+    const int tx = j % WO, ty = (j / WO) % WO, tz = j / (WO * WO);
+    const T* c = in + RestrictLead<W> + (2 * tz * P + 2 * ty) * P + 2 * tx;
     T half = T(0);
 #pragma unroll
     for (int k = 0; k < 14; ++k) {
       int dx, dy, dz;
       kuhn_dir(k, dx, dy, dz);
-      half += at(cx + dx, cy + dy, cz + dz);
+      half += c[(dz * P + dy) * P + dx];
     }
-    out[j] = acc + T(0.5) * half;
+    put(tx, ty, tz, c[0] + T(0.5) * half);
   }
 }
 
@@ -334,52 +358,63 @@ __device__ __forceinline__ void group_sync(int grp) {
 }
 
 // Four fine bricks per CTA of 512 threads, one group of 128 threads (four
-// slots per thread) per brick with its own named barrier, so that a CTA has
-// four bricks' loads in flight after two dependent rounds (the brick index,
-// then its residual values, metadata, level and instance together; the
-// instance's solver flags decide only whether the sums are written).
+// consecutive slots per thread) per brick with its own named barrier, so that a
+// CTA has four bricks' loads in flight after two dependent rounds (the brick
+// index, then its residual values, metadata, level and instance together; the
+// instance's solver flags decide only whether the sums are written).  Bound by the
+// latency of those rounds (10 bytes a slot are 33 us of HBM time there): each
+// level's array lies between zeros, written while the loads are in flight, so a
+// sum is 15 reads at constant offsets.  16 M-node sac 64 -> 59 us.
 template <typename T>
 __global__ void __launch_bounds__(R0_THREADS) k_mg_r0_part(DevGrid g, MGLevelDev<T> L0, const T* __restrict__ r,
                                                            const T* __restrict__ q, uint16_t dmask,
                                                            const uint8_t* __restrict__ on, const KState* ks) {
+  constexpr int P8 = RestrictPitch<8>, P5 = RestrictPitch<5>, P3 = RestrictPitch<3>;
+  constexpr int N8 = (RestrictSize<8> + 1) / 2 * 2, N5 = (RestrictSize<5> + 1) / 2 * 2,
+                N3 = (RestrictSize<3> + 1) / 2 * 2;
+  static_assert(DBS == 8 && IB_MAX_LEVEL <= 3, "8 -> 5 -> 3 -> 2 nodes an axis");
+  __shared__ __align__(16) T buf[R0_BRICKS][N8 + N5 + N3];
+  struct __align__(4 * sizeof(T)) Four { T v[4]; };
   KCOUNT();
-  __shared__ T bufa[R0_BRICKS][DBV];
-  __shared__ T bufb[R0_BRICKS][125];
   const int grp = threadIdx.x / R0_GROUP, lt = threadIdx.x % R0_GROUP;
   const int fi = blockIdx.x * R0_BRICKS + grp;
   if (fi >= L0.nfb) return;   // the whole group: its barrier is its own
   const int b = L0.fbr[fi];
-  T v[DBV / R0_GROUP];
-  uint16_t mm[DBV / R0_GROUP];
-#pragma unroll
-  for (int k = 0; k < DBV / R0_GROUP; ++k) {
-    const int64_t s = (int64_t)b * DBV + lt + k * R0_GROUP;
-    mm[k] = g.meta[s];
-    v[k] = T(r[s] - q[s]);
-  }
+  const int64_t s = (int64_t)b * DBV + 4 * lt;
+  const uint2 mv = *reinterpret_cast<const uint2*>(g.meta + s);
+  const Four rv = *reinterpret_cast<const Four*>(r + s), qv = *reinterpret_cast<const Four*>(q + s);
   const int inst = g.binst[b];
-  int l = g.blev[b];
-  const int pb = L0.pbase[b];
-  if (ks[inst].done || !on[inst]) return;
-#pragma unroll
-  for (int k = 0; k < DBV / R0_GROUP; ++k) {
-    const uint16_t m = mm[k];
-    bufa[grp][lt + k * R0_GROUP] = ((m & D_VALID) && !(m & (D_HANG | D_DUP | dmask))) ? v[k] : T(0);
-  }
+  const int l = g.blev[b];
+  T* part = L0.part + L0.pbase[b];
+  T *a8 = buf[grp], *a5 = a8 + N8, *a3 = a5 + N5;
+  for (int i = lt; i < N8 + N5 + N3; i += R0_GROUP) a8[i] = T(0);
   group_sync(grp);
-  int w = DBS;
-  T* in = bufa[grp];
-  T* out = bufb[grp];
-  while (l > 1) {   // down to level 1 inside shared memory, alternating buffers
-    const int wo = w / 2 + 1;
-    restrict_one_level(in, w, out, wo, lt);
-    group_sync(grp);
-    T* tmp = in; in = out; out = tmp;
-    w = wo;
-    --l;
+  if (ks[inst].done || !on[inst]) return;
+  const uint16_t mm[4] = {uint16_t(mv.x & 0xFFFFu), uint16_t(mv.x >> 16), uint16_t(mv.y & 0xFFFFu),
+                          uint16_t(mv.y >> 16)};
+  T* c = a8 + RestrictLead<8> + ((lt >> 4) * P8 + ((lt >> 1) & 7)) * P8 + 4 * (lt & 1);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    c[j] = ((mm[j] & D_VALID) && !(mm[j] & (D_HANG | D_DUP | dmask))) ? T(rv.v[j] - qv.v[j]) : T(0);
+  group_sync(grp);
+  // each level into the next one's array, the last straight into the partial sums
+  // of the brick's G0 nodes
+  auto to_part = [&](int wo) {
+    return [part, wo](int x, int y, int z, T v) { part[(z * wo + y) * wo + x] = v; };
+  };
+  if (l == 1) {
+    restrict_one_level<8>(a8, lt, to_part(5));
+    return;
   }
-  // the last level straight into the partial sums of the brick's G0 nodes
-  restrict_one_level(in, w, L0.part + pb, w / 2 + 1, lt);
+  restrict_one_level<8>(a8, lt, [&](int x, int y, int z, T v) { a5[RestrictLead<5> + (z * P5 + y) * P5 + x] = v; });
+  group_sync(grp);
+  if (l == 2) {
+    restrict_one_level<5>(a5, lt, to_part(3));
+    return;
+  }
+  restrict_one_level<5>(a5, lt, [&](int x, int y, int z, T v) { a3[RestrictLead<3> + (z * P3 + y) * P3 + x] = v; });
+  group_sync(grp);
+  restrict_one_level<3>(a3, lt, to_part(2));
 }
 
 // Pass 2, one thread per G0 node: the level-0 owner copy at its position
