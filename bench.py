@@ -226,7 +226,7 @@ def class_bytes(cls, vb, multigrid=False):
         7: 3 * 7 * vb + 2,             # BiCGStab x, r update: x rw, ph, sh, s, t, rh read, r write (3 comps)
         8: 3 * 5 * vb + vb + 2,        # BiCGStab p update: r, v read, p rw, ph write (3 comps), D^-1
         9: 2 * vb + 2,                 # V-cycle stencil apply: read x, meta; write q
-        10: 5 * vb + 2,                # V-cycle smoothing update: read z, r, q, D^-1, meta; write z
+        10: (4 if vb == 4 else 5) * vb + 2,   # V-cycle sweep: read z, r, D^-1, meta; write z (FP64: q as well)
     }.get(cls)
 
 
@@ -253,8 +253,8 @@ CLASS_NAMES = {0: "k_poisson_cg (p = z + beta p, q = K p, fused p.q)", 1: "k_cg_
                5: "k_cg_p<mass>",
                6: "momentum apply, 15 coefficients, 3 comps (k_apply15_mom32 on the mixed path)",
                7: "k_bcgv_xr<momentum>",
-               8: "k_bcgv_p<momentum>", 9: "k_poisson_cg<apply> (V-cycle smoothing stencil)",
-               10: "k_mg_c_smooth (V-cycle smoothing update)", 11: "V-cycle transfers and coarse levels"}
+               8: "k_bcgv_p<momentum>", 9: "V-cycle stencil apply (k_poisson7_staged on the mixed path)",
+               10: "V-cycle sweep (k_poisson7_staged<false, true>; FP64: k_mg_c_smooth after an apply)", 11: "V-cycle transfers and coarse levels"}
 
 
 TUNE_CACHE = os.path.join(ROOT, "paper_2007_02082_gb300", "tune_cache.json")

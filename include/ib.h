@@ -181,8 +181,8 @@ typedef struct {
  *     [IB_TUNE_STREAM_CHUNK]    bricks per CTA of the streaming Krylov
  *                               kernels: 4 or 8 (default)
  *     [IB_TUNE_MG_SMALL]        multigrid levels with at most this many nodes
- *                               (64 .. 1048576, default 8192) run in one CTA
- *                               per problem
+ *                               (64 .. 1048576, default 8192) run in one
+ *                               cluster of CTAs per problem
  *     [IB_TUNE_MG_SWEEPS]       damped-Jacobi sweeps before and after the
  *                               coarse correction on the composite level and
  *                               G0: 1 .. 4 (default 2); the V-cycle stays a
@@ -244,7 +244,7 @@ typedef struct {
      class since ib_set_boundary; class = base + {0 operator apply, 1 vector
      update, 2 direction update}, base 0 Poisson, 3 mass, 6 momentum; the
      multigrid V-cycle: 9 composite stencil applies, 10 composite smoothing
-     updates, 11 transfers and coarse levels */
+     (sweeps in one pass, or the updates after an apply), 11 transfers and coarse levels */
   double prof_ms[12];
   int64_t prof_launches[12];
   int64_t kernel_launches;  /* kernels launched by this process's library so far */

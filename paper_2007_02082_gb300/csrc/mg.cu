@@ -204,10 +204,11 @@ __global__ void k_mg_fp_gather(MGLevelDev<T> L0, const uint8_t* __restrict__ on,
 // set-up data is read before the wait for the previous kernel (programmatic
 // dependent launch), so the first wave's reads overlap that kernel's tail.
 // Bound by the latency of its dependent rounds (chunk, values, footprint) at
-// three CTAs an SM, not by HBM (8 bytes a node).  A node's place in its cell, and so its four footprint entries and weights, depend on the thread
-// and the level alone (a G0 cell is no wider than a brick: three levels at most)
-// unless the brick reaches the last lattice plane; they are formed once per
-// level of the chunk.  16 M-node sac 105 -> 90 us, 64x64x256 L1 tube 27 -> 24.
+// three CTAs an SM, not by HBM (8 bytes a node).  A node's place in its cell,
+// and so its four footprint entries and weights, depend on the thread and the
+// level alone (a G0 cell is no wider than a brick: three levels at most) unless
+// the brick reaches the last lattice plane; they are formed once per level of
+// the chunk.  16 M-node sac 105 -> 90 us, 64x64x256 L1 tube 27 -> 24.
 template <typename T>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 3 : 2)
     k_mg_c_prolong(DevGrid g, MGLevelDev<T> L0, const T* __restrict__ zin, T* __restrict__ zout, uint16_t dmask,
@@ -763,7 +764,7 @@ __global__ void __launch_bounds__(LV_THREADS) k_mg_levels(LevelsArgs<T> a, const
     }
     if (!grid_barrier(a.bar, a.ninst, a.aerr)) return;
   }
-  // small levels and the coarsest solve, a CTA per problem
+  // small levels and the coarsest solve, here a CTA per problem
   __shared__ T tile[LV_TILE];
   for (int i = blockIdx.x; i < a.ninst; i += gridDim.x) {
     __syncthreads();
@@ -819,9 +820,8 @@ void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T*
   // one sweep: the fused stencil and update, then its interface nodes; or (FP64, other
   // launch choices) the apply with its sums, then the update
   auto sweep = [&](const T* zin, T* zout) {
-    bool fused = false;
-    timed(0, [&] { fused = fe_poisson_smooth<T>(g, zin, zout, r, q, dinv, w, dmask, ksm, mg.on, st); });
-    if (fused) {
+    if (fe_poisson_smooths<T>(g, zin, zout, r, dinv)) {
+      timed(1, [&] { fe_poisson_smooth<T>(g, zin, zout, r, q, dinv, w, dmask, ksm, mg.on, st); });
       if (g.n_if)
         IBG_LAUNCH(k_mg_if_smooth<T>, (g.n_if + 255) / 256, 256, 0, st, g, zin, zout, r, (const T*)q, dinv, dmask, mg.on,
                    w, ks);

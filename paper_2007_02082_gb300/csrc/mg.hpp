@@ -38,7 +38,7 @@ namespace ibg {
 
 constexpr int MG_MAX_LEVELS = 12;
 constexpr int64_t MG_MAX_COARSEST = 1024;   // nodes of the coarsest level (dense inverse)
-constexpr int64_t MG_SMALL_NODES = 8192;    // levels at most this size run in one CTA per problem
+constexpr int64_t MG_SMALL_NODES = 8192;    // levels at most this size run in one cluster per problem
 
 struct MGLevelHost {
   int64_t n[3] = {0, 0, 0};         // cells per axis
@@ -85,7 +85,7 @@ struct MGHost {
 inline int mg_targets_per_axis(int l) { return (6 + (1 << l)) / (1 << l) + 1; }
 
 // Build the hierarchy of one composite grid; levels with at most small_nodes
-// nodes run in one CTA per problem (small_start).  On failure (no outlet node at
+// nodes run in one cluster of CTAs per problem (small_start).  On failure (no outlet node at
 // all, or a transfer weight that points at a missing node) ok = false and the
 // Poisson solve of that problem keeps the Jacobi preconditioner.
 void build_mg(const HostGrid& G, MGHost& mg, int64_t small_nodes = MG_SMALL_NODES);

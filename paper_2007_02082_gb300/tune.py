@@ -2,8 +2,8 @@
 
 The choices change speed, not the method: the Poisson stencil kernel (staged
 asynchronously or register-pipelined), the bricks per CTA of the streaming
-Krylov kernels, the size below which multigrid levels run in one CTA per
-problem, and the damped-Jacobi sweeps of the V-cycle (a symmetric
+Krylov kernels, the size below which multigrid levels run in one cluster
+of CTAs per problem, and the damped-Jacobi sweeps of the V-cycle (a symmetric
 preconditioner for any sweep count, so the solution is the same to the
 solver tolerance; the iteration count and the time per step change).
 
