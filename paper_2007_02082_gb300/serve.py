@@ -33,7 +33,7 @@ from . import IBBatch, IBGrid
 # (column, FP64 value, FP32 copy if mixed), per entry of the coarsest
 # multigrid level's dense inverse (in the Krylov precision), and per problem
 # (solver states, reduction buffers, small tables)
-BYTES_PER_SLOT = {"mixed": 560, "fp64": 660}
+BYTES_PER_SLOT = {"mixed": 548, "fp64": 660}
 BYTES_PER_ROW = {"mixed": 1400 + 24 + 84 + 4, "fp64": 1400}
 BYTES_PER_NNZ = {"mixed": 16, "fp64": 12}
 BYTES_PER_CINV = {"mixed": 4, "fp64": 8}
