@@ -884,16 +884,17 @@ __global__ void __launch_bounds__(512) k_add_f2d_active(DevGrid g, const float* 
 // chunk, a brick a group and step, four nodes a thread with 16-byte accesses; each
 // brick's sums are formed in the order of a 512-thread CTA with a node a thread
 // (sixteen warps of 32 nodes), then in FP64.  Bound by HBM.  16 M-node sac,
-// the scaling pass it replaces included: Jacobi CG 678 -> 447 us; the whole
-// step 110.0 -> 108.4 ms.
+// the scaling pass it replaces included: BiCGStab 636 -> 268 us, Jacobi CG 678 ->
+// 284, MG CG 400 -> 96.  A component's sums are formed before the next one's
+// values are read: 64 registers where all nine at once took 90 (one CTA an SM,
+// Jacobi CG 447 us).
 enum StartKind : int { START_MG = 0, START_JACOBI = 1, START_BCG = 2 };
 
 template <int KIND, int NC>
-__global__ void __launch_bounds__(512) k_start32(DevGrid g, const double* __restrict__ r64, float* __restrict__ r,
-                                                 float* __restrict__ z, float* __restrict__ p, float* __restrict__ v,
-                                                 const float* __restrict__ dinv, uint16_t dmask, KState* ks,
-                                                 double* partials, unsigned* counter, Cond cond, const OState* os,
-                                                 int coupled) {
+__global__ void __launch_bounds__(512, KIND == START_JACOBI && NC == 3 ? 2 : 3)
+    k_start32(DevGrid g, const double* __restrict__ r64, float* __restrict__ r, float* __restrict__ z,
+              float* __restrict__ p, float* __restrict__ v, const float* __restrict__ dinv, uint16_t dmask, KState* ks,
+              double* partials, unsigned* counter, Cond cond, const OState* os, int coupled) {
   KCOUNT();
   constexpr int NS = KIND == START_JACOBI ? 3 : 2, NV = NS * NC;
   __shared__ float sh[4][NV][16];
@@ -911,17 +912,17 @@ __global__ void __launch_bounds__(512) k_start32(DevGrid g, const double* __rest
       const uint2 mv = *reinterpret_cast<const uint2*>(g.meta + s);
       const uint16_t* mm = reinterpret_cast<const uint16_t*>(&mv);
       const bool any = ((mm[0] | mm[1] | mm[2] | mm[3]) & D_VALID) != 0;
-      float a[NV][4];
+      float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (KIND == START_JACOBI && any) dv = *reinterpret_cast<const float4*>(dinv + s);
+      const float de[4] = {dv.x, dv.y, dv.z, dv.w};
 #pragma unroll
-      for (int k = 0; k < NV; ++k)
+      for (int c = 0; c < NC; ++c) {
+        float a[NS][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) a[k][j] = 0.f;
-      if (any) {   // brick padding stays zero
-        float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (KIND == START_JACOBI) dv = *reinterpret_cast<const float4*>(dinv + s);
-        const float de[4] = {dv.x, dv.y, dv.z, dv.w};
+        for (int k = 0; k < NS; ++k)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
+          for (int j = 0; j < 4; ++j) a[k][j] = 0.f;
+        if (any) {   // brick padding stays zero
           const int64_t i = c * g.nslots + s;
           const float4 h0 = *reinterpret_cast<const float4*>(r64 + i), h1 = *reinterpret_cast<const float4*>(r64 + i + 2);
           const float hi[4] = {h0.x, h0.z, h1.x, h1.z}, lo[4] = {h0.y, h0.w, h1.y, h1.w};
@@ -939,9 +940,9 @@ __global__ void __launch_bounds__(512) k_start32(DevGrid g, const double* __rest
             rv[j] = keep ? bv : 0.f;
             zv[j] = __fmul_rn(rv[j], de[j]);
             if (dof) {
-              if (KIND == START_JACOBI) a[NS * c][j] = __fmul_rn(rv[j], zv[j]);
-              a[NS * c + NS - 2][j] = __fmul_rn(rv[j], rv[j]);
-              a[NS * c + NS - 1][j] = __fmul_rn(bv, bv);
+              if (KIND == START_JACOBI) a[0][j] = __fmul_rn(rv[j], zv[j]);
+              a[NS - 2][j] = __fmul_rn(rv[j], rv[j]);
+              a[NS - 1][j] = __fmul_rn(bv, bv);
             }
           }
           const float4 r4 = make_float4(rv[0], rv[1], rv[2], rv[3]), zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -956,16 +957,16 @@ __global__ void __launch_bounds__(512) k_start32(DevGrid g, const double* __rest
             *reinterpret_cast<float4*>(v + i) = zero;
           }
         }
-      }
-      // the 32 nodes of eight threads, as a warp's tree
+        // the 32 nodes of eight threads, as a warp's tree
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
+        for (int k = 0; k < NS; ++k) {
 #pragma unroll
-        for (int q = 4; q > 0; q >>= 1)
+          for (int q = 4; q > 0; q >>= 1)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) a[k][j] += __shfl_xor_sync(0xffffffffu, a[k][j], q);
-        const float t = (a[k][0] + a[k][2]) + (a[k][1] + a[k][3]);
-        if ((lane & 7) == 0) sh[grp][k][lt >> 3] = t;
+            for (int j = 0; j < 4; ++j) a[k][j] += __shfl_xor_sync(0xffffffffu, a[k][j], q);
+          const float t = (a[k][0] + a[k][2]) + (a[k][1] + a[k][3]);
+          if ((lane & 7) == 0) sh[grp][NS * c + k][lt >> 3] = t;
+        }
       }
       asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory");
 #pragma unroll

@@ -31,7 +31,7 @@ namespace {
 // the nodes suffices.  Each set is summed over the lanes in one butterfly; the
 // 9 x 9 Cholesky solves of 32 points share one warp, a point a lane.  ib_wss on
 // the 32,000 points of the refined 64x64x256 tube, host copies included: 7.95 ms
-// with a thread per point and two passes, 3.45 ms here.
+// with a thread per point and two passes, 1.8 ms here.
 constexpr int WSS_PTS = 32;       // points of a CTA
 constexpr int WSS_WARPS = 8;
 
