@@ -533,8 +533,12 @@ __global__ void __launch_bounds__(512) k_bcgv_p(DevGrid g, const T* __restrict__
 }
 
 // mode 0: alpha = rho / (rh, v);  mode 1: omega = (t, s) / (t, t)
+// Reads only (6 V + 2 bytes a slot), bound by the latency of metadata and values:
+// four CTAs an SM in FP32 (32 registers, 8 bytes of spill) take 87 us on the 16
+// M-node sac and 22 on the 64x64x256 L1 tube, three 101 and 26, two with
+// two steps' loads in flight 113 and 31.
 template <typename T, int NC>
-__global__ void __launch_bounds__(512) k_bcgv_dot(DevGrid g, const T* __restrict__ a1, const T* __restrict__ b1v,
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 4 : 3) k_bcgv_dot(DevGrid g, const T* __restrict__ a1, const T* __restrict__ b1v,
                                                   uint16_t dmask, int mode, KState* ks, double* partials,
                                                   unsigned* counter, int coupled) {
   KCOUNT();
