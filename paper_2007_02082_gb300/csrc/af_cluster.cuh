@@ -76,18 +76,6 @@ __device__ __forceinline__ void cluster_store(uint32_t a, double v) {
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
-// a / b as T.  FP32: rounded from the quotient to about 2^-46, by one correction
-// of an FP32 division (an FP64 division is a chain of a dozen FP64
-// instructions, and every row waits for it), FP64 where FP32 could not hold
-// the operands.
-__device__ __forceinline__ float quotient(double a, double b, float) {
-  const unsigned ea = (unsigned(__double2hiint(a)) >> 20) & 0x7FFu, eb = (unsigned(__double2hiint(b)) >> 20) & 0x7FFu;
-  if (ea - 923u > 200u || eb - 923u > 200u) return float(a / b);   // outside 2^-100 .. 2^100
-  const float inv = __frcp_rn(float(b));
-  const float q = __fmul_rn(float(a), inv);
-  return fmaf(float(fma(-double(q), b, a)), inv, q);
-}
-__device__ __forceinline__ double quotient(double a, double b, double) { return a / b; }
 // sum over the first `width` lanes (a power of two), valid in lane 0
 __device__ __forceinline__ double lanes_sum(double x, int width) {
   for (int o = width >> 1; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
@@ -218,11 +206,13 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   };
   auto wrow = [&](int i) { return i < own0 - w0 ? i : i + rpc; };   // window row of the i-th row of others
   const uint32_t ghost0 = t < wn - rpc ? owner(w0 + wrow(t)) : 0u;
-  // The sums over rows carry the bits of the loop's kernels in FP32, where an
-  // ill-conditioned S makes the number of passes, and whether FP64 takes over,
-  // hang on them: FP32 within the blocks of rows that those kernels sum, in
-  // their order (p.q: 32 rows, four to a warp, then eight warps; r.z and r.r:
-  // 256 rows, 32 to a warp, then eight warps), FP64 beyond.
+  // The sums over rows carry the bits of the loop's kernels in FP32 within the blocks
+  // of rows that those kernels sum, in their order (p.q: 32 rows, four to a
+  // warp, then eight warps; r.z and r.r: 256 rows, 32 to a warp, then eight
+  // warps): an ill-conditioned S makes the number of passes, and whether FP64
+  // takes over, hang on them.  Beyond the blocks both add in FP64, in another order
+  // (p.q from 1025 rows on, r.z and r.r from 4097), and both round FP64 quotients
+  // to FP32, so that the scalars differ only where the last bit of FP64 decides.
   auto unit_sums = [&](auto& v, auto nv, int u, int buf) {   // a warp's 32 rows, in one butterfly (warp_sums)
     constexpr int NV = decltype(nv)::value, P = NV == 3 ? 4 : 8, PB = NV == 3 ? 2 : 3;
     constexpr int off[5] = {NV == 3 ? 2 : 16, NV == 3 ? 1 : 8, NV == 3 ? 16 : 4, NV == 3 ? 8 : 2, NV == 3 ? 4 : 1};
@@ -457,7 +447,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
             k.done = 1;
             k.status = 5;
           } else {
-            al = quotient(k.rz, pq, T(0));
+            al = T(k.rz / pq);
           }
           sal[w] = al;
         }
@@ -499,7 +489,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
           else if (rr <= k.tt) k.done = 1;
           else if (k.iter >= k.max_iter) { k.done = 1; k.status = 4; }
           else {
-            be = quotient(rzn, k.rz, T(0));
+            be = T(rzn / k.rz);
             k.rz = rzn;
           }
         }
