@@ -10,7 +10,9 @@
 // that needs it from the owners' residuals (distributed shared memory), S
 // kept in shared memory as far as it fits (16-bit columns into that window), partial
 // sums stored straight into every CTA, two hardware barriers an iteration
-// (about 500 cycles each).
+// (about 500 cycles each; a third one where some CTA has no window).  It takes the
+// problems for which it is the faster side (af_plan.hpp): dense systems beyond
+// the shared memories and points in an order that needs p from everywhere go to the loop.
 // A problem's arithmetic depends on its own rows only, so it keeps its bits
 // alone and in any batch; problems of a batch run side by side.
 // Bound: latency of the barriers and scalars at a few hundred rows (3.8 us an
@@ -20,13 +22,9 @@
 // 32x32x128 tube 25.4 -> 12.0 ms (of which the reductions alone gave a third).
 #pragma once
 
-namespace ibg {
+#include "af_plan.hpp"
 
-constexpr int AFC_THREADS = 1024;
-constexpr int AFC_RPT = 2;                  // rows per thread at most (x stays in registers)
-constexpr int AFC_UNITS = 128;              // 32-row units of a problem that exchanges their sums
-constexpr int AFC_MAX = 16;                 // CTAs per cluster at most
-constexpr int AFC_SMEM = 218 * 1024;        // dynamic shared memory asked for (with the static part below 227 KB)
+namespace ibg {
 
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t smem, uint32_t rank) {
   uint32_t a;
@@ -82,21 +80,6 @@ __device__ __forceinline__ double lanes_sum(double x, int width) {
   return x;
 }
 
-// bytes of shared memory per row: p (four values), r with 1/diag, q and the row's first entry
-template <typename T>
-__host__ __device__ constexpr int afc_row_bytes() { return 11 * int(sizeof(T)) + 4; }
-// Padded rows of a problem that runs in clusters of cl CTAs.  FP32: up to where
-// the loop's launches cost the same (32,000 rows of 10 entries: 14 us an
-// iteration here, about 16 in the loop; 8160 rows of 41: 10 against 22).
-// FP64: while the FP64 rate of 16 SMs costs less than the loop's launches
-// (2000 rows of 40 entries 11.5 us against 25; 32,000 rows of 10 measured 80 against 50).
-template <typename T>
-__host__ __device__ constexpr int64_t afc_max_rows(int cl) { return int64_t(cl) * (sizeof(T) == 4 ? 2048 : 384); }
-static_assert(AFC_UNITS == 128, "16 blocks of 256 rows at most");
-static_assert(2048 <= AFC_THREADS * AFC_RPT, "x of a CTA's rows is kept in registers");
-template <typename T>
-__host__ __device__ constexpr bool afc_fits(int64_t n, int cl) { return cl > 0 && n <= afc_max_rows<T>(cl); }
-
 using three = std::integral_constant<int, 3>;
 using six = std::integral_constant<int, 6>;
 
@@ -117,15 +100,12 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   const int inst = blockIdx.x / cl;
   const int64_t R0 = int64_t(ib.seg_t[inst]) * 256;
   const int n = (ib.seg_t[inst + 1] - ib.seg_t[inst]) * 256;   // whole blocks of 256 rows
-  // uniform over the cluster: nothing to do, or too large for a cluster
-  if (n == 0 || !afc_fits<T>(n, cl) || (ks[3 * inst].done && ks[3 * inst + 1].done && ks[3 * inst + 2].done)) return;
+  // uniform over the cluster: nothing to do, or a problem of the loop's
+  if (!(ib.af_route[inst] & (sizeof(T) == 4 ? AF_CLUSTER32 : AF_CLUSTER64)) || (ks[3 * inst].done && ks[3 * inst + 1].done && ks[3 * inst + 2].done)) return;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  // rows per CTA: FP32 whole units of 32 rows where the problem's units fit the
-  // exchange, else whole blocks of 256 (so that a CTA holds whole blocks
-  // of the sums); FP64 units of 32
-  const bool units = sizeof(T) == 4 && n <= 32 * AFC_UNITS;
-  const int gran = sizeof(T) == 8 || units ? 32 : 256;
-  const int rper = (n / gran + int(cl) - 1) / int(cl) * gran;
+  const AfcShape sh = afc_shape<T>(n, int(cl));
+  const bool units = sh.units;
+  const int rper = sh.rper, ubytes = sh.ubytes;
   const int rpc = max(0, min(n - int(rank) * rper, rper));   // rows of this CTA
   const int64_t row0 = R0 + int64_t(rank) * rper;
   const int e0 = rpc ? ib.rowptr[row0] : 0, ne = rpc ? ib.rowptr[row0 + rpc] - e0 : 0;
@@ -152,9 +132,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   }
   __syncthreads();
   const int own0 = min(int(rank) * rper, n);   // the problem's row of the CTA's first one
-  const int ubytes = units ? 12 * (n / 32) * int(sizeof(T)) : 0;
-  const int room = AFC_SMEM - 64 - ubytes - rper * afc_row_bytes<T>();
-  const bool fast = win <= room / int(16 * sizeof(T));   // the window takes half the room at most
+  const bool fast = win <= sh.window;
   const int G = fast ? win : 0;
   const int w0 = max(0, own0 - G), wn = min(n, own0 + rpc + G) - w0;   // window: rows [w0, w0 + wn) of the problem
   // in place of part: the sums of every 32 rows of the problem, [2][6][n / 32]
@@ -164,7 +142,7 @@ __global__ void __launch_bounds__(AFC_THREADS, 1)
   T* p = pw + 4 * (own0 - w0);
   T* q = pw + 4 * wn;                      // [rpc][3]
   T* cv = q + 3 * rpc;                     // cached values of S ...
-  const int cap = fast ? min(ne, (room - (wn - rpc) * int(4 * sizeof(T))) / int(sizeof(T) + 2) / 2 * 2) : 0;
+  const int cap = fast ? min(ne, afc_cached<T>(sh, wn - rpc)) : 0;
   const int capr = (cap + 1) / 2 * 2;      // (an even number of 16-bit places)
   uint16_t* cc = reinterpret_cast<uint16_t*>(cv + capr);   // ... and their columns' places in the window
   int* rp = reinterpret_cast<int*>(cc + capr);             // [rpc + 1] entries relative to e0

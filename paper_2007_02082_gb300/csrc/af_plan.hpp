@@ -1,0 +1,114 @@
+// Layout of the force solve by a thread-block cluster (af_cluster.cuh) and the
+// rule that gives a problem to it or to the loop of launches.  Plain C++, so that
+// the host decides at set-up with the numbers that the kernel uses.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+
+#if defined(__CUDACC__)
+#define AFC_HD __host__ __device__
+#else
+#define AFC_HD
+#endif
+
+namespace ibg {
+
+constexpr int AFC_THREADS = 1024;
+constexpr int AFC_RPT = 2;                  // rows per thread at most (x stays in registers)
+constexpr int AFC_UNITS = 128;              // 32-row units of a problem that exchanges their sums
+constexpr int AFC_MAX = 16;                 // CTAs per cluster at most
+constexpr int AFC_SMEM = 218 * 1024;        // dynamic shared memory asked for (with the static part below 227 KB)
+static_assert(AFC_UNITS == 128, "16 blocks of 256 rows at most");
+
+// bytes of shared memory per row: p (four values), r with 1/diag, q and the row's first entry
+template <typename T>
+AFC_HD constexpr int afc_row_bytes() { return 11 * int(sizeof(T)) + 4; }
+
+// Padded rows of a problem that a cluster of cl CTAs takes at most.
+template <typename T>
+AFC_HD constexpr int64_t afc_max_rows(int cl) { return int64_t(cl) * (sizeof(T) == 4 ? 2048 : 384); }
+static_assert(2048 <= AFC_THREADS * AFC_RPT, "x of a CTA's rows is kept in registers");
+
+// How the n rows (whole blocks of 256) of a problem lie in a cluster of cl CTAs.
+// Rows per CTA: FP32 whole units of 32 rows where the problem's units fit the
+// exchange, else whole blocks of 256 (so that a CTA holds whole blocks
+// of the sums); FP64 units of 32.
+struct AfcShape {
+  bool units;   // every 32 rows' sums are exchanged
+  int rper;     // rows per CTA (fewer in the last ones)
+  int ubytes;   // shared memory of the units' sums
+  int room;     // shared memory left for the others' p and the cached part of S
+  int window;   // the others' rows a CTA may need on either side to keep a window of p: half the room at most
+};
+template <typename T>
+AFC_HD constexpr AfcShape afc_shape(int n, int cl) {
+  const bool units = sizeof(T) == 4 && n <= 32 * AFC_UNITS;
+  const int gran = sizeof(T) == 8 || units ? 32 : 256;
+  const int rper = (n / gran + cl - 1) / cl * gran;
+  const int ubytes = units ? 12 * (n / 32) * int(sizeof(T)) : 0;
+  const int room = AFC_SMEM - 64 - ubytes - rper * afc_row_bytes<T>();
+  return AfcShape{units, rper, ubytes, room, room / int(16 * sizeof(T))};
+}
+// Entries of S a CTA keeps beside a window of `others` rows.
+template <typename T>
+AFC_HD constexpr int afc_cached(const AfcShape& s, int others) {
+  return (s.room - others * int(4 * sizeof(T))) / int(sizeof(T) + 2) / 2 * 2;
+}
+
+// The first and last column of every row of a problem (row and column 0: the problem's first row).
+struct AfcRows {
+  const int32_t* rowptr;   // [n + 1], any base
+  const int32_t *lo, *hi;  // [n] columns; lo > hi: no entries
+};
+
+// Time of an iteration in nanoseconds as measured, of the slowest CTA.  A cluster
+// pays for its barriers and scalars, for rows, for entries in shared memory, for
+// entries that did not fit (read again every iteration by 16 SMs) and, where a
+// CTA's columns reach too far for a window (points that are not listed
+// along the wall), for reading every p from its owner.  The loop of launches uses the
+// whole GPU and pays for its launches; beyond some rows also for rows.
+// Measured, FP32, us an iteration, cluster against loop.  Points along the wall, 34
+// entries a row: 8160 rows 9.6 / 18.8, 12,000 12.0 / 19.0, 16,000 18.5 / 19.0, 20,000 23.2 /
+// 21.5, 32,000 37.2 / 25.5; 9 entries a row: 32,000 13.8 / 22.0.  Points in random order, 34
+// entries: 2000 6.6 / 19.5, 4000 29 / 20, 8160 86 / 21, 32,000 255 / 32.
+// FP64, 34 entries: 2000 rows 11.5 / 23.9, 6000 24.6 / 28.4; random order 2000 25.5 / 24.4, 6000 95 / 29.
+template <typename T>
+inline double afc_cluster_ns(const AfcRows& a, int n, int cl) {
+  constexpr bool f32 = sizeof(T) == 4;
+  constexpr double base = f32 ? 4600 : 5100, row = f32 ? 2.4 : 11.4, hit = f32 ? 0.21 : 1.18,
+                   miss = f32 ? 0.55 : 2.0, far = f32 ? 4.0 : 6.0;
+  const AfcShape s = afc_shape<T>(n, cl);
+  double worst = 0.0;
+  for (int r0 = 0; r0 < n; r0 += s.rper) {
+    const int r1 = std::min(n, r0 + s.rper);
+    int lo = r0, hi = r1 - 1;
+    for (int i = r0; i < r1; ++i)
+      if (a.lo[i] <= a.hi[i]) lo = std::min(lo, a.lo[i]), hi = std::max(hi, a.hi[i]);
+    const int need = std::max(r0 - lo, hi - r1 + 1), ne = a.rowptr[r1] - a.rowptr[r0];
+    double t = base + row * s.rper;
+    if (need <= s.window) {
+      const int others = std::min(n, r1 + need) - std::max(0, r0 - need) - (r1 - r0);
+      const int cap = std::min(ne, afc_cached<T>(s, others));
+      t += hit * cap + miss * (ne - cap);
+    } else {
+      t += far * ne;
+    }
+    worst = std::max(worst, t);
+  }
+  return worst;
+}
+template <typename T>
+inline double afc_loop_ns(int n) {
+  return sizeof(T) == 4 ? 18500 + 0.3 * std::max(0, n - 16000) : 22500 + 0.5 * std::max(0, n - 4500);
+}
+
+// Whether a cluster solves the problem.  By the problem's own rows and the
+// device's cluster size alone, so that its bits do not depend on the batch it runs
+// in; after a move of the points the choice stays (any S is solved right either way).
+template <typename T>
+inline bool afc_takes(const AfcRows& a, int n, int cl) {
+  return cl > 0 && n > 0 && n <= afc_max_rows<T>(cl) && afc_cluster_ns<T>(a, n, cl) <= afc_loop_ns<T>(n);
+}
+
+}  // namespace ibg

@@ -855,7 +855,13 @@ ib_status engine_build(Engine& E) {
   ib.sp_slot = d_sps; ib.sp_off = d_spo; ib.sp_ent = d_spe; ib.n_sp = int64_t(sps.size());
   ib.pinst = d_pinst; ib.seg_t = d_segt; ib.seg_w = d_segw; ib.seg_g = d_segg; ib.pscale = d_pscale;
   ib.iorigin = d_iorg; ib.ihf = d_ihf; ib.icoef = d_icoef; ib.binst = d_binst;
-  if (Mt) ib_choose_solver(ib, segt.data());
+  if (Mt) {
+    std::vector<uint8_t> route(n);
+    ib_choose_solver(ib, segt.data(), rowptr.data(), col.data(), E.mixed, route.data());
+    uint8_t* d_route;
+    TRY(upload(E, &d_route, route));
+    ib.af_route = d_route;
+  }
   TRY(dalloc(E, &ib.W, 64 * Mt, true));
   TRY(dalloc(E, &ib.val, int64_t(col.size()), true));
   E.af_cap = int64_t(col.size());

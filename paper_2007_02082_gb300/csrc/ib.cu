@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <vector>
 
 #include "async.cuh"
 #include "ib.hpp"
@@ -348,18 +349,34 @@ static int afc_cluster_size() {
   return 0;
 }
 
-void ib_choose_solver(IBDev& ib, const int32_t* seg_t) {
-  ib.af_cl32 = afc_cluster_size<float>();
-  ib.af_cl64 = afc_cluster_size<double>();
+void ib_choose_solver(IBDev& ib, const int32_t* seg_t, const int32_t* rowptr, const int32_t* col, bool mixed,
+                      uint8_t* route) {
+  const int cl32 = mixed ? afc_cluster_size<float>() : 0, cl64 = afc_cluster_size<double>();
+  ib.af_cl32 = ib.af_cl64 = 0;
   ib.af_big32 = ib.af_big64 = false;
-  for (int n = 0; n < ib.ninst; ++n) {
-    const int64_t rows = int64_t(seg_t[n + 1] - seg_t[n]) * 256;
-    if (!afc_fits<float>(rows, ib.af_cl32)) ib.af_big32 = true;
-    if (!afc_fits<double>(rows, ib.af_cl64)) ib.af_big64 = true;
+  std::vector<int32_t> lo, hi;
+  for (int i = 0; i < ib.ninst; ++i) {
+    const int64_t r0 = int64_t(seg_t[i]) * 256;
+    const int n = (seg_t[i + 1] - seg_t[i]) * 256;
+    route[i] = 0;
+    if (n == 0) continue;
+    lo.assign(n, 1);
+    hi.assign(n, 0);
+    for (int r = 0; r < n && n <= afc_max_rows<float>(AFC_MAX); ++r)
+      if (rowptr[r0 + r] < rowptr[r0 + r + 1]) {
+        const auto e = std::minmax_element(col + rowptr[r0 + r], col + rowptr[r0 + r + 1]);
+        lo[r] = int32_t(*e.first - r0);
+        hi[r] = int32_t(*e.second - r0);
+      }
+    const AfcRows a{rowptr + r0, lo.data(), hi.data()};
+    if (afc_takes<float>(a, n, cl32)) route[i] |= AF_CLUSTER32, ib.af_cl32 = cl32;
+    else ib.af_big32 = true;
+    if (afc_takes<double>(a, n, cl64)) route[i] |= AF_CLUSTER64, ib.af_cl64 = cl64;
+    else ib.af_big64 = true;
   }
 }
 
-// the cluster solve of every problem that fits; x: the iterate (updated), r: its residual
+// the cluster solve of every problem routed to it; x: the iterate (updated), r: its residual
 template <typename T>
 static void af_cluster_solve(const IBDev& ib, int cl, const T* val, const T* dinv, T* x, const T* r, KState* ks,
                              cudaStream_t st) {
@@ -400,7 +417,7 @@ cudaError_t ib_solve(const IBDev& ib, const double* BF, double* G, double* work,
   IBG_LAUNCH((k_af_start<double>), gt, IBB, 0, st, ib, ib.dinv, BF, (const double*)q, r, z, p, ks, rb.partials,
              rb.counter, cond, (const OState*)nullptr);
   if (cluster) af_cluster_solve<double>(ib, ib.af_cl64, ib.val, ib.dinv, G, r, ks, st);
-  // the problems too large for a cluster (the others are done by now):
+  // the other problems (those are done by now):
   // k_af_start left p = z and beta = 0; the direction ping-pongs between p and
   // p2, two iterations per loop body
   double* p2 = work + 4 * L;
@@ -523,7 +540,7 @@ cudaError_t ib_solve_mixed(const IBDev& ib, const double* BF, double* G, double*
       IBG_LAUNCH((k_af_update<float>), gt, IBB, 0, s2, ib, (const float*)ib.dinv32, e32, r, z, (const float*)pnew,
                  (const float*)q, ks, rb.partials, rb.counter, c2);
     };
-    if (ib.af_big32) {   // the problems too large for a cluster
+    if (ib.af_big32) {   // the other problems
       cudaError_t e = run_loop(cc, s, ci, ks, ks_host, ib.ninst * 3, max_iter, 4, 32,
                                [&](cudaStream_t s2, const Cond& c2) {
         iter(s2, c2, pa, pb);

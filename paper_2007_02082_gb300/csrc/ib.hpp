@@ -46,14 +46,19 @@ struct IBDev {
   const int32_t* n_sp_dev = nullptr;
   int64_t sp_cap = 0;
   // force solve (ib_choose_solver): CTAs of the cluster that solves a problem
-  // in one launch (0: no clusters) and whether some problem is too large for one
-  // and takes the launch-per-pass loop, in FP32 and FP64
+  // in one launch (0: no problem is solved so), the problems that are ([ninst], AF_CLUSTER
+  // bits), and whether some problem takes the launch-per-pass loop, in FP32 and FP64
   int32_t af_cl32 = 0, af_cl64 = 0;
+  const uint8_t* af_route = nullptr;
   bool af_big32 = true, af_big64 = true;
 };
+enum : uint8_t { AF_CLUSTER32 = 1, AF_CLUSTER64 = 2 };
 
-// Choose each problem's force solver by its padded row count (seg_t, host copy).
-void ib_choose_solver(IBDev& ib, const int32_t* seg_t);
+// Choose each problem's force solver (af_plan.hpp) from host copies of seg_t,
+// rowptr and col: route takes the AF_CLUSTER bits of the ninst problems, for the caller
+// to upload to ib.af_route.  Without mixed no FP32 solve is planned.
+void ib_choose_solver(IBDev& ib, const int32_t* seg_t, const int32_t* rowptr, const int32_t* col, bool mixed,
+                      uint8_t* route);
 
 // Eq. 17-18: W[i][a] = phi((x_a - X_i)/hx) phi((y_a - Y_i)/hy) phi((z_a - Z_i)/hz).
 void ib_weights(const IBDev& ib, cudaStream_t st);

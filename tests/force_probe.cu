@@ -86,11 +86,14 @@ int main(int argc, char** argv) {
   ib.dinv = put(dinv);
   ib.val32 = put(std::vector<float>(val.begin(), val.end()));
   ib.dinv32 = put(std::vector<float>(dinv.begin(), dinv.end()));
-  ib_choose_solver(ib, st.data());
+  std::vector<uint8_t> route(n);
+  ib_choose_solver(ib, st.data(), rowptr.data(), col.data(), mixed, route.data());
   if (head[2] >= 0) {
     ib.af_cl32 = ib.af_cl64 = int32_t(head[2]);
     ib.af_big32 = ib.af_big64 = head[2] == 0;
+    for (uint8_t& v : route) v = head[2] ? AF_CLUSTER32 | AF_CLUSTER64 : 0;
   }
+  ib.af_route = put(route);
   RedBuf rb;
   rb.partials = put(std::vector<double>(2 * (M / 8 + 1) * 16 + n * 16 + 64));
   rb.counter = put(std::vector<unsigned>(M / 8 + 2));

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import scipy.sparse as sp
 
+import workloads as W
 from tests import force_system as F
 
 pytestmark = pytest.mark.gpu
@@ -75,3 +76,44 @@ def test_cluster_and_loop_agree(probe, tmp_path, M, spacing, shuffled, cluster, 
         assert np.array_equal(a, l)
     tol = 22e-5 + 6e-5 if mixed else 22e-12
     assert np.all(np.linalg.norm(a - l, axis=0) <= tol * np.linalg.norm(l, axis=0))
+
+
+@pytest.mark.parametrize("mixed", [1, 0])
+def test_library_routes_problems_of_a_batch_apart(probe, tmp_path, mixed):
+    """A problem of the loop's (points in random order) between two of the clusters':
+    the library's choice gives each the bits it has alone."""
+    systems = [F.system(F.tube_points(M, 1.6, R, shuffled=s), shift=0.1)
+               for M, R, s in ((700, 13, False), (8160, 25, True), (2000, 13, False))]
+    bs = [np.random.default_rng(S.shape[0]).normal(size=(S.shape[0], 3)) for S in systems]
+    kw = dict(rtol=1e-12 if not mixed else 0.0, rtol_inner=1e-5)
+    head, G, _ = F.solve(probe, tmp_path, systems, bs, mixed, -1, **kw)
+    for i, (S, b) in enumerate(zip(systems, bs)):
+        ha, (a,), _ = F.solve(probe, tmp_path, [S], [b], mixed, 0 if i == 1 else 16, **kw)
+        assert np.array_equal(head[i, :3], ha[0, :3]) and np.array_equal(G[i], a), i
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_batch_with_a_loop_member(precision):
+    """Steps of a batch whose second member's force system goes to the loop (8160
+    points in random order) and the others' to clusters: each member as alone."""
+    from paper_2007_02082_gb300 import IBBatch, IBGrid
+    mid = W.cylinder_case(n=(32, 32, 128), M=8160, seed=92, nu=0.05, dt=0.005)
+    k = np.random.default_rng(5).permutation(len(mid["X"]))
+    mid["X"], mid["dS"], mid["UB"] = (np.ascontiguousarray(mid[f][k]) for f in ("X", "dS", "UB"))
+    cases = [W.cylinder_case(n=(8, 8, 16), length=2.0, M=270, seed=91, nu=0.1, dt=0.01), mid,
+             W.cylinder_refined_small(n=(16, 16, 20), seed=93)]
+    alone = []
+    for c in cases:
+        g = IBGrid(c, precision=precision)
+        g.ipcs_step(2)
+        alone.append([g.ib_fields_get(f) for f in ("U", "P", "F_LAG")])
+        g.close()
+    mem = [IBGrid(c, precision=precision, deferred=True) for c in cases]
+    b = IBBatch(mem)
+    assert np.all(b.step(2) == 0)
+    for i, m in enumerate(mem):
+        for f, ref in zip(("U", "P", "F_LAG"), alone[i]):
+            assert np.array_equal(m.ib_fields_get(f), ref), (i, f)
+    b.close()
+    for m in mem:
+        m.close()
