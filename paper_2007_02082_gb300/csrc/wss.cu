@@ -63,25 +63,27 @@ __device__ __forceinline__ bool selected(const MoveGrid& G, const double* X, con
 // lanes of the warp (every lane takes part, valid or not); returns their number.
 // queue: 64 entries of the warp.
 template <typename Body>
-__device__ __forceinline__ int for_nodes(const MoveGrid& G, const double* X, const double* np_, double rc2,
+__device__ __forceinline__ int for_nodes(const MoveGrid& G, const double* X, const double* np_, double rc2, double inv,
                                          const int32_t (&rad)[3], int2* queue, Body&& body) {
   const int lane = threadIdx.x & 31;
   Box box;
   float f[3], h[3], nf[3];
   int32_t c[3];
   double nmax = fmax(fabs(np_[0]), fmax(fabs(np_[1]), fabs(np_[2])));
-  // normals that FP32 cannot scale are left to the exact test
+  // the FP32 test is in units of the largest spacing (inv is its reciprocal), so
+  // that no length of a problem leaves the FP32 range; normals that FP32
+  // cannot scale are left to the exact test
   const bool plain = nmax > 0.0 && isfinite(np_[0]) && isfinite(np_[1]) && isfinite(np_[2]);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     c[a] = int32_t(floor((X[a] - G.origin[a]) / G.hf[a]));
     box.lo[a] = max(c[a] - rad[a], 0);
     box.n[a] = max(0, min(c[a] + 1 + rad[a], int32_t(G.nf[a])) - box.lo[a] + 1);
-    f[a] = float(X[a] - (G.origin[a] + double(c[a]) * G.hf[a]));
-    h[a] = float(G.hf[a]);
+    f[a] = float((X[a] - (G.origin[a] + double(c[a]) * G.hf[a])) * inv);
+    h[a] = float(G.hf[a] * inv);
     nf[a] = plain ? float(np_[a] / nmax) : 0.f;
   }
-  const float r2max = float(rc2) * 1.001f, dmax = 1e-3f * sqrtf(float(rc2));
+  constexpr float r2max = float(WSS_RADIUS * WSS_RADIUS * 1.001), dmax = float(1e-3 * WSS_RADIUS);
   const int n = box.n[0] * box.n[1] * box.n[2];
   int kept = 0, in = 0;   // nodes of the queue (uniform over the warp)
   auto flush = [&](int m) {
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(32 * WSS_WARPS)
     double m[32], b[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) m[j] = b[j] = 0.0;
-    const int n = for_nodes(G, X + 3 * (p0 + k), nrm + 3 * (p0 + k), rc2, rad, queue[w],
+    const int n = for_nodes(G, X + 3 * (p0 + k), nrm + 3 * (p0 + k), rc2, inv, rad, queue[w],
                             [&](bool ok, int32_t s, const double (&d)[3]) {
       if (!ok) return;
       const double x = d[0] * inv, y = d[1] * inv, z = d[2] * inv;
