@@ -61,7 +61,7 @@ cudaError_t fe_init_tables() {
   if ((e = cudaMemcpyToSymbol(c_sten, h_sten, sizeof(h_sten))) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_toff, toff, sizeof(toff))) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_slot_of_rel, slot_of_rel, sizeof(slot_of_rel))) != cudaSuccess) return e;
-  std::vector<uint4> tw(256 * 15);
+  uint4 tw[256 * 15];   // 60 KB of stack: a C entry calls this, so nothing here may throw
   unsigned long long mw[256];
   for (int mk = 0; mk < 256; ++mk) {
     for (int k = 0; k < 15; ++k) {
@@ -73,7 +73,7 @@ cudaError_t fe_init_tables() {
     mw[mk] = (unsigned long long)(mass_weight(mk, 0) / 2) << 56;
     for (int k = 1; k < 15; ++k) mw[mk] |= (unsigned long long)mass_weight(mk, k) << (4 * k - 4);
   }
-  if ((e = cudaMemcpyToSymbol(g_transw, tw.data(), tw.size() * sizeof(uint4))) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(g_transw, tw, sizeof(tw))) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(g_massw, mw, sizeof(mw))) != cudaSuccess) return e;
   return cudaSuccess;
 }
