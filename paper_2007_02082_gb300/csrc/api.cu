@@ -766,6 +766,7 @@ ib_status engine_build(Engine& E) {
     TRY(upload(E, &d_poff, poff));
     P7Hdr* d_phdr;
     TRY(upload(E, &d_phdr, phdr));
+    g.sms = nsm;
     g.p7_ctas = G;
     g.p7_off = d_poff;
     g.p7_hdr = reinterpret_cast<const int4*>(d_phdr);

@@ -162,6 +162,7 @@ struct DevGrid {
   int32_t p7_ctas;
   const int32_t* __restrict__ p7_off;   // [p7_ctas + 1]
   const int4* __restrict__ p7_hdr;      // [nbricks][4]
+  int32_t sms;                          // SMs of the device
 };
 
 // Per brick of the persistent Poisson schedule: the brick, its face neighbours

@@ -1507,10 +1507,10 @@ int fe_p7_ctas_per_sm() {
 // the chunks are fewer than two CTAs per SM a CTA's walk through its bricks is the
 // kernel's time (8x8x16 tube, 2 chunks: sweep 4.6 -> 2.4 us); beyond that the parts'
 // own start (tables, ring fill) costs more than the shorter walk gives
-// (312 chunks in four parts: 8.6 -> 9.9 us).
+// (312 chunks in four parts on 152 SMs: 8.6 -> 9.9 us).
 static int p7_split(const DevGrid& g) {
   int s = 1;
-  while (s < P7_CHUNK && int64_t(g.nchunks) * s * 2 <= 152 * 2) s *= 2;
+  while (s < P7_CHUNK && int64_t(g.nchunks) * s * 2 <= 2 * int64_t(g.sms)) s *= 2;
   return s;
 }
 
