@@ -1931,20 +1931,16 @@ void fe_poisson_apply(const DevGrid& g, const T* x, T* q, uint16_t dmask, KState
 
 // The fused sweep is an instance of the staged kernel: FP32 on 16-byte
 // boundaries, not under the launch choices of the other two stencil kernels.
-template <typename T>
-bool fe_poisson_smooths(const DevGrid& g, const T* z, const T* zout, const T* r, const T* dinv) {
+bool fe_poisson_smooths(const DevGrid& g, const float* z, const float* zout, const float* r, const float* dinv) {
   auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  return sizeof(T) == 4 && g.poisson_kernel <= 1 && a16(z) && a16(zout) && a16(r) && a16(dinv);
+  return g.poisson_kernel <= 1 && a16(z) && a16(zout) && a16(r) && a16(dinv);
 }
 
-template <typename T>
-void fe_poisson_smooth(const DevGrid& g, const T* z, T* zout, const T* r, T* q, const T* dinv, T omega,
-                       uint16_t dmask, KState* ks, const uint8_t* on, cudaStream_t st) {
-  if constexpr (sizeof(T) == 4) {
-    const int split = p7_split(g);
-    IBG_LAUNCH((k_poisson7_staged<false, true>), g.nchunks * split, P7_THREADS, (p7_smem<1, 2>()), st, g, z, r, zout, q,
-               dmask, ks, (double*)nullptr, (unsigned*)nullptr, on, dinv, omega, split);
-  }
+void fe_poisson_smooth(const DevGrid& g, const float* z, float* zout, const float* r, float* q, const float* dinv,
+                       float omega, uint16_t dmask, KState* ks, const uint8_t* on, cudaStream_t st) {
+  const int split = p7_split(g);
+  IBG_LAUNCH((k_poisson7_staged<false, true>), g.nchunks * split, P7_THREADS, (p7_smem<1, 2>()), st, g, z, r, zout, q,
+             dmask, ks, (double*)nullptr, (unsigned*)nullptr, on, dinv, omega, split);
 }
 
 template <typename T>
@@ -2098,12 +2094,6 @@ template void fe_apply_local<double>(const DevGrid&, const OpDesc<double>&, int,
                                      cudaStream_t);
 template void fe_poisson_apply<float>(const DevGrid&, const float*, float*, uint16_t, KState*, const uint8_t*,
                                       cudaStream_t);
-template bool fe_poisson_smooths<float>(const DevGrid&, const float*, const float*, const float*, const float*);
-template bool fe_poisson_smooths<double>(const DevGrid&, const double*, const double*, const double*, const double*);
-template void fe_poisson_smooth<float>(const DevGrid&, const float*, float*, const float*, float*, const float*, float,
-                                      uint16_t, KState*, const uint8_t*, cudaStream_t);
-template void fe_poisson_smooth<double>(const DevGrid&, const double*, double*, const double*, double*,
-                                       const double*, double, uint16_t, KState*, const uint8_t*, cudaStream_t);
 template void fe_poisson_apply<double>(const DevGrid&, const double*, double*, uint16_t, KState*, const uint8_t*,
                                        cudaStream_t);
 template void fe_sync<double>(const DevGrid&, int, double*, uint16_t, cudaStream_t);

@@ -98,11 +98,9 @@ void fe_poisson_apply(const DevGrid& g, const T* x, T* q, uint16_t dmask, KState
 // One damped-Jacobi sweep zout = z + omega D^-1 (r - K z) in one pass over the
 // chunks, interface nodes excepted: q holds the level's part of K z at interface and
 // hanging nodes for their own kernel.  Only where fe_poisson_smooths says so.
-template <typename T>
-bool fe_poisson_smooths(const DevGrid& g, const T* z, const T* zout, const T* r, const T* dinv);
-template <typename T>
-void fe_poisson_smooth(const DevGrid& g, const T* z, T* zout, const T* r, T* q, const T* dinv, T omega,
-                       uint16_t dmask, KState* ks, const uint8_t* on, cudaStream_t st);
+bool fe_poisson_smooths(const DevGrid& g, const float* z, const float* zout, const float* r, const float* dinv);
+void fe_poisson_smooth(const DevGrid& g, const float* z, float* zout, const float* r, float* q, const float* dinv,
+                       float omega, uint16_t dmask, KState* ks, const uint8_t* on, cudaStream_t st);
 
 // Hanging nodes take the mean of their parents (nc components; x2 optional).
 template <typename T>

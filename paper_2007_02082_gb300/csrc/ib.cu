@@ -116,31 +116,16 @@ __device__ __forceinline__ void spmv_row(int64_t i, int lane, const int32_t* __r
     for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
 }
 
-// q = S p; p.q -> alpha (mode 1) | y = S x (mode 0).  Warp per row, 8 rows per block.
-__global__ void __launch_bounds__(IBB) k_af_apply(IBDev ib, const double* __restrict__ p, double* __restrict__ q,
-                                                  int mode, KState* ks, double* partials, unsigned* counter) {
+// y = S x.  Warp per row, 8 rows per block.
+__global__ void __launch_bounds__(IBB) k_af_apply(IBDev ib, const double* __restrict__ x, double* __restrict__ y) {
   KCOUNT();
   const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  double acc[3] = {0, 0, 0};
-  if (i < ib.M) spmv_row(i, lane, ib.rowptr, ib.col, ib.val, p, acc);
-  double v[3] = {0, 0, 0};
-  if (i < ib.M && lane == 0)
-    for (int c = 0; c < 3; ++c) {
-      q[3 * i + c] = acc[c];
-      v[c] = p[3 * i + c] * acc[c];
-    }
-  if (mode == 0) return;
-  double* out = partials + (int64_t)gridDim.x * 3;
-  if (!grid_sum_last<double, 3>(v, partials, counter, ib.seg_w, ib.ninst, ib.pinst[(int64_t)blockIdx.x * (IBB / 32)], out)) return;
-  for (int e = threadIdx.x; e < ib.ninst * 3; e += blockDim.x) {
-    KState& k = ks[e];
-    if (k.done) continue;
-    const double pq = out[e];
-    k.pq = pq;
-    if (!(pq > 0.0) || !isfinite(pq)) { k.done = 1; k.status = 5; k.alpha = 0.0; continue; }
-    k.alpha = k.rz / pq;
-  }
+  if (i >= ib.M) return;
+  double acc[3];
+  spmv_row(i, lane, ib.rowptr, ib.col, ib.val, x, acc);
+  if (lane == 0)
+    for (int c = 0; c < 3; ++c) y[3 * i + c] = acc[c];
 }
 
 // CG iteration form of the SpMV: p_new = z + beta p_old (read on the fly for
@@ -413,7 +398,7 @@ cudaError_t ib_solve(const IBDev& ib, const double* BF, double* G, double* work,
   }
   const int gw = int((ib.M * 32 + IBB - 1) / IBB);   // warp-per-row grids
   const int gt = int((ib.M + IBB - 1) / IBB);        // thread-per-row grids
-  IBG_LAUNCH(k_af_apply, gw, IBB, 0, st, ib, G, q, 0, ks, rb.partials, rb.counter);
+  IBG_LAUNCH(k_af_apply, gw, IBB, 0, st, ib, (const double*)G, q);
   IBG_LAUNCH((k_af_start<double>), gt, IBB, 0, st, ib, ib.dinv, BF, (const double*)q, r, z, p, ks, rb.partials,
              rb.counter, cond, (const OState*)nullptr);
   if (cluster) af_cluster_solve<double>(ib, ib.af_cl64, ib.val, ib.dinv, G, r, ks, st);
@@ -518,7 +503,7 @@ cudaError_t ib_solve_mixed(const IBDev& ib, const double* BF, double* G, double*
   const int gi = (ib.ninst + 127) / 128;
   IBG_LAUNCH(k_init_outer, gi, 128, 0, st, os, ib.ninst, 3, rtol * rtol, max_outer);
   auto residual = [&](cudaStream_t s, const Cond& cl, const Cond& cb) {
-    IBG_LAUNCH(k_af_apply, gw, IBB, 0, s, ib, (const double*)G, y64, 0, ks, rb.partials, rb.counter);
+    IBG_LAUNCH(k_af_apply, gw, IBB, 0, s, ib, (const double*)G, y64);
     IBG_LAUNCH(k_af_resid_outer, gt, IBB, 0, s, ib, BF, (const double*)y64, r32, e32, os, rb.partials, rb.counter,
                cl, cb);
   };

@@ -11,15 +11,14 @@
 namespace ibg {
 
 // Points of all instances, each instance's rows padded to a multiple of 256
-// (padding rows have no support and no A_F entries), so that both the
-// thread-per-row (256 rows per block) and warp-per-row (8 rows per block)
-// kernels have whole blocks per instance for segmented reductions.
+// (padding rows have no support and no A_F entries), so that the kernels with
+// 256 and with 32 rows per block have whole blocks per instance for segmented
+// reductions.
 struct IBDev {
   int64_t M;               // padded total
   int32_t ninst;
   const int32_t* pinst;    // [M] instance of each row
   const int32_t* seg_t;    // [ninst + 1] block range, 256 rows per block
-  const int32_t* seg_w;    // [ninst + 1] block range, 8 rows per block
   const int32_t* seg_g;    // [ninst + 1] block range, 32 rows per block
   const double* pscale;    // [M] dt / (rho h^3) of the row's instance
   float* val32 = nullptr;  // FP32 copies of val and dinv (mixed path)

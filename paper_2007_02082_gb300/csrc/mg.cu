@@ -152,10 +152,9 @@ __global__ void __launch_bounds__(512) k_mg_c_smooth(DevGrid g, const T* __restr
 
 // The same at interface nodes after the fused sweep (fe_poisson_smooth): K z is the
 // sum of both copies' parts and half of each hanging child's, as k_sync forms it.
-template <typename T>
-__global__ void k_mg_if_smooth(DevGrid g, const T* __restrict__ zin, T* __restrict__ zout, const T* __restrict__ r,
-                               const T* __restrict__ q, const T* __restrict__ dinv, uint16_t dmask,
-                               const uint8_t* __restrict__ on, T omega, const KState* ks) {
+__global__ void k_mg_if_smooth(DevGrid g, const float* __restrict__ zin, float* __restrict__ zout, const float* __restrict__ r,
+                               const float* __restrict__ q, const float* __restrict__ dinv, uint16_t dmask,
+                               const uint8_t* __restrict__ on, float omega, const KState* ks) {
   KCOUNT();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= g.n_if) return;
@@ -163,16 +162,16 @@ __global__ void k_mg_if_smooth(DevGrid g, const T* __restrict__ zin, T* __restri
   const int32_t k0 = g.if_off[e], k1 = g.if_off[e + 1];
   const int inst = g.binst[s[0] / DBV];
   const uint16_t m[2] = {g.meta[s[0]], g.meta[s[1]]};
-  T z[2], rv[2], d[2];
+  float z[2], rv[2], d[2];
 #pragma unroll
   for (int j = 0; j < 2; ++j) z[j] = zin[s[j]], rv[j] = r[s[j]], d[j] = dinv[s[j]];
-  T tot = q[s[0]] + q[s[1]];
-  for (int k = k0; k < k1; ++k) tot += T(0.5) * q[g.if_kid[k]];
-  if (m[0] & dmask) tot = T(0);
+  float tot = q[s[0]] + q[s[1]];
+  for (int k = k0; k < k1; ++k) tot += 0.5f * q[g.if_kid[k]];
+  if (m[0] & dmask) tot = 0.f;
   if (ks[inst].done || !on[inst]) return;
 #pragma unroll
   for (int j = 0; j < 2; ++j)
-    zout[s[j]] = keep_slot(m[j], dmask) ? T(z[j] + omega * d[j] * (rv[j] - tot)) : T(0);
+    zout[s[j]] = keep_slot(m[j], dmask) ? float(z[j] + omega * d[j] * (rv[j] - tot)) : 0.f;
 }
 
 // Composite <-> G0 transfers.  The weights are those of P1 interpolation on
@@ -820,12 +819,17 @@ void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T*
   // one sweep: the fused stencil and update, then its interface nodes; or (FP64, other
   // launch choices) the apply with its sums, then the update
   auto sweep = [&](const T* zin, T* zout) {
-    if (fe_poisson_smooths<T>(g, zin, zout, r, dinv)) {
-      timed(1, [&] { fe_poisson_smooth<T>(g, zin, zout, r, q, dinv, w, dmask, ksm, mg.on, st); });
-      if (g.n_if)
-        IBG_LAUNCH(k_mg_if_smooth<T>, (g.n_if + 255) / 256, 256, 0, st, g, zin, zout, r, (const T*)q, dinv, dmask, mg.on,
-                   w, ks);
-    } else {
+    bool fused = false;
+    if constexpr (sizeof(T) == 4) {
+      fused = fe_poisson_smooths(g, zin, zout, r, dinv);
+      if (fused) {
+        timed(1, [&] { fe_poisson_smooth(g, zin, zout, r, q, dinv, w, dmask, ksm, mg.on, st); });
+        if (g.n_if)
+          IBG_LAUNCH(k_mg_if_smooth, (g.n_if + 255) / 256, 256, 0, st, g, zin, zout, r, (const float*)q, dinv, dmask,
+                     mg.on, w, ks);
+      }
+    }
+    if (!fused) {
       apply(zin);
       timed(1, [&] {
         IBG_LAUNCH(k_mg_c_smooth<T>, g.nschunks, DBV, 0, st, g, zin, zout, r, q, dinv, dmask, mg.on, w, ks);

@@ -78,12 +78,6 @@ struct MGDev {
   bool any = false;                    // some problem uses multigrid
 };
 
-// z = B r: one symmetric V-cycle per problem with multigrid, z = D^-1 r for
-// the others.  r, z, zs, q are composite vectors (zs and q are scratch); dinv
-// the composite Jacobi inverse.  Problems whose KState is done are skipped.
-// z_started: the caller has left the first smoothing step, z = omega D^-1 r (D^-1 r
-// without multigrid; zero off the kept slots), in z.  With prof set, launches are timed by class: pcls + 0 the composite stencil
-// applies, pcls + 1 the composite smoothing updates, pcls + 2 the rest.
 // kernel attributes (shared memory), once per device
 cudaError_t mg_configure();
 // CTAs of the cooperative coarse-level kernel that fit on the device at once
@@ -91,6 +85,13 @@ cudaError_t mg_configure();
 template <typename T>
 int mg_levels_ctas();
 
+// z = B r: one symmetric V-cycle per problem with multigrid, z = D^-1 r for
+// the others.  r, z, zs, q are composite vectors (zs and q are scratch); dinv
+// the composite Jacobi inverse.  Problems whose KState is done are skipped.
+// z_started: the caller has left the first smoothing step, z = omega D^-1 r (D^-1 r
+// without multigrid; zero off the kept slots), in z.  With prof set, launches are
+// timed by class: pcls + 0 the composite stencil applies, pcls + 1 the composite
+// smoothing updates, pcls + 2 the rest.
 template <typename T>
 void mg_vcycle(const DevGrid& g, const MGDev<T>& mg, const T* r, T* z, T* zs, T* q, const T* dinv, uint16_t dmask,
                const KState* ks, cudaStream_t st, Prof* prof = nullptr, int pcls = 0, bool z_started = false);

@@ -57,11 +57,10 @@ int main(int argc, char** argv) {
   const bool mixed = head[1] != 0;
   const auto rows = take<int64_t>(f, n);
   int64_t M = 0;
-  std::vector<int32_t> st(1, 0), sw(1, 0), sg(1, 0), pinst;
+  std::vector<int32_t> st(1, 0), sg(1, 0), pinst;
   for (int i = 0; i < n; ++i) {
     M += rows[i];
     st.push_back(int32_t(M / 256));
-    sw.push_back(int32_t(M / 8));
     sg.push_back(int32_t(M / 32));
     pinst.resize(M, i);
   }
@@ -78,7 +77,6 @@ int main(int argc, char** argv) {
   ib.ninst = n;
   ib.pinst = put(pinst);
   ib.seg_t = put(st);
-  ib.seg_w = put(sw);
   ib.seg_g = put(sg);
   ib.rowptr = put(rowptr);
   ib.col = put(col);
@@ -95,8 +93,8 @@ int main(int argc, char** argv) {
   }
   ib.af_route = put(route);
   RedBuf rb;
-  rb.partials = put(std::vector<double>(2 * (M / 8 + 1) * 16 + n * 16 + 64));
-  rb.counter = put(std::vector<unsigned>(M / 8 + 2));
+  rb.partials = put(std::vector<double>(2 * (M / 32 + 1) * 16 + n * 16 + 64));
+  rb.counter = put(std::vector<unsigned>(M / 32 + 2));
   KState* ks = put(std::vector<KState>(3 * n));
   OState* os = put(std::vector<OState>(n));
   SolveRec* rec = put(std::vector<SolveRec>(4 * n));
