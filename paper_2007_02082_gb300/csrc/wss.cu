@@ -63,25 +63,26 @@ __device__ __forceinline__ bool selected(const MoveGrid& G, const double* X, con
 // lanes of the warp (every lane takes part, valid or not); returns their number.
 // queue: 64 entries of the warp.
 template <typename Body>
-__device__ __forceinline__ int for_nodes(const MoveGrid& G, const double* X, const double* np_, double rc2, double inv,
-                                         const int32_t (&rad)[3], int2* queue, Body&& body) {
+__device__ __forceinline__ int for_nodes(const MoveGrid& G, const double* X, const double* np_, double rc2,
+                                         const float (&h)[3], const int32_t (&rad)[3], int2* queue, Body&& body) {
   const int lane = threadIdx.x & 31;
   Box box;
-  float f[3], h[3], nf[3];
+  float f[3], nf[3];
   int32_t c[3];
   double nmax = fmax(fabs(np_[0]), fmax(fabs(np_[1]), fabs(np_[2])));
-  // the FP32 test is in units of the largest spacing (inv is its reciprocal), so
+  // the FP32 test is in units of the largest spacing (h: the spacings in them), so
   // that no length of a problem leaves the FP32 range; normals that FP32
   // cannot scale are left to the exact test
-  const bool plain = nmax > 0.0 && isfinite(np_[0]) && isfinite(np_[1]) && isfinite(np_[2]);
+  const bool plain = nmax >= 1e-300 && isfinite(np_[0]) && isfinite(np_[1]) && isfinite(np_[2]);
+  const double rn = 1.0 / nmax;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    c[a] = int32_t(floor((X[a] - G.origin[a]) / G.hf[a]));
+    const double x = (X[a] - G.origin[a]) / G.hf[a];
+    c[a] = int32_t(floor(x));
     box.lo[a] = max(c[a] - rad[a], 0);
     box.n[a] = max(0, min(c[a] + 1 + rad[a], int32_t(G.nf[a])) - box.lo[a] + 1);
-    f[a] = float((X[a] - (G.origin[a] + double(c[a]) * G.hf[a])) * inv);
-    h[a] = float(G.hf[a] * inv);
-    nf[a] = plain ? float(np_[a] / nmax) : 0.f;
+    f[a] = float(x - double(c[a])) * h[a];
+    nf[a] = plain ? float(np_[a] * rn) : 0.f;
   }
   constexpr float r2max = float(WSS_RADIUS * WSS_RADIUS * 1.001), dmax = float(1e-3 * WSS_RADIUS);
   const int n = box.n[0] * box.n[1] * box.n[2];
@@ -166,8 +167,8 @@ __device__ __forceinline__ double transpose_sum(double (&a)[32]) {
 __global__ void __launch_bounds__(32 * WSS_WARPS)
     k_wss(MoveGrid G, int64_t M, const double* __restrict__ X, const double* __restrict__ UB,
           const double* __restrict__ nrm, const double* __restrict__ u, int64_t ns, double eps, double rc2,
-          int32_t rx, int32_t ry, int32_t rz, double mu2, double* __restrict__ wss, double* __restrict__ grad,
-          int32_t* __restrict__ err) {
+          float hx, float hy, float hz, int32_t rx, int32_t ry, int32_t rz, double mu2, double* __restrict__ wss,
+          double* __restrict__ grad, int32_t* __restrict__ err) {
   KCOUNT();
   __shared__ double mom[WSS_PTS][33];       // sum_q w_q z_q^gamma of every point
   __shared__ double rhs[WSS_PTS][33];       // sum_q w_q P_r(z_q) (u_i(q) - U_B,i), at 9 i + r
@@ -177,13 +178,14 @@ __global__ void __launch_bounds__(32 * WSS_WARPS)
   const int64_t p0 = int64_t(blockIdx.x) * WSS_PTS;
   const int np = int(min(int64_t(WSS_PTS), M - p0));
   const int32_t rad[3] = {rx, ry, rz};
+  const float h[3] = {hx, hy, hz};
   const double inv = 1.0 / eps;
   for (int k = w; k < np; k += WSS_WARPS) {
     const double* ub = UB + 3 * (p0 + k);
     double m[32], b[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) m[j] = b[j] = 0.0;
-    const int n = for_nodes(G, X + 3 * (p0 + k), nrm + 3 * (p0 + k), rc2, inv, rad, queue[w],
+    const int n = for_nodes(G, X + 3 * (p0 + k), nrm + 3 * (p0 + k), rc2, h, rad, queue[w],
                             [&](bool ok, int32_t s, const double (&d)[3]) {
       if (!ok) return;
       const double x = d[0] * inv, y = d[1] * inv, z = d[2] * inv;
@@ -310,8 +312,9 @@ void wss_compute(const MoveGrid& G, const double hf[3], int64_t M, const double*
   const double rc = WSS_RADIUS * e;
   int32_t r[3];
   for (int a = 0; a < 3; ++a) r[a] = int32_t(std::ceil(rc / hf[a])) + 1;
-  IBG_LAUNCH(k_wss, unsigned((M + WSS_PTS - 1) / WSS_PTS), 32 * WSS_WARPS, 0, st, G, M, X, UB, nrm, u, ns, e, rc * rc, r[0], r[1], r[2],
-             2.0 * nu_rho, wss, grad, err);
+  IBG_LAUNCH(k_wss, unsigned((M + WSS_PTS - 1) / WSS_PTS), 32 * WSS_WARPS, 0, st, G, M, X, UB, nrm, u, ns, e, rc * rc,
+             float(hf[0] / e), float(hf[1] / e), float(hf[2] / e), r[0], r[1], r[2], 2.0 * nu_rho, wss,
+             grad, err);
 }
 
 }  // namespace ibg
