@@ -37,12 +37,11 @@ __constant__ int16_t c_toff[15];               // tile offset of each stencil sl
 __constant__ int8_t c_slot_of_rel[27];
 // Weights of every incident-cell mask for bodies with a run-time mask; the lanes
 // of a warp hold few different masks, so the rows stay in L1.
-// Transpose couplings, row [mask][k], byte 3 i + j (signed), for the FP64 momentum
+// Transpose couplings, row [mask][k] (trans_pack), for the FP64 momentum
 // operator of the symmetric form (33x33x131 tube: 288 -> 259 us; in FP32 the loads
 // cost more than forming the weights, 43 against 35 us)
 __device__ uint4 g_transw[256 * 15];
-// mass, off-diagonal weights 4 bits each (neighbour k at 4 (k - 1)), half the
-// diagonal weight in the top byte, for the FP32 operator (16 M-node sac: 238 -> 229 us)
+// mass (mass_pack), for the FP32 operator (16 M-node sac: 238 -> 229 us)
 __device__ unsigned long long g_massw[256];
 
 static const int8_t h_sten[15][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
@@ -64,14 +63,9 @@ cudaError_t fe_init_tables() {
   uint4 tw[256 * 15];   // 60 KB of stack: a C entry calls this, so nothing here may throw
   unsigned long long mw[256];
   for (int mk = 0; mk < 256; ++mk) {
-    for (int k = 0; k < 15; ++k) {
-      int8_t b[16] = {};
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) b[3 * i + j] = int8_t(trans_weight(mk, k, i, j));
-      std::memcpy(&tw[mk * 15 + k], b, 16);
-    }
-    mw[mk] = (unsigned long long)(mass_weight(mk, 0) / 2) << 56;
-    for (int k = 1; k < 15; ++k) mw[mk] |= (unsigned long long)mass_weight(mk, k) << (4 * k - 4);
+    for (int k = 0; k < 15; ++k)
+      tw[mk * 15 + k] = make_uint4(trans_pack(mk, k, 0), trans_pack(mk, k, 1), trans_pack(mk, k, 2), 0u);
+    mw[mk] = mass_pack(mk);
   }
   if ((e = cudaMemcpyToSymbol(g_transw, tw, sizeof(tw))) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(g_massw, mw, sizeof(mw))) != cudaSuccess) return e;
@@ -131,10 +125,6 @@ __device__ __forceinline__ constexpr bool const_mask() {
 // stencil factors.  xk(k, v) loads the three components at neighbour k.
 // (Couplings that are zero for every mask, 36 of 135, are left out of the run-time
 // body too: FP64 333 -> 288 us on the 33x33x131 tube.)
-__host__ __device__ constexpr bool trans_couples(int k, int i, int j) {   // some mask gives (k, i, j) a weight
-  constexpr int t[15] = {0x1ff, 0x0ef, 0x0ef, 0x0fe, 0x0fe, 0x1ee, 0x1ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee};
-  return (t[k] >> (3 * i + j)) & 1;
-}
 template <typename T, typename MK, typename XK>
 __device__ __forceinline__ void add_transpose(MK mk, const T* F, T dtnu, XK&& xk, T (&out)[3]) {
   T acc[3][3];
@@ -159,8 +149,7 @@ __device__ __forceinline__ void add_transpose(MK mk, const T* F, T dtnu, XK&& xk
           int w;
           if constexpr (sizeof(T) == 8) {
             const int e = 3 * i + j;
-            const unsigned word = e < 4 ? row.x : e < 8 ? row.y : row.z;
-            w = int((word >> (8 * (e & 3)) & 0xFFu) ^ 0x80u) - 128;
+            w = trans_unpack(e < 4 ? row.x : e < 8 ? row.y : row.z, e);
           } else {
             w = trans_weight(mk, k, i, j);
           }
@@ -1680,8 +1669,7 @@ __global__ void __launch_bounds__(512, (sizeof(T) == 4 && OP == OP_MASS && !PB) 
           for (int k = 0; k < 15; ++k) {
             T wk;
             if constexpr (sizeof(T) == 4 && !const_mask<decltype(mk)>())
-              wk = __uint_as_float(0x4B000000u | unsigned(k == 0 ? 2u * unsigned(mw >> 56)
-                                                                  : unsigned(mw >> (4 * k - 4)) & 15u)) - 8388608.f;
+              wk = __uint_as_float(0x4B000000u | mass_unpack(mw, k)) - 8388608.f;
             else
               wk = wconv<T>(mass_weight(mk, k));
             if constexpr (V4) {

@@ -235,4 +235,31 @@ IBG_HD int trans_weight(int mask, int k, int i, int j) {
   }
 }
 
+// Whether any mask gives the coupling (k, i, j) a weight: 99 of the 135 do.
+IBG_HD constexpr bool trans_couples(int k, int i, int j) {
+  constexpr int t[15] = {0x1ff, 0x0ef, 0x0ef, 0x0fe, 0x0fe, 0x1ee, 0x1ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee, 0x0ee};
+  return (t[k] >> (3 * i + j)) & 1;
+}
+
+// Tables by mask.  Mass: off-diagonal weights 4 bits each (neighbour k at 4 (k - 1)),
+// half the diagonal weight in the top byte.
+IBG_HD unsigned long long mass_pack(int mask) {
+  unsigned long long w = (unsigned long long)(mass_weight(mask, 0) / 2) << 56;
+  for (int k = 1; k < 15; ++k) w |= (unsigned long long)mass_weight(mask, k) << (4 * k - 4);
+  return w;
+}
+IBG_HD unsigned mass_unpack(unsigned long long w, int k) {
+  return k == 0 ? 2u * unsigned(w >> 56) : unsigned(w >> (4 * k - 4)) & 15u;
+}
+// Transpose couplings of one neighbour: byte 3 i + j (signed) of three words.
+IBG_HD unsigned trans_pack(int mask, int k, int word) {
+  unsigned w = 0;
+  for (int e = 4 * word; e < 4 * word + 4 && e < 9; ++e)
+    w |= (unsigned(trans_weight(mask, k, e / 3, e % 3)) & 0xFFu) << (8 * (e & 3));
+  return w;
+}
+IBG_HD int trans_unpack(unsigned word, int e) {   // word: the one that holds entry e
+  return int((word >> (8 * (e & 3)) & 0xFFu) ^ 0x80u) - 128;
+}
+
 }  // namespace ibg
