@@ -56,59 +56,62 @@ AFC_HD constexpr int afc_cached(const AfcShape& s, int others) {
   return (s.room - others * int(4 * sizeof(T))) / int(sizeof(T) + 2) / 2 * 2;
 }
 
-// The first and last column of every row of a problem (row and column 0: the problem's first row).
-struct AfcRows {
-  const int32_t* rowptr;   // [n + 1], any base
-  const int32_t *lo, *hi;  // [n] columns; lo > hi: no entries
-};
-
-// Time of an iteration in nanoseconds as measured, of the slowest CTA.  A cluster
-// pays for its barriers and scalars, for rows, for entries in shared memory, for
-// entries that did not fit (read again every iteration by 16 SMs) and, where a
-// CTA's columns reach too far for a window (points that are not listed
-// along the wall), for reading every p from its owner.  The loop of launches uses the
-// whole GPU and pays for its launches; beyond some rows also for rows.
+// Time of an iteration in picoseconds as measured (whole numbers: the same choice on
+// the host and on the device).  A cluster pays for its barriers and scalars, for rows,
+// for entries in shared memory, for entries that did not fit (read again every
+// iteration by 16 SMs) and, where a CTA's columns reach too far for a
+// window (points that are not listed along the wall), for reading every p from its
+// owner; its slowest CTA counts.  The loop of launches uses the whole GPU and
+// pays for its launches, beyond some rows also for rows.
 // Measured, FP32, us an iteration, cluster against loop.  Points along the wall, 34
 // entries a row: 8160 rows 9.6 / 18.8, 12,000 12.0 / 19.0, 16,000 18.5 / 19.0, 20,000 23.2 /
 // 21.5, 32,000 37.2 / 25.5; 9 entries a row: 32,000 13.8 / 22.0.  Points in random order, 34
 // entries: 2000 6.6 / 19.5, 4000 29 / 20, 8160 86 / 21, 32,000 255 / 32.
 // FP64, 34 entries: 2000 rows 11.5 / 23.9, 6000 24.6 / 28.4; random order 2000 25.5 / 24.4, 6000 95 / 29.
+
+// The CTA with rows r0 .. r0 + s.rper of n, `ne` entries, columns lo .. hi (from the
+// problem's first row; lo > hi: no entries).
 template <typename T>
-inline double afc_cluster_ns(const AfcRows& a, int n, int cl) {
+AFC_HD constexpr int64_t afc_cta_ps(const AfcShape& s, int n, int r0, int ne, int lo, int hi) {
   constexpr bool f32 = sizeof(T) == 4;
-  constexpr double base = f32 ? 4600 : 5100, row = f32 ? 2.4 : 11.4, hit = f32 ? 0.21 : 1.18,
-                   miss = f32 ? 0.55 : 2.0, far = f32 ? 4.0 : 6.0;
-  const AfcShape s = afc_shape<T>(n, cl);
-  double worst = 0.0;
-  for (int r0 = 0; r0 < n; r0 += s.rper) {
-    const int r1 = std::min(n, r0 + s.rper);
-    int lo = r0, hi = r1 - 1;
-    for (int i = r0; i < r1; ++i)
-      if (a.lo[i] <= a.hi[i]) lo = std::min(lo, a.lo[i]), hi = std::max(hi, a.hi[i]);
-    const int need = std::max(r0 - lo, hi - r1 + 1), ne = a.rowptr[r1] - a.rowptr[r0];
-    double t = base + row * s.rper;
-    if (need <= s.window) {
-      const int others = std::min(n, r1 + need) - std::max(0, r0 - need) - (r1 - r0);
-      const int cap = std::min(ne, afc_cached<T>(s, others));
-      t += hit * cap + miss * (ne - cap);
-    } else {
-      t += far * ne;
-    }
-    worst = std::max(worst, t);
-  }
-  return worst;
+  constexpr int64_t base = f32 ? 4600000 : 5100000, row = f32 ? 2400 : 11400, hit = f32 ? 210 : 1180,
+                    miss = f32 ? 550 : 2000, far = f32 ? 4000 : 6000;
+  const int r1 = r0 + s.rper < n ? r0 + s.rper : n;
+  const int below = lo <= hi && lo < r0 ? r0 - lo : 0, above = lo <= hi && hi >= r1 ? hi - r1 + 1 : 0;
+  const int need = below > above ? below : above;
+  int64_t t = base + row * s.rper;
+  if (need > s.window) return t + far * ne;
+  const int w0 = r0 > need ? r0 - need : 0, w1 = r1 + need < n ? r1 + need : n;
+  const int room = afc_cached<T>(s, w1 - w0 - (r1 - r0)), cap = ne < room ? ne : room;
+  return t + hit * cap + miss * (ne - cap);
 }
 template <typename T>
-inline double afc_loop_ns(int n) {
-  return sizeof(T) == 4 ? 18500 + 0.3 * std::max(0, n - 16000) : 22500 + 0.5 * std::max(0, n - 4500);
+AFC_HD constexpr int64_t afc_loop_ps(int n) {
+  return sizeof(T) == 4 ? 18500000 + (n > 16000 ? int64_t(300) * (n - 16000) : 0)
+                        : 22500000 + (n > 4500 ? int64_t(500) * (n - 4500) : 0);
 }
 
-// Whether a cluster solves the problem.  By the problem's own rows and the
-// device's cluster size alone, so that its bits do not depend on the batch it runs
-// in; after a move of the points the choice stays (any S is solved right either way).
+// Whether a cluster of cl CTAs solves the problem of n rows whose slowest CTA
+// takes `ps`.  By the problem's own rows and the device's cluster size alone, so that its
+// bits do not depend on the batch it runs in.
 template <typename T>
-inline bool afc_takes(const AfcRows& a, int n, int cl) {
-  return cl > 0 && n > 0 && n <= afc_max_rows<T>(cl) && afc_cluster_ns<T>(a, n, cl) <= afc_loop_ns<T>(n);
+AFC_HD constexpr bool afc_takes(int64_t n, int cl, int64_t ps) {
+  return cl > 0 && n > 0 && n <= afc_max_rows<T>(cl) && ps <= afc_loop_ps<T>(int(n));
+}
+// ps from rowptr ([n + 1], any base) and the problem's first entry of col, whose first
+// row has number row0 there.  Where no cluster takes n rows: 0.
+template <typename T>
+inline int64_t afc_cluster_ps(const int32_t* rowptr, const int32_t* col, int32_t row0, int64_t n, int cl) {
+  int64_t worst = 0;
+  if (cl <= 0 || n > afc_max_rows<T>(cl)) return 0;
+  const AfcShape s = afc_shape<T>(int(n), cl);
+  for (int r0 = 0; r0 < n; r0 += s.rper) {
+    const int32_t *e0 = col + (rowptr[r0] - rowptr[0]), *e1 = col + (rowptr[std::min<int64_t>(n, r0 + s.rper)] - rowptr[0]);
+    const auto mm = std::minmax_element(e0, e1);
+    worst = std::max(worst, afc_cta_ps<T>(s, int(n), r0, int(e1 - e0), e0 < e1 ? *mm.first - row0 : 1,
+                                          e0 < e1 ? *mm.second - row0 : 0));
+  }
+  return worst;
 }
 
 }  // namespace ibg

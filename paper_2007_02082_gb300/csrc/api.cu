@@ -112,6 +112,7 @@ struct Engine {
   int32_t *mv_bins = nullptr, *mv_rcnt = nullptr, *mv_scratch = nullptr, *mv_err = nullptr;
   int32_t *mv_scnt = nullptr, *mv_sstart = nullptr, *mv_sfill = nullptr, *mv_sflag = nullptr, *mv_sidx = nullptr;
   double *mv_xprev = nullptr, *mv_ubprev = nullptr;
+  unsigned long long* mv_plan = nullptr;   // [2] times that choose the force solver
   int64_t af_cap = 0;             // capacity of ib.col / ib.val
   bool mv_graph_stale = false;    // a rebuild reallocated a list the step graphs hold
   double *wss_n = nullptr, *wss_w = nullptr, *wss_g = nullptr;   // wall shear stress buffers
@@ -141,7 +142,10 @@ struct Engine {
   MGDev<double> mg64;
   Prof prof;
   bool use_graph = true;
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  // the step's graphs by buffer parity and, in steps of two, by the force solvers that
+  // the points of a moving wall choose (af_route of the one problem)
+  cudaGraphExec_t gexec[8] = {};
+  uint8_t route = 0;
   cudaStream_t cap_st = nullptr;
   CaptureCtx cc;
   // per-instance host counters
@@ -235,8 +239,8 @@ ib_status upload(Engine& E, T** p, const std::vector<T>& v) {
 
 void engine_free(Engine& E) {
   if (E.st) cudaStreamSynchronize(E.st);
-  for (int k = 0; k < 2; ++k)
-    if (E.gexec[k]) { cudaGraphExecDestroy(E.gexec[k]); E.gexec[k] = nullptr; }
+  for (cudaGraphExec_t& x : E.gexec)
+    if (x) { cudaGraphExecDestroy(x); x = nullptr; }
   for (void* p : E.allocs) raw_free(E.freef, E.actx, p);
   E.allocs.clear();
   E.bytes = 0;
@@ -859,6 +863,7 @@ ib_status engine_build(Engine& E) {
     uint8_t* d_route;
     TRY(upload(E, &d_route, route));
     ib.af_route = d_route;
+    if (n == 1) E.route = route[0];
   }
   TRY(dalloc(E, &ib.W, 64 * Mt, true));
   TRY(dalloc(E, &ib.val, int64_t(col.size()), true));
@@ -1038,7 +1043,8 @@ ib_status engine_step(Engine& E) {
   cudaStream_t st = E.st;
   const int par = (E.u == E.ubuf[0]) ? 0 : 1;
   if (E.use_graph) {
-    if (!E.gexec[par]) {
+    cudaGraphExec_t& exec = E.gexec[par + 2 * E.route];
+    if (!exec) {
       cudaGraph_t graph = nullptr;
       cudaStream_t cs = E.cap_st;
       CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
@@ -1052,15 +1058,15 @@ ib_status engine_step(Engine& E) {
         E.err = std::string("graph capture failed: ") + cudaGetErrorString(e != cudaSuccess ? e : e2);
         return IB_ECUDA;
       }
-      e = cudaGraphInstantiate(&E.gexec[par], graph, 0);
+      e = cudaGraphInstantiate(&exec, graph, 0);
       cudaGraphDestroy(graph);
       if (e != cudaSuccess) {
-        E.gexec[par] = nullptr;
+        exec = nullptr;
         E.err = std::string("graph instantiation failed: ") + cudaGetErrorString(e);
         return IB_ECUDA;
       }
     }
-    CK(cudaGraphLaunch(E.gexec[par], st));
+    CK(cudaGraphLaunch(exec, st));
   } else {
     E.cc.capturing = false;
     cudaError_t e = enqueue_step(E, E.u, E.un, E.p, E.pn, st);
@@ -1545,6 +1551,7 @@ ib_status move_alloc(Engine& E) {
   TRY(dalloc(E, &E.mv_sflag, ns + 1, true));
   TRY(dalloc(E, &E.mv_sidx, ns + 1, true));
   TRY(dalloc(E, &E.mv_xprev, 3 * M + 1, true));
+  TRY(dalloc(E, &E.mv_plan, 2, true));
   TRY(dalloc(E, &E.mv_ubprev, 3 * M + 1, true));
   // spreading lists at their largest (every support node of every point free)
   int32_t *sp_ent, *sp_slot, *sp_off;
@@ -1603,6 +1610,7 @@ ib_status move_rebuild(Engine& E) {
     E.mv_graph_stale = true;
   }
   mv_af_fill(G, M, org, E.mv_bins, rowptr, const_cast<int32_t*>(ib.col), st);
+  ib_plan_moved(ib, E.mv_plan, st);
   ib_weights(ib, st);
   ib_assemble(ib, st);
   mv_spread(M, ns, slot, fb, E.mv_scnt, E.mv_sstart, E.mv_sfill, E.mv_sflag, E.mv_sidx,
@@ -1648,8 +1656,8 @@ ib_status ib_set_points(ib_grid* g, int64_t M, const double* X, const double* UB
   // the captured step graphs read the list lengths from the device; only a
   // reallocated buffer (first move, a larger A_F) needs a new capture
   if (E.mv_graph_stale) {
-    for (int k = 0; k < 2; ++k)
-      if (E.gexec[k]) { cudaGraphExecDestroy(E.gexec[k]); E.gexec[k] = nullptr; }
+    for (cudaGraphExec_t& x : E.gexec)
+      if (x) { cudaGraphExecDestroy(x); x = nullptr; }
     E.mv_graph_stale = false;
   }
   // host copies of the inputs and supports (exported by ib_fields_get)
@@ -1661,7 +1669,16 @@ ib_status ib_set_points(ib_grid* g, int64_t M, const double* X, const double* UB
     CKG(cudaMemcpyAsync(H.ib_slot.data(), E.ib.slot, 64 * M * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CKG(cudaMemcpyAsync(H.ib_free.data(), E.ib.freeb, M * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
   }
+  unsigned long long ps[2] = {0, 0};
+  CKG(cudaMemcpyAsync(ps, E.mv_plan, sizeof(ps), cudaMemcpyDeviceToHost, st));
   CKG(cudaStreamSynchronize(st));
+  // the force solver of the new points, as a fresh handle would choose it
+  const uint8_t route = ib_moved_route(E.ib, ps);
+  if (M && route != E.route) {
+    CKG(cudaMemcpyAsync(const_cast<uint8_t*>(E.ib.af_route), &route, 1, cudaMemcpyHostToDevice, st));
+    CKG(cudaStreamSynchronize(st));
+    E.route = route;
+  }
 #undef CKG
   return IB_OK;
 }

@@ -7,7 +7,6 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
-#include <vector>
 
 #include "async.cuh"
 #include "ib.hpp"
@@ -300,6 +299,40 @@ void ib_weights(const IBDev& ib, cudaStream_t st) {
              ib.ihf, ib.W);
 }
 
+// afc_cluster_ps of one problem on the device: a CTA for each CTA of the cluster, FP32 in
+// y = 0, FP64 in y = 1
+__global__ void __launch_bounds__(IBB) k_af_plan(IBDev ib, unsigned long long* __restrict__ ps) {
+  KCOUNT();
+  __shared__ int slo[IBB / 32], shi[IBB / 32];
+  const bool f32 = blockIdx.y == 0;
+  const int cl = f32 ? ib.af_cl32 : ib.af_cl64, n = int(ib.M);
+  if (int(blockIdx.x) >= cl || n > (f32 ? afc_max_rows<float>(cl) : afc_max_rows<double>(cl))) return;
+  const AfcShape s = f32 ? afc_shape<float>(n, cl) : afc_shape<double>(n, cl);
+  const int r0 = int(blockIdx.x) * s.rper;
+  if (r0 >= n) return;
+  const int e0 = ib.rowptr[r0], e1 = ib.rowptr[min(n, r0 + s.rper)];
+  int lo = n, hi = -1;
+  for (int e = e0 + int(threadIdx.x); e < e1; e += IBB) {
+    const int k = ib.col[e];
+    lo = min(lo, k);
+    hi = max(hi, k);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) {
+    slo[threadIdx.x >> 5] = lo;
+    shi[threadIdx.x >> 5] = hi;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < IBB / 32; ++w) {
+    lo = min(lo, slo[w]);
+    hi = max(hi, shi[w]);
+  }
+  atomicMax(ps + blockIdx.y, (unsigned long long)(f32 ? afc_cta_ps<float>(s, n, r0, e1 - e0, lo, hi)
+                                                      : afc_cta_ps<double>(s, n, r0, e1 - e0, lo, hi)));
+}
+
 template <typename T>
 static cudaLaunchConfig_t afc_config(int ninst, int cl, cudaLaunchAttribute* attr, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
@@ -334,31 +367,38 @@ static int afc_cluster_size() {
   return 0;
 }
 
+// the bits of a problem of n rows, added to the switches over all problems
+static uint8_t route_of(IBDev& ib, int64_t n, int64_t ps32, int64_t ps64) {
+  const bool c32 = afc_takes<float>(n, ib.af_cl32, ps32), c64 = afc_takes<double>(n, ib.af_cl64, ps64);
+  ib.af_small32 |= c32;
+  ib.af_small64 |= c64;
+  ib.af_big32 |= n > 0 && !c32;
+  ib.af_big64 |= n > 0 && !c64;
+  return uint8_t((c32 ? AF_CLUSTER32 : 0) | (c64 ? AF_CLUSTER64 : 0));
+}
+
 void ib_choose_solver(IBDev& ib, const int32_t* seg_t, const int32_t* rowptr, const int32_t* col, bool mixed,
                       uint8_t* route) {
-  const int cl32 = mixed ? afc_cluster_size<float>() : 0, cl64 = afc_cluster_size<double>();
-  ib.af_cl32 = ib.af_cl64 = 0;
-  ib.af_big32 = ib.af_big64 = false;
-  std::vector<int32_t> lo, hi;
+  ib.af_cl32 = mixed ? afc_cluster_size<float>() : 0;
+  ib.af_cl64 = afc_cluster_size<double>();
+  ib.af_small32 = ib.af_small64 = ib.af_big32 = ib.af_big64 = false;
   for (int i = 0; i < ib.ninst; ++i) {
-    const int64_t r0 = int64_t(seg_t[i]) * 256;
-    const int n = (seg_t[i + 1] - seg_t[i]) * 256;
-    route[i] = 0;
-    if (n == 0) continue;
-    lo.assign(n, 1);
-    hi.assign(n, 0);
-    for (int r = 0; r < n && n <= afc_max_rows<float>(AFC_MAX); ++r)
-      if (rowptr[r0 + r] < rowptr[r0 + r + 1]) {
-        const auto e = std::minmax_element(col + rowptr[r0 + r], col + rowptr[r0 + r + 1]);
-        lo[r] = int32_t(*e.first - r0);
-        hi[r] = int32_t(*e.second - r0);
-      }
-    const AfcRows a{rowptr + r0, lo.data(), hi.data()};
-    if (afc_takes<float>(a, n, cl32)) route[i] |= AF_CLUSTER32, ib.af_cl32 = cl32;
-    else ib.af_big32 = true;
-    if (afc_takes<double>(a, n, cl64)) route[i] |= AF_CLUSTER64, ib.af_cl64 = cl64;
-    else ib.af_big64 = true;
+    const int64_t r0 = int64_t(seg_t[i]) * 256, n = int64_t(seg_t[i + 1]) * 256 - r0;
+    const int32_t *rp = rowptr + r0, *c = col + rp[0];
+    route[i] = route_of(ib, n, afc_cluster_ps<float>(rp, c, int32_t(r0), n, ib.af_cl32),
+                        afc_cluster_ps<double>(rp, c, int32_t(r0), n, ib.af_cl64));
   }
+}
+
+void ib_plan_moved(const IBDev& ib, unsigned long long* ps, cudaStream_t st) {
+  cudaMemsetAsync(ps, 0, 2 * sizeof(*ps), st);
+  if (ib.M > 0 && ib.M <= afc_max_rows<float>(AFC_MAX))
+    IBG_LAUNCH(k_af_plan, dim3(AFC_MAX, 2), IBB, 0, st, ib, ps);
+}
+
+uint8_t ib_moved_route(IBDev& ib, const unsigned long long* ps) {
+  ib.af_small32 = ib.af_small64 = ib.af_big32 = ib.af_big64 = false;
+  return route_of(ib, ib.M, int64_t(ps[0]), int64_t(ps[1]));
 }
 
 // the cluster solve of every problem routed to it; x: the iterate (updated), r: its residual
@@ -391,7 +431,7 @@ cudaError_t ib_solve(const IBDev& ib, const double* BF, double* G, double* work,
   double *r = work, *z = work + L, *p = work + 2 * L, *q = work + 3 * L;
   IBG_LAUNCH(k_init_states, (ib.ninst * 3 + 127) / 128, 128, 0, st, ks, ib.ninst * 3, rtol * rtol, max_iter);
   Cond cond;
-  const bool cluster = ib.af_cl64 > 0, loop = ib.af_big64;
+  const bool cluster = ib.af_small64, loop = ib.af_big64;
   if (loop && cc && cc->capturing) {
     cudaError_t e = cond_handle(st, 0, &cond);
     if (e != cudaSuccess) return e;
@@ -518,7 +558,7 @@ cudaError_t ib_solve_mixed(const IBDev& ib, const double* BF, double* G, double*
     }
     IBG_LAUNCH((k_af_start<float>), gt, IBB, 0, s, ib, (const float*)ib.dinv32, (const float*)r32,
                (const float*)nullptr, r, z, pa, ks, rb.partials, rb.counter, ci, (const OState*)os);
-    if (ib.af_cl32 > 0) af_cluster_solve<float>(ib, ib.af_cl32, ib.val32, ib.dinv32, e32, r, ks, s);
+    if (ib.af_small32) af_cluster_solve<float>(ib, ib.af_cl32, ib.val32, ib.dinv32, e32, r, ks, s);
     auto iter = [&](cudaStream_t s2, const Cond& c2, const float* pold, float* pnew) {
       IBG_LAUNCH((k_af_apply_p<float>), g8, IBB, 0, s2, ib, (const float*)ib.val32, (const float*)z, pold, pnew, q,
                  ks, rb.partials, rb.counter);

@@ -44,11 +44,12 @@ struct IBDev {
   // device and launches cover sp_cap entries, so a captured step stays valid
   const int32_t* n_sp_dev = nullptr;
   int64_t sp_cap = 0;
-  // force solve (ib_choose_solver): CTAs of the cluster that solves a problem
-  // in one launch (0: no problem is solved so), the problems that are ([ninst], AF_CLUSTER
-  // bits), and whether some problem takes the launch-per-pass loop, in FP32 and FP64
+  // force solve: CTAs of the device's cluster (0: none), the AF_CLUSTER bits of every
+  // problem ([ninst]), and over all problems whether some problem is solved by a
+  // cluster and whether some takes the launch-per-pass loop, in FP32 and FP64
   int32_t af_cl32 = 0, af_cl64 = 0;
   const uint8_t* af_route = nullptr;
+  bool af_small32 = false, af_small64 = false;
   bool af_big32 = true, af_big64 = true;
 };
 enum : uint8_t { AF_CLUSTER32 = 1, AF_CLUSTER64 = 2 };
@@ -58,6 +59,11 @@ enum : uint8_t { AF_CLUSTER32 = 1, AF_CLUSTER64 = 2 };
 // to upload to ib.af_route.  Without mixed no FP32 solve is planned.
 void ib_choose_solver(IBDev& ib, const int32_t* seg_t, const int32_t* rowptr, const int32_t* col, bool mixed,
                       uint8_t* route);
+// The same for the one problem of a handle whose points moved, from the rows on the
+// device: ps[0], ps[1] take the FP32 and FP64 times, from which ib_moved_route
+// gives the bits and sets ib's switches.
+void ib_plan_moved(const IBDev& ib, unsigned long long* ps, cudaStream_t st);
+uint8_t ib_moved_route(IBDev& ib, const unsigned long long* ps);
 
 // Eq. 17-18: W[i][a] = phi((x_a - X_i)/hx) phi((y_a - Y_i)/hy) phi((z_a - Z_i)/hz).
 void ib_weights(const IBDev& ib, cudaStream_t st);

@@ -89,6 +89,7 @@ int main(int argc, char** argv) {
   if (head[2] >= 0) {
     ib.af_cl32 = ib.af_cl64 = int32_t(head[2]);
     ib.af_big32 = ib.af_big64 = head[2] == 0;
+    ib.af_small32 = ib.af_small64 = head[2] != 0;
     for (uint8_t& v : route) v = head[2] ? AF_CLUSTER32 | AF_CLUSTER64 : 0;
   }
   ib.af_route = put(route);
