@@ -520,10 +520,14 @@ struct SmallArgs {
 // or one CTA (k_mg_levels); sync makes the vectors written before it visible to
 // all of them.
 struct CtaTeam {
+  using Ld = PlainLoad;
+  static constexpr bool STAGED = false;
   int t = threadIdx.x, n = blockDim.x, rank = 0, ctas = 1;
   __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
 struct ClusterTeam {
+  using Ld = FreshLoad;
+  static constexpr bool STAGED = true;   // the dense inverse goes through shared memory
   int t, n, rank, ctas;
   __device__ ClusterTeam() {
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -540,10 +544,10 @@ struct ClusterTeam {
 // The small levels and the coarsest solve of problem i, by the whole team;
 // each node's value is computed by one thread, in an order that does not
 // depend on the team.  tile: tile_len values of shared memory for the
-// dense inverse.
+// dense inverse (a staged team's).
 template <typename T, typename Team>
 __device__ void small_cycle(const SmallArgs<T>& a, int i, const KState* ks, const Team& tm, T* tile, int tile_len) {
-  using Ld = FreshLoad;
+  using Ld = typename Team::Ld;
   if (!a.on[i] || ks[i].done) return;
   const int k0 = a.small[i], K = a.coarsest[i];
   const int t = tm.t, nt = tm.n;
@@ -579,32 +583,42 @@ __device__ void small_cycle(const SmallArgs<T>& a, int i, const KState* ks, cons
     }
     tm.sync();
   }
-  // coarsest: x = A^-1 b with the (symmetrised) dense inverse, by columns; each
-  // CTA takes a range of rows and stages their entries in shared memory (a
-  // row's sum is one chain of n terms: from memory its loads would wait in turn)
+  // coarsest: x = A^-1 b with the (symmetrised) dense inverse, by columns.  A row's sum
+  // is one chain of n terms.  Each CTA of a cluster takes a range of rows and
+  // stages their entries in shared memory (from memory a short range's loads would wait in
+  // turn); a CTA alone has its threads full of rows and reads them as they
+  // come (k_mg_levels with a staged tile of 16 KB: 139 us on the 32x32x128 tube, 80 without).
   {
     const MGLevelDev<T>& L = a.lev[K];
     const int j0 = L.noff[i], n = L.noff[i + 1] - j0;
     const T* Ai = a.cinv + a.cinv_off[i];
-    const int nr = (n + tm.ctas - 1) / tm.ctas, r0 = min(tm.rank * nr, n), rows = min(nr, n - r0);
-    const int ct = max(1, tile_len / (nr + 1));   // columns of a tile, after their entries of b
-    for (int rb = 0; rb < rows; rb += int(blockDim.x)) {
-      const int m = min(rows - rb, int(blockDim.x));
-      T v = T(0);
-      for (int c0 = 0; c0 < n; c0 += ct) {
-        const int nc = min(ct, n - c0);
-        __syncthreads();
-        for (int e = threadIdx.x; e < nc * m; e += blockDim.x) {
-          const int c = e / m;
-          tile[nc + e] = Ai[(int64_t)(c0 + c) * n + r0 + rb + (e - c * m)];
-        }
-        for (int c = threadIdx.x; c < nc; c += blockDim.x) tile[c] = Ld::ld(L.b + j0 + c0 + c);
-        __syncthreads();
-        if (int(threadIdx.x) < m)
-#pragma unroll 8
-          for (int c = 0; c < nc; ++c) v += tile[nc + c * m + threadIdx.x] * tile[c];
+    if constexpr (!Team::STAGED) {
+      for (int r = t; r < n; r += nt) {
+        T v = T(0);
+        for (int c = 0; c < n; ++c) v += Ai[(int64_t)c * n + r] * Ld::ld(L.b + j0 + c);
+        L.xa[j0 + r] = v;
       }
-      if (int(threadIdx.x) < m) L.xa[j0 + r0 + rb + threadIdx.x] = v;
+    } else {
+      const int nr = (n + tm.ctas - 1) / tm.ctas, r0 = min(tm.rank * nr, n), rows = min(nr, n - r0);
+      const int ct = max(1, tile_len / (nr + 1));   // columns of a tile, after their entries of b
+      for (int rb = 0; rb < rows; rb += int(blockDim.x)) {
+        const int m = min(rows - rb, int(blockDim.x));
+        T v = T(0);
+        for (int c0 = 0; c0 < n; c0 += ct) {
+          const int nc = min(ct, n - c0);
+          __syncthreads();
+          for (int e = threadIdx.x; e < nc * m; e += blockDim.x) {
+            const int c = e / m;
+            tile[nc + e] = Ai[(int64_t)(c0 + c) * n + r0 + rb + (e - c * m)];
+          }
+          for (int c = threadIdx.x; c < nc; c += blockDim.x) tile[c] = Ld::ld(L.b + j0 + c0 + c);
+          __syncthreads();
+          if (int(threadIdx.x) < m)
+#pragma unroll 8
+            for (int c = 0; c < nc; ++c) v += tile[nc + c * m + threadIdx.x] * tile[c];
+        }
+        if (int(threadIdx.x) < m) L.xa[j0 + r0 + rb + threadIdx.x] = v;
+      }
     }
     tm.sync();
   }
@@ -676,7 +690,6 @@ void launch_small(const SmallArgs<T>& a, int ninst, const KState* ks, cudaStream
 // (cooperative launch); each barrier wait is bounded in wall-clock time, and
 // on expiry the CTA records ASYNC_TIMEOUT for every problem and returns.
 constexpr int LV_THREADS = 512;
-constexpr int LV_TILE = 4096;   // values of shared memory for the dense inverse
 
 template <typename T>
 struct LevelsArgs {
@@ -764,11 +777,7 @@ __global__ void __launch_bounds__(LV_THREADS) k_mg_levels(LevelsArgs<T> a, const
     if (!grid_barrier(a.bar, a.ninst, a.aerr)) return;
   }
   // small levels and the coarsest solve, here a CTA per problem
-  __shared__ T tile[LV_TILE];
-  for (int i = blockIdx.x; i < a.ninst; i += gridDim.x) {
-    __syncthreads();
-    small_cycle(S, i, ks, CtaTeam(), tile, LV_TILE);
-  }
+  for (int i = blockIdx.x; i < a.ninst; i += gridDim.x) small_cycle(S, i, ks, CtaTeam(), (T*)nullptr, 0);
   if (!grid_barrier(a.bar, a.ninst, a.aerr)) return;
   // levels up: prolongation, post-smoothing; each level's result ends in xa
   for (int k = a.max_big - 1; k >= 0; --k) {
