@@ -88,7 +88,7 @@ AFC_HD constexpr int64_t afc_cta_ps(const AfcShape& s, int n, int r0, int ne, in
 template <typename T>
 AFC_HD constexpr int64_t afc_loop_ps(int n) {
   return sizeof(T) == 4 ? 18500000 + (n > 16000 ? int64_t(300) * (n - 16000) : 0)
-                        : 22500000 + (n > 4500 ? int64_t(500) * (n - 4500) : 0);
+                        : 22500000 + (n > 4500 ? int64_t(2000) * (n - 4500) : 0);
 }
 
 // Whether a cluster of cl CTAs solves the problem of n rows whose slowest CTA

@@ -39,6 +39,7 @@ def route(probe, tmp_path, M, spacing, R, shuffled, cl=16):
     (4000, 2.4, 25, True, True, None),
     (4000, 1.25, 25, True, False, False),
     (6000, 1.25, 25, True, False, False),
+    (6000, 1.25, 25, False, True, True),
     (6000, 2.4, 25, False, True, True),
     (8160, 1.25, 25, True, False, False),
     (12000, 1.25, 25, False, True, False),
