@@ -217,7 +217,7 @@ def class_bytes(cls, vb, multigrid=False):
     """Algorithmic bytes per stored valid node slot of one launch of a kernel class."""
     return {
         0: 4 * vb + 2,                 # Poisson CG stencil: read z, p_old, meta; write p_new, q
-        1: (6 if multigrid else 7) * vb + 2,   # CG update: x rw, r rw, p, q read, meta (+ D^-1 read, z write)
+        1: (8 if multigrid else 7) * vb + 2,   # CG update: x rw, r rw, p, q, D^-1, meta read; z written
         2: 3 * vb,                     # p = z + beta p: z read, p rw
         3: 12 * vb + 2,                # mass CG stencil, 3 comps: read z, p_old; write p_new, q
         4: 3 * 6 * vb + vb + 2,        # mass CG update, 3 components + D^-1

@@ -15,11 +15,12 @@
 // the shared memories and points in an order that needs p from everywhere go to the loop.
 // A problem's arithmetic depends on its own rows only, so it keeps its bits
 // alone and in any batch; problems of a batch run side by side.
-// Bound: latency of the barriers and scalars at a few hundred rows (3.8 us an
-// iteration), shared-memory wavefronts of the product at some thousand dense rows
-// (8160 rows of 41 entries: 10 us), in FP64 the FP64 rate of 16 SMs (2000 rows: 11.5 us).
-// A step: 8x8x16 tube 21.6 -> 5.2 ms, 16x16x64 tube in FP64 31.6 -> 14.4 ms, dense
-// 32x32x128 tube 25.4 -> 12.0 ms (of which the reductions alone gave a third).
+// Bound: latency of the barriers and scalars at a few hundred rows (3.9 us an
+// iteration); at some thousand dense rows barriers and shared-memory latency, the
+// shared-memory pipe at 57 % (8160 rows of 41 entries: 10 us); in FP64 the FP64 pipe of
+// 16 SMs, 57 % busy between barriers (2000 rows of 40: 11 us).
+// A step: 8x8x16 tube 19.1 -> 5.25 ms, 16x16x64 tube in FP64 30.9 -> 13.9 ms, dense
+// 32x32x128 tube 22.5 -> 11.1 ms (of which the reductions alone gave a third).
 #pragma once
 
 #include "af_plan.hpp"

@@ -1091,7 +1091,9 @@ __device__ __forceinline__ void p7_issue(const DevGrid& g, unsigned char* stage,
 // brick's own nodes, so K z is neither written nor read again: 18 bytes a
 // node instead of 32.  Nodes whose K z is an interface sum are left to
 // k_mg_if_smooth: q receives the level's part at interface and hanging nodes
-// only.  Bound by the stages in flight, as the apply.  A sweep of the 16 M-node
+// only.  Bound by HBM over many waves: whole bricks are copied, padding included, so that
+// the 59 M-node aorta moves 1.59 GB a launch where 18 bytes a node are 1.06, in 227 us
+// (1.03 of the copy bandwidth); in one wave by ring fill and tail.  A sweep of the 16 M-node
 // sac with its interface nodes: 98 -> 74 us (apply, sums, update -> one pass, interface nodes).
 template <bool CG, bool SMOOTH = false>
 __global__ void __launch_bounds__(P7_THREADS, SMOOTH ? 6 : 8)

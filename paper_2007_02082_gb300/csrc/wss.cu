@@ -30,8 +30,8 @@ namespace {
 // the derivatives are linear in the 27 moments of the velocity, so one pass over
 // the nodes suffices.  Each set is summed over the lanes in one butterfly; the
 // 9 x 9 Cholesky solves of 32 points share one warp, a point a lane.  ib_wss on
-// the 32,000 points of the refined 64x64x256 tube, host copies included: 7.95 ms
-// with a thread per point and two passes, 1.8 ms here.
+// the 32,000 points of the refined 64x64x256 tube, host copies included: 7.91 ms
+// with a thread per point and two passes, 1.78 ms here (FP64 pipe 66 % busy).
 constexpr int WSS_PTS = 32;       // points of a CTA
 constexpr int WSS_WARPS = 8;
 
