@@ -59,35 +59,42 @@ AFC_HD constexpr int afc_cached(const AfcShape& s, int others) {
 // Time of an iteration in picoseconds as measured (whole numbers: the same choice on
 // the host and on the device).  A cluster pays for its barriers and scalars, for rows,
 // for entries in shared memory, for entries that did not fit (read again every
-// iteration by 16 SMs) and, where a CTA's columns reach too far for a
-// window (points that are not listed along the wall), for reading every p from its
-// owner; its slowest CTA counts.  The loop of launches uses the whole GPU and
+// iteration by 16 SMs) and, where a CTA's columns reach too far for a window
+// (points that are not listed along the wall), for reading every foreign p from its
+// owner and for a third barrier (a foreign p costs more the larger their part, as then all
+// CTAs read from all); its slowest CTA counts.  The loop of launches uses the whole GPU and
 // pays for its launches, beyond some rows also for rows.
 // Measured, FP32, us an iteration, cluster against loop.  Points along the wall, 34
 // entries a row: 8160 rows 9.6 / 18.8, 12,000 12.0 / 19.0, 16,000 18.5 / 19.0, 20,000 23.2 /
 // 21.5, 32,000 37.2 / 25.5; 9 entries a row: 32,000 13.8 / 22.0.  Points in random order, 34
 // entries: 2000 6.6 / 19.5, 4000 29 / 20, 8160 86 / 21, 32,000 255 / 32.
 // FP64, 34 entries: 2000 rows 11.5 / 23.9, 6000 24.6 / 28.4; random order 2000 25.5 / 24.4, 6000 95 / 29.
+// A tube's points followed by those of a sac on it (some CTAs without a window, a tenth of
+// their entries foreign): 6837 rows of 16 entries 10.9 / 18.0, 15,234 of 18 16.1 / 19.5.
+// Over some 250 systems the choice cost at most 17 % against the faster side.
 
-// The CTA with rows r0 .. r0 + s.rper of n, `ne` entries, columns lo .. hi (from the
-// problem's first row; lo > hi: no entries).
+// The CTA with rows r0 .. r0 + s.rper of n, `ne` entries, `nf` of them in columns of other
+// CTAs, columns lo .. hi (from the problem's first row; lo > hi: no entries).
 template <typename T>
-AFC_HD constexpr int64_t afc_cta_ps(const AfcShape& s, int n, int r0, int ne, int lo, int hi) {
+AFC_HD constexpr int64_t afc_cta_ps(const AfcShape& s, int n, int r0, int ne, int nf, int lo, int hi) {
   constexpr bool f32 = sizeof(T) == 4;
   constexpr int64_t base = f32 ? 4600000 : 5100000, row = f32 ? 2400 : 11400, hit = f32 ? 210 : 1180,
-                    miss = f32 ? 550 : 2000, far = f32 ? 4000 : 6000;
+                    miss = f32 ? 550 : 2000, own = f32 ? 210 : 1000, third = 1500000,
+                    foreign = f32 ? 1600 : 2500, crowd = f32 ? 2900 : 3500;
   const int r1 = r0 + s.rper < n ? r0 + s.rper : n;
   const int below = lo <= hi && lo < r0 ? r0 - lo : 0, above = lo <= hi && hi >= r1 ? hi - r1 + 1 : 0;
   const int need = below > above ? below : above;
   int64_t t = base + row * s.rper;
-  if (need > s.window) return t + far * ne;
+  if (need > s.window) return t + third + own * (ne - nf) + foreign * nf + crowd * nf * nf / ne;   // ne > 0
   const int w0 = r0 > need ? r0 - need : 0, w1 = r1 + need < n ? r1 + need : n;
   const int room = afc_cached<T>(s, w1 - w0 - (r1 - r0)), cap = ne < room ? ne : room;
   return t + hit * cap + miss * (ne - cap);
 }
+// (The loop was measured at 17.5 to 21 us in FP32 below 16,000 rows; the cluster's estimate
+// is some 10 % high for dense rows near the line, so the line lies at the upper end.)
 template <typename T>
 AFC_HD constexpr int64_t afc_loop_ps(int n) {
-  return sizeof(T) == 4 ? 18500000 + (n > 16000 ? int64_t(300) * (n - 16000) : 0)
+  return sizeof(T) == 4 ? 20500000 + (n > 16000 ? int64_t(300) * (n - 16000) : 0)
                         : 22500000 + (n > 4500 ? int64_t(2000) * (n - 4500) : 0);
 }
 
@@ -106,10 +113,16 @@ inline int64_t afc_cluster_ps(const int32_t* rowptr, const int32_t* col, int32_t
   if (cl <= 0 || n > afc_max_rows<T>(cl)) return 0;
   const AfcShape s = afc_shape<T>(int(n), cl);
   for (int r0 = 0; r0 < n; r0 += s.rper) {
-    const int32_t *e0 = col + (rowptr[r0] - rowptr[0]), *e1 = col + (rowptr[std::min<int64_t>(n, r0 + s.rper)] - rowptr[0]);
-    const auto mm = std::minmax_element(e0, e1);
-    worst = std::max(worst, afc_cta_ps<T>(s, int(n), r0, int(e1 - e0), e0 < e1 ? *mm.first - row0 : 1,
-                                          e0 < e1 ? *mm.second - row0 : 0));
+    const int r1 = int(std::min<int64_t>(n, r0 + s.rper));
+    const int32_t *e0 = col + (rowptr[r0] - rowptr[0]), *e1 = col + (rowptr[r1] - rowptr[0]);
+    int lo = int(n), hi = -1, nf = 0;
+    for (const int32_t* e = e0; e < e1; ++e) {
+      const int k = *e - row0;
+      lo = std::min(lo, k);
+      hi = std::max(hi, k);
+      nf += k < r0 || k >= r1;
+    }
+    worst = std::max(worst, afc_cta_ps<T>(s, int(n), r0, int(e1 - e0), nf, lo, hi));
   }
   return worst;
 }

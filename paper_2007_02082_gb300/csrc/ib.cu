@@ -303,34 +303,39 @@ void ib_weights(const IBDev& ib, cudaStream_t st) {
 // y = 0, FP64 in y = 1
 __global__ void __launch_bounds__(IBB) k_af_plan(IBDev ib, unsigned long long* __restrict__ ps) {
   KCOUNT();
-  __shared__ int slo[IBB / 32], shi[IBB / 32];
+  __shared__ int slo[IBB / 32], shi[IBB / 32], snf[IBB / 32];
   const bool f32 = blockIdx.y == 0;
   const int cl = f32 ? ib.af_cl32 : ib.af_cl64, n = int(ib.M);
   if (int(blockIdx.x) >= cl || n > (f32 ? afc_max_rows<float>(cl) : afc_max_rows<double>(cl))) return;
   const AfcShape s = f32 ? afc_shape<float>(n, cl) : afc_shape<double>(n, cl);
   const int r0 = int(blockIdx.x) * s.rper;
   if (r0 >= n) return;
-  const int e0 = ib.rowptr[r0], e1 = ib.rowptr[min(n, r0 + s.rper)];
-  int lo = n, hi = -1;
+  const int r1 = min(n, r0 + s.rper);
+  const int e0 = ib.rowptr[r0], e1 = ib.rowptr[r1];
+  int lo = n, hi = -1, nf = 0;
   for (int e = e0 + int(threadIdx.x); e < e1; e += IBB) {
     const int k = ib.col[e];
     lo = min(lo, k);
     hi = max(hi, k);
+    nf += k < r0 || k >= r1;
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
+  nf = __reduce_add_sync(0xffffffffu, nf);
   if ((threadIdx.x & 31) == 0) {
     slo[threadIdx.x >> 5] = lo;
     shi[threadIdx.x >> 5] = hi;
+    snf[threadIdx.x >> 5] = nf;
   }
   __syncthreads();
   if (threadIdx.x != 0) return;
   for (int w = 1; w < IBB / 32; ++w) {
     lo = min(lo, slo[w]);
     hi = max(hi, shi[w]);
+    nf += snf[w];
   }
-  atomicMax(ps + blockIdx.y, (unsigned long long)(f32 ? afc_cta_ps<float>(s, n, r0, e1 - e0, lo, hi)
-                                                      : afc_cta_ps<double>(s, n, r0, e1 - e0, lo, hi)));
+  atomicMax(ps + blockIdx.y, (unsigned long long)(f32 ? afc_cta_ps<float>(s, n, r0, e1 - e0, nf, lo, hi)
+                                                      : afc_cta_ps<double>(s, n, r0, e1 - e0, nf, lo, hi)));
 }
 
 template <typename T>

@@ -25,6 +25,23 @@ def tube_points(M, spacing, R, seed=3, shuffled=False):
     return X[rng.permutation(M)] if shuffled else X
 
 
+def sac_points(M, spacing, R, seed=3):
+    """A tube's points, ring by ring, then those of a sphere of 1.2 R halfway along it
+    that lie outside the tube: rows next to one another on the wall far apart in the list."""
+    rng = np.random.default_rng(seed)
+    m = 3 * M // 10
+    X = tube_points(M - m, spacing, R, seed)
+    k = np.arange(4 * m)
+    z, a = 1 - (2 * k + 1) / (4.0 * m), np.pi * (1 + 5 ** 0.5) * k
+    s = np.sqrt(1 - z * z)
+    c = np.array([R + 4 + 1.4 * R, R + 4, 4 + 0.5 * (X[-1, 2] - 4)])
+    N = np.stack([s * np.cos(a), s * np.sin(a), z], -1)
+    Y = c + 1.2 * R * N
+    Y = Y[np.hypot(Y[:, 0] - R - 4, Y[:, 1] - R - 4) > R]
+    near = np.linalg.norm(X - c, axis=1) > 1.2 * R
+    return np.concatenate([X[near], Y[np.sort(rng.permutation(len(Y))[:m])]])
+
+
 def _phi(r):
     r = np.abs(r)
     a = (3 - 2 * r + np.sqrt(np.maximum(1 + 4 * r - 4 * r * r, 0))) / 8
